@@ -94,9 +94,12 @@ void flgf_destroy(flgf_ctx* ctx);
  * counterpart; they exist for tuning the spectrum multiply-accumulate:
  *   FLGF_CTX_LIST_PCT  0..100 (default 30): an interaction tile whose useful
  *                      (target, source) pairs are below this percentage of the
- *                      work of the dense parent-group kernel (8 x 8 children of
- *                      every neighbour parent pair, absent blocks included)
- *                      runs on the pair-list kernel instead; 0 = never.
+ *                      work of the dense kernel runs on the pair-list kernel
+ *                      instead; 0 = never.  The dense work of a pair of
+ *                      neighbour parents is 8 x 8 child pairs (absent blocks
+ *                      included); on the finest octree level, whose dense form
+ *                      multiplies whole parents (FP64, and FP32 with
+ *                      FLGF_CTX_MAC >= 1), it counts as 32 (FP64) or 16 (FP32).
  *   FLGF_CTX_TILE      tile in parents, t0 | t1 << 8 | t2 << 16 with
  *                      1 <= t_a <= 8, t0 t1 t2 <= 128 and
  *                      (t0 + 2)(t1 + 2)(t2 + 2) <= 397; default 4 x 4 x 8.
@@ -104,16 +107,20 @@ void flgf_destroy(flgf_ctx* ctx);
  *                      their order is the order in which parents are packed
  *                      into the dense kernel's groups.
  *   FLGF_CTX_MAC       FP32 contexts: the kernels of the spectrum MAC.
- *                      1 (default): dense tiles with one target parent per
- *                      warp and two frequencies per thread (absent
- *                      cells and children are skipped warp-uniformly), sparse
+ *                      1 (default): dense tiles of the finest octree level as
+ *                      convolutions between parents (one zero-padded FFT per
+ *                      parent of (2N)^3 cells), of the coarser levels with one
+ *                      target parent per warp and two frequencies per thread
+ *                      (absent cells and children are skipped), sparse
  *                      tiles (FLGF_CTX_LIST_PCT) as pair lists with one target
  *                      per warp and one frequency per thread; 2: the same
- *                      dense kernel, sparse tiles in the shared-memory
+ *                      dense kernels, sparse tiles in the shared-memory
  *                      pair-list kernel (one target per thread); 0: the
  *                      parent-group kernel (one parent per thread) and the
  *                      shared-memory pair-list kernel.  FP64 contexts always
- *                      use form 0; FLGF_CTX_ORDER applies to form 0 only.
+ *                      use form 0, but for the finest octree level, where
+ *                      their dense tiles are convolutions between parents;
+ *                      FLGF_CTX_ORDER applies to form 0 only.
  *   FLGF_CTX_ORDER     0 (default): the parents of each dense-kernel group keep
  *                      the tile order; 1: they are ordered by their set of
  *                      neighbours with sources (most first, equal sets

@@ -35,7 +35,11 @@ struct flgf_ctx {
   double* d_J1 = nullptr;
   void* d_kspec = nullptr;
   size_t kstride = 0;  // complex elements per octree level
+  void* d_pspec = nullptr;  // the 27 parent kernel spectra of the finest octree level (parent.cu)
   std::vector<double> J1;
+  // whether dense tiles of the finest octree level run between parents (all
+  // but the FP32 parent-group form, FLGF_CTX_MAC = 0)
+  bool parent_form() const { return prec == FLGF_FP64 || mac >= 1; }
 };
 
 namespace {
@@ -161,6 +165,11 @@ struct PhaseOff {  // arena offsets and counts of one phase's launch lists
   size_t fl_groups = 0, fl_rows = 0, fl_dlms = 0, fl_tgt = 0, fl_cells = 0;
   int fl_ncomp = 1, fl_cstride = 0;  // components sharing the frequency-lane groups, their column stride
   bool fl_split = false;              // rows nearly all full: the two-path product form
+  // the finest octree level between parents (parent.cu): the first n_pf
+  // frequency-lane groups, their row and column tables, and the children of
+  // the source and target parents (one component's; the others follow in order)
+  int n_pf = 0, pf_max_cells = 0, pf_max_parents = 0, n_pfs = 0, n_pft = 0, pf_src_stride = 0, pf_tgt_stride = 0;
+  size_t pf_rows = 0, pf_ccol = 0, pf_tcol = 0, pf_sch = 0, pf_tch = 0, pf_scale = 0;
   int n_fll = 0; size_t fll_groups = 0, fll_tgt = 0, fll_beg = 0, fll_len = 0, fll_ent = 0;
   int n_inv = 0, n_inv0 = 0; size_t inv_sid = 0, inv_gid = 0, inv_scale = 0;  // finest octree level first (n_inv0)
   std::vector<int> n_itp; std::vector<size_t> itp_ch, itp_par, itp_cpos;
@@ -208,6 +217,10 @@ struct flgf_blockset {
   bool adj_solved = false;
   void* spec = nullptr;
   void* acc = nullptr;
+  void* pf_src = nullptr;  // half-transformed spectra of the source and target parents of a phase
+  void* pf_dst = nullptr;
+  void* apf_src = nullptr;  // the adjoint's, where its phases need more room than pf_src / pf_dst have
+  void* apf_dst = nullptr;
   void* lap_in = nullptr;
   void* lap_out = nullptr;
   int* d_err = nullptr;
@@ -256,6 +269,7 @@ extern "C" void flgf_destroy(flgf_ctx* ctx) {
   cudaFree(ctx->d_table);
   cudaFree(ctx->d_J1);
   cudaFree(ctx->d_kspec);
+  cudaFree(ctx->d_pspec);
   delete ctx;
 }
 
@@ -308,8 +322,15 @@ extern "C" int flgf_create(flgf_ctx** out, const flgf_opts* o) {
   const size_t csz = ctx->prec == FLGF_FP64 ? 16 : 8;
   ctx->kstride = (size_t)kNOff * NW;
   STEP(cudaMalloc(&ctx->d_kspec, csz * ctx->kstride * ctx->max_oct));
-  STEP(cudaMalloc(&karr, sizeof(double) * (size_t)kNOff * P * P * P));
-  STEP(cudaMalloc(&tmp, 2 * 16 * (size_t)kNOff * NW));
+  STEP(cudaMalloc(&ctx->d_pspec, csz * pf_kernel_values(N)));
+  STEP(cudaMalloc(&karr, sizeof(double) * (size_t)kNOff * P * P * P));  // also the 27 parent arrays of 8 P^3
+  STEP(cudaMalloc(&tmp, std::max<size_t>(2 * 16 * (size_t)kNOff * NW, pf_setup_bytes(N))));
+  STEP(launch_parent_kernel_arrays(ctx->d_table, R, (double)R, (double)ctx->RA, N, karr, ctx->stream));
+  if (ctx->prec == FLGF_FP64) {
+    STEP(launch_pf_setup<double>(N, karr, tmp, ctx->d_pspec, ctx->stream));
+  } else {
+    STEP(launch_pf_setup<float>(N, karr, tmp, ctx->d_pspec, ctx->stream));
+  }
   for (int k = 0; k < ctx->max_oct; ++k) {
     STEP(launch_kernel_arrays(ctx->d_table, R, (double)R, (double)ctx->RA, N, k, karr, ctx->stream));
     void* lvl = (char*)ctx->d_kspec + csz * ctx->kstride * k;
@@ -429,6 +450,10 @@ extern "C" void flgf_blockset_destroy(flgf_blockset* bs) {
   cudaFree(bs->aunodes);
   cudaFree(bs->spec);
   cudaFree(bs->acc);
+  cudaFree(bs->pf_src);
+  cudaFree(bs->pf_dst);
+  cudaFree(bs->apf_src);
+  cudaFree(bs->apf_dst);
   cudaFree(bs->lap_in);
   cudaFree(bs->lap_out);
   cudaFree(bs->d_err);
@@ -456,6 +481,9 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   // inverse FFT list: finest octree level, then the coarser ones (their own launch)
   std::vector<int> fwd_gid, fwd_sid, inv_sid, inv_gid, inv_sid_c, inv_gid_c;
   std::vector<double> inv_scale, inv_scale_c;
+  // sources and targets (with the squared spacing) of the finest octree level
+  std::vector<int> src0;
+  std::vector<std::pair<int, double>> tgt0;
   // parents with targets of dense tiles per octree level, in tile order
   std::vector<std::vector<ParentRec>> dpool;
   std::vector<ListGroup> groups;
@@ -519,6 +547,10 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       return it == in.idx[k].end() ? -1 : it->second;
     };
     const bool excl = k > 0;
+    // products of a neighbour cell in the dense kernel, in units of a child
+    // pair's: 64 of the child-pair kernels; the parent form's cost (8 products
+    // and its share of the parents' transforms) is that of kPfPairs pairs
+    const int per_cell = k == 0 && ctx->parent_form() ? pf_pairs(ctx->prec == FLGF_FP64) : 64;
     for (int t0 = lo[0]; t0 <= hi[0]; t0 += TP[0])
       for (int t1 = lo[1]; t1 <= hi[1]; t1 += TP[1])
         for (int t2 = lo[2]; t2 <= hi[2]; t2 += TP[2]) {
@@ -611,7 +643,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
                     r.cell[e][b] = inr ? sg[b * NQ + (q[0] * tl.Rg[1] + q[1]) * tl.Rg[2] + q[2]] : -1;
                     any_src |= r.cell[e][b] >= 0;
                   }
-                  dense += any_src ? 64 : 0;
+                  dense += any_src ? per_cell : 0;
                 }
                 recs.push_back(r);
               }
@@ -646,14 +678,15 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     for (size_t k = 0; k < in.lv.size(); ++k) {
       for (size_t i = 0; i < in.lv[k].size(); ++i) {
         const int gid = in.gid0[k] + (int)i;
-        if (in.is_src[k][i]) {
-          fwd_gid.push_back(gid);
-          fwd_sid.push_back(gid - ph.gid_begin);
-        }
+        if (in.is_src[k][i]) (k == 0 ? src0 : fwd_gid).push_back(gid);
         if (in.need_tgt[k][i]) {
-          (k == 0 ? inv_sid : inv_sid_c).push_back(gid - ph.gid_begin);
-          (k == 0 ? inv_gid : inv_gid_c).push_back(gid);
-          (k == 0 ? inv_scale : inv_scale_c).push_back(in.h * in.h);
+          if (k == 0) {
+            tgt0.push_back({gid, in.h * in.h});
+          } else {
+            inv_sid_c.push_back(gid - ph.gid_begin);
+            inv_gid_c.push_back(gid);
+            inv_scale_c.push_back(in.h * in.h);
+          }
           if ((int)k < in.top) {
             const I3& c = in.lv[k][i];
             const int pi = in.idx[k + 1].at(key3(c[0] >> 1, c[1] >> 1, c[2] >> 1));
@@ -666,10 +699,6 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       jobs.push_back(TileJob{&in, (int)k});
     }
   }
-  const int n_inv0 = (int)inv_gid.size();
-  inv_gid.insert(inv_gid.end(), inv_gid_c.begin(), inv_gid_c.end());
-  inv_sid.insert(inv_sid.end(), inv_sid_c.begin(), inv_sid_c.end());
-  inv_scale.insert(inv_scale.end(), inv_scale_c.begin(), inv_scale_c.end());
   // run the tile jobs on the host's cores; the results are merged in job order,
   // so the launch lists do not depend on the number of threads
   {
@@ -702,16 +731,104 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       for (auto& r : job.lrecs) lpool[job.k].push_back(std::move(r));
     }
   }
-  // dense MAC: parent groups of every octree level (or frequency-lane groups)
+  // block spectra and inverse transforms of the finest octree level: where it
+  // runs between parents, only the blocks of the pair lists
+  if (count) {
+    bs->n_fwd += (int64_t)(fwd_gid.size() + src0.size());
+    bs->n_inv += (int64_t)(inv_gid_c.size() + tgt0.size());
+    for (int k = 0; k <= maxtop; ++k) bs->n_koff += kNOff;
+  }
+  const bool pform = ctx->parent_form();
+  {
+    std::vector<uint8_t> lsrc(ph.nblocks, !pform), ltgt(ph.nblocks, !pform);
+    if (pform && !lpool.empty())
+      for (const auto& r : lpool[0]) {
+        ltgt[r.first] = 1;
+        for (int w : r.second) lsrc[w >> 9] = 1;
+      }
+    for (int gid : src0)
+      if (lsrc[gid - ph.gid_begin]) fwd_gid.push_back(gid);
+    for (const auto& t : tgt0)
+      if (ltgt[t.first - ph.gid_begin]) {
+        inv_sid.push_back(t.first - ph.gid_begin);
+        inv_gid.push_back(t.first);
+        inv_scale.push_back(t.second);
+      }
+    for (int gid : fwd_gid) fwd_sid.push_back(gid - ph.gid_begin);
+  }
+  const int n_inv0 = (int)inv_gid.size();
+  inv_gid.insert(inv_gid.end(), inv_gid_c.begin(), inv_gid_c.end());
+  inv_sid.insert(inv_sid.end(), inv_sid_c.begin(), inv_sid_c.end());
+  inv_scale.insert(inv_scale.end(), inv_scale_c.begin(), inv_scale_c.end());
+  // dense MAC: parent groups of every octree level (or frequency-lane groups;
+  // the finest level's are those of the products between parents)
   HadLists hl;
   FlLists fll;
   for (int k = 0; k < (int)dpool.size(); ++k) {
-    if (fl)
+    if (k == 0 && pform) {
+      const bool f64 = ctx->prec == FLGF_FP64;
+      pack_fl_groups(0, dpool[0], fll, pf_max_parents(f64), pf_max_cells(f64));
+      ph.n_pf = (int)fll.groups.size();
+      ph.pf_max_cells = fll.max_cells;
+      ph.pf_max_parents = fll.max_parents;
+    } else if (fl)
       pack_fl_groups(k, dpool[k], fll);
     else
       pack_parent_groups(k, dpool[k], nchunk, had_kernel_units(ctx->prec == FLGF_FP64), hl, ctx->order_by_list);
   }
   ph.n_fl = (int)fll.groups.size();
+  if (ph.n_pf > 0) {
+    std::vector<double> scale_of(ph.nblocks, 0.0);
+    for (const auto& t : tgt0) scale_of[t.first - ph.gid_begin] = t.second;
+    std::unordered_map<int, int> col_of;  // first source child of a parent -> its column
+    std::vector<int> ccol, tcol, sch, tch;
+    std::vector<double> pscale;
+    std::vector<uint16_t> prow;
+    for (int gi = 0; gi < ph.n_pf; ++gi) {
+      const FlGroup& g = fll.groups[gi];
+      for (int c = 0; c < g.ncell; ++c) {
+        const int* ch = &fll.cells[(size_t)(g.cell_off + c) * 8];
+        int key = -1;
+        for (int b = 0; b < 8 && key < 0; ++b) key = ch[b];
+        const auto it = col_of.emplace(key, (int)col_of.size());
+        if (it.second)
+          for (int b = 0; b < 8; ++b) sch.push_back(ch[b] < 0 ? -1 : ch[b] + ph.gid_begin);
+        ccol.push_back(it.first->second);
+      }
+      for (int m = 0; m < g.nact; ++m) {
+        const int* t = &fll.tgt_ids[(size_t)(g.row_off + m) * 8];
+        double sc = 0.0;
+        tcol.push_back((int)pscale.size());
+        for (int b = 0; b < 8; ++b) {
+          tch.push_back(t[b] < 0 ? -1 : t[b] + ph.gid_begin);
+          if (t[b] >= 0) sc = scale_of[t[b]];
+        }
+        pscale.push_back(sc);
+        const uint16_t* row = &fll.rows[(size_t)(g.row_off + m) * kFlRowStride];
+        const size_t r0 = prow.size();
+        prow.resize(r0 + kPfRow, (uint16_t)(33 * g.ncell));
+        for (int j = 0; j < row[0]; ++j) prow[r0 + (row[1 + j] >> 11)] = (uint16_t)(33 * (row[1 + j] & 0x7FF));
+      }
+    }
+    // the components of a vector block set: the same parents, shifted blocks
+    ph.pf_src_stride = (int)sch.size() / 8;
+    ph.pf_tgt_stride = (int)tch.size() / 8;
+    const int cs = ph.nblocks / vcomp;
+    const size_t ns = sch.size(), nt = tch.size(), np = pscale.size();
+    for (int c = 1; c < vcomp; ++c) {
+      for (size_t i = 0; i < ns; ++i) sch.push_back(sch[i] < 0 ? -1 : sch[i] + c * cs);
+      for (size_t i = 0; i < nt; ++i) tch.push_back(tch[i] < 0 ? -1 : tch[i] + c * cs);
+      for (size_t i = 0; i < np; ++i) pscale.push_back(pscale[i]);
+    }
+    ph.n_pfs = (int)sch.size() / 8;
+    ph.n_pft = (int)tch.size() / 8;
+    ph.pf_rows = ar.add(prow);
+    ph.pf_ccol = ar.add(ccol);
+    ph.pf_tcol = ar.add(tcol);
+    ph.pf_sch = ar.add(sch);
+    ph.pf_tch = ar.add(tch);
+    ph.pf_scale = ar.add(pscale);
+  }
   {
     size_t rows = 0, full = 0;
     for (const FlGroup& g : fll.groups)
@@ -786,11 +903,6 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       max_group_src = std::max(max_group_src, g.nsrc);
       groups.push_back(g);
     }
-  }
-  if (count) {
-    bs->n_fwd += (int64_t)fwd_gid.size();
-    bs->n_inv += (int64_t)inv_gid.size();
-    for (int k = 0; k <= maxtop; ++k) bs->n_koff += kNOff;
   }
   ph.n_prep = (int)prep_src.size();
   ph.prep_src = ar.add(prep_src);
@@ -1117,6 +1229,16 @@ static int plan_blockset(flgf_ctx* ctx, flgf_blockset* bs, int n_problems, const
   return FLGF_OK;
 }
 
+// Most source and target parents of a phase (parent.cu).
+static std::pair<size_t, size_t> pf_need(const std::vector<PhaseOff>& phases) {
+  std::pair<size_t, size_t> n{0, 0};
+  for (const PhaseOff& ph : phases) {
+    n.first = std::max(n.first, (size_t)ph.n_pfs);
+    n.second = std::max(n.second, (size_t)ph.n_pft);
+  }
+  return n;
+}
+
 static int blockset_create(flgf_ctx* ctx, int n_problems, const int* n_levels, const int* nblk,
                            const int32_t* coords, const double* h0, const uint8_t* want, int ncomp,
                            flgf_blockset** out) {
@@ -1157,6 +1279,9 @@ static int blockset_create(flgf_ctx* ctx, int n_problems, const int* n_levels, c
   if (e == cudaSuccess) e = alloc(&bs->wfield, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->spec, 2 * rs * NW * bs->max_phase_blocks);
   if (e == cudaSuccess) e = alloc(&bs->acc, 2 * rs * NW * bs->max_phase_blocks);
+  const auto pf = pf_need(bs->ph);
+  if (e == cudaSuccess) e = alloc(&bs->pf_src, 2 * rs * pf_parent_values(N) * pf.first);
+  if (e == cudaSuccess) e = alloc(&bs->pf_dst, 2 * rs * pf_parent_values(N) * pf.second);
   if (e == cudaSuccess) e = alloc(&bs->lap_in, rs * N3 * bs->max_level_blocks);
   if (e == cudaSuccess) e = alloc(&bs->lap_out, rs * N3 * bs->max_level_blocks);
   if (e == cudaSuccess) e = alloc((void**)&bs->d_err, sizeof(int));
@@ -1223,7 +1348,7 @@ static int build_adjoint(flgf_blockset* bs) {
   if (bs->masked) return fail(ctx, FLGF_ESTATE, "the adjoint needs a block set without a target mask");
   const size_t N3 = (size_t)ctx->N * ctx->N * ctx->N;
   // start from nothing, so a call after a failed one (out of memory) rebuilds cleanly
-  for (void** p : {&bs->gseed, &bs->gW, &bs->gf, &bs->gtmp, &bs->aunodes}) {
+  for (void** p : {&bs->gseed, &bs->gW, &bs->gf, &bs->gtmp, &bs->aunodes, &bs->apf_src, &bs->apf_dst}) {
     cudaFree(*p);
     *p = nullptr;
   }
@@ -1332,6 +1457,10 @@ static int build_adjoint(flgf_blockset* bs) {
   if (e == cudaSuccess) e = alloc(&bs->gf, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->gtmp, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->aunodes, rs * N3 * bs->G);
+  const auto have = pf_need(bs->ph), need = pf_need(bs->aph);
+  const size_t pv = 2 * rs * pf_parent_values(ctx->N);
+  if (e == cudaSuccess && need.first > have.first) e = alloc(&bs->apf_src, pv * need.first);
+  if (e == cudaSuccess && need.second > have.second) e = alloc(&bs->apf_dst, pv * need.second);
   if (e == cudaSuccess) e = cudaMemset(bs->gseed, 0, rs * N3 * bs->B);
   if (e != cudaSuccess) {
     const int code = (e == cudaErrorMemoryAllocation) ? FLGF_ENOMEM : FLGF_ECUDA;
@@ -1432,7 +1561,7 @@ struct StageScope {
 // FMM of one phase: upward pass over `nodes`, forward FFTs, spectrum MAC,
 // inverse FFTs and downward pass into `unodes`.
 template <typename R>
-cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, R* unodes) {
+cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, R* unodes, void* pf_src, void* pf_dst) {
   flgf_ctx* c = bs->ctx;
   const int N = c->N;
   cudaStream_t s = c->stream;
@@ -1461,14 +1590,20 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
     StageScope sc(bs, 2);
     KRUN(ph.n_fwd, launch_fft_forward<R>(N, nodes, ar.at<int>(ph.fwd_gid), ar.at<int>(ph.fwd_sid), ph.n_fwd, bs->spec,
                                          ph.nblocks, s));
+    KRUN(ph.n_pfs, launch_pf_forward<R>(N, nodes, ar.at<int>(ph.pf_sch), ph.n_pfs, pf_src, s));
   }
   {
     StageScope sc(bs, 3);
+    KRUN(ph.n_pf, launch_pf_mac<R>(N, ar.at<FlGroup>(ph.fl_groups), ph.n_pf, ph.pf_max_cells, ph.pf_max_parents,
+                                   ar.at<uint16_t>(ph.pf_rows), ar.at<int>(ph.pf_ccol), ar.at<int>(ph.pf_tcol), pf_src,
+                                   ph.n_pfs, pf_dst, ph.n_pft, c->d_pspec, ph.fl_ncomp, ph.pf_src_stride,
+                                   ph.pf_tgt_stride, s));
     KRUN(ph.n_work, launch_hadamard<R>(N, ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
                                        ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
                                        ar.at<uint16_t>(ph.par_tab), bs->spec, bs->acc, ph.nblocks, c->d_kspec,
                                        c->kstride, s));
-    KRUN(ph.n_fl, launch_hadamard_fl(N, ar.at<FlGroup>(ph.fl_groups), ph.n_fl, ph.fl_max_cells, ph.fl_max_parents,
+    const int n_fl = ph.n_fl - ph.n_pf;
+    KRUN(n_fl, launch_hadamard_fl(N, ar.at<FlGroup>(ph.fl_groups) + ph.n_pf, n_fl, ph.fl_max_cells, ph.fl_max_parents,
                                      ar.at<uint16_t>(ph.fl_rows), ar.at<uint32_t>(ph.fl_dlms), ar.at<int>(ph.fl_tgt),
                                      ar.at<int>(ph.fl_cells), bs->spec, bs->acc, ph.nblocks, c->d_kspec, c->kstride,
                                      ph.fl_ncomp, ph.fl_cstride, ph.fl_split, s));
@@ -1482,6 +1617,7 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
   }
   {
     StageScope sc(bs, 4);
+    KRUN(ph.n_pft, launch_pf_inverse<R>(N, pf_dst, ar.at<int>(ph.pf_tch), ar.at<double>(ph.pf_scale), ph.n_pft, unodes, s));
     KRUN(ph.n_inv0, launch_fft_inverse<R>(N, bs->acc, ph.nblocks, ar.at<int>(ph.inv_sid), ar.at<int>(ph.inv_gid),
                                           ar.at<double>(ph.inv_scale), ph.n_inv0, unodes, s, false));
     const int nc = ph.n_inv - ph.n_inv0;
@@ -1539,7 +1675,8 @@ cudaError_t enqueue_adjoint(flgf_blockset* bs) {
       KRUN(ao.n_prep, launch_combine_blocks<R>(N, nodes, aa.at<int>(ao.prep_dst), gseed, aa.at<int>(ao.prep_s1), gW,
                                                aa.at<int>(ao.prep_s2), 0, ao.n_prep, s));
     }
-    if ((e = enqueue_fmm<R>(bs, aa, bs->aph[l], unodes)) != cudaSuccess) return e;
+    if ((e = enqueue_fmm<R>(bs, aa, bs->aph[l], unodes, bs->apf_src ? bs->apf_src : bs->pf_src,
+                            bs->apf_dst ? bs->apf_dst : bs->pf_dst)) != cudaSuccess) return e;
     {
       StageScope sc(bs, 6);
       KRUN(ao.n_gacc, launch_combine_blocks<R>(N, gf, aa.at<int>(ao.gacc_dst), unodes, aa.at<int>(ao.gacc_s1), unodes,
@@ -1599,7 +1736,7 @@ cudaError_t enqueue_solve(flgf_blockset* bs) {
       KRUN(ph.n_prep, launch_copy_blocks<R>(N, fwork, ar.at<int>(ph.prep_src), nodes, ar.at<int>(ph.prep_dst),
                                             ar.at<uint8_t>(ph.prep_zero), ph.n_prep, s));
     }
-    if ((e = enqueue_fmm<R>(bs, bs->ar, ph, unodes)) != cudaSuccess) return e;
+    if ((e = enqueue_fmm<R>(bs, bs->ar, ph, unodes, bs->pf_src, bs->pf_dst)) != cudaSuccess) return e;
     {
       StageScope sc(bs, 6);
       R* wf = (R*)bs->wfield;

@@ -418,21 +418,21 @@ static int fl_cell_key(const int* ch) {
   return -1;
 }
 
-void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L) {
+void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L, int max_parents, int max_cells) {
   size_t pos = 0;
   while (pos < recs.size()) {
     // consecutive parents (tile order, so they share cells) while the group's cells fit
     std::unordered_map<int, int> cell_of;
     std::vector<const int*> cells;
     std::vector<size_t> members;
-    while (pos < recs.size() && (int)members.size() < kFlMaxParents) {
+    while (pos < recs.size() && (int)members.size() < max_parents) {
       const ParentRec& r = recs[pos];
       int add = 0;
       for (int e = 0; e < 27; ++e) {
         const int key = fl_cell_key(r.cell[e]);
         add += key >= 0 && !cell_of.count(key);
       }
-      if (!members.empty() && (int)cells.size() + add > kFlMaxCells) break;
+      if (!members.empty() && (int)cells.size() + add > max_cells) break;
       for (int e = 0; e < 27; ++e) {
         const int key = fl_cell_key(r.cell[e]);
         if (key >= 0 && !cell_of.count(key)) {

@@ -1,6 +1,6 @@
 // Internal launcher interface between the host orchestration (flgf_api.cu)
-// and the kernels (lgf.cu, fft.cu, hadamard.cu, hadamard_fl.cu, stencil.cu,
-// meshgen.cu, flgf_static.cu).  Not part of the public C ABI.
+// and the kernels (lgf.cu, fft.cu, parent.cu, hadamard.cu, hadamard_fl.cu,
+// stencil.cu, meshgen.cu, flgf_static.cu).  Not part of the public C ABI.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -161,8 +161,10 @@ struct FlLists {
   std::vector<int> cells;      // [cells][8] spectrum column or -1
   int max_cells = 0, max_parents = 0;
 };
-// Packs parent records, in order, into frequency-lane groups of one octree level.
-void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L);
+// Packs parent records, in order, into frequency-lane groups of one octree
+// level, of at most max_parents parents and max_cells neighbour cells.
+void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L, int max_parents = kFlMaxParents,
+                    int max_cells = kFlMaxCells);
 uint32_t fl_delta_mask(int level, int e, const int* tgt, const int* src);
 size_t fl_smem_bytes(int max_cells, int max_parents);
 // ncomp > 1: a vector block set's components, whose spectrum columns are
@@ -198,6 +200,54 @@ cudaError_t launch_hadamard_fll(int N, const FllGroup* groups, int ngroups, cons
                                 const int* len, const uint32_t* ent, const void* spec, void* acc, int spec_blocks,
                                 const void* kspec, size_t kspec_level_stride, cudaStream_t s);
 
+// ---- the finest octree level between parents (parent.cu) ---------------------
+// The groups are the frequency-lane groups of octree level 0.  Per parent of a
+// group a row of kPfRow uint16: entry e < 27 = 33 x (index of neighbour e's
+// cell in the group), or 33 x ncell (a zero line) where it has no sources; per
+// cell the column of its parent in the source spectra, per target parent its
+// column in the result.  Spectra: [unit][column][32] complex (see parent.cu).
+constexpr int kPfRow = 32;
+constexpr int kPfMacThreads = 256;
+// Cost of a neighbour pair of parents, its share of the parents' transforms
+// included, in child pairs of the pair lists (the rule of FLGF_CTX_LIST_PCT).
+constexpr int pf_pairs(bool fp64) { return fp64 ? 32 : 16; }
+// Group limits: FP32 two CTAs of at most 113 KB per SM, FP64 one.
+constexpr int pf_max_cells(bool fp64) { return fp64 ? 192 : 256; }
+constexpr int pf_max_parents(bool fp64) { return fp64 ? 64 : 128; }
+// Shared memory of the product kernel: lines of the cells (and a zero one) and
+// of the parents, then (16-byte aligned) the rows and columns, then for FP64
+// the real and imaginary parts' sums of the cells' lines.
+template <typename R>
+constexpr size_t pf_row_offset(int max_cells, int max_parents) {
+  return ((size_t)(max_cells + 1 + max_parents) * 33 * 2 * sizeof(R) + 15) / 16 * 16;
+}
+template <typename R>
+constexpr size_t pf_sum_offset(int max_cells, int max_parents) {
+  return (pf_row_offset<R>(max_cells, max_parents) + (size_t)max_parents * (kPfRow * 2 + 4) + (size_t)max_cells * 4 + 15) /
+         16 * 16;
+}
+template <typename R>
+constexpr size_t pf_smem_bytes(int max_cells, int max_parents) {
+  return pf_sum_offset<R>(max_cells, max_parents) + (sizeof(R) == 8 ? (size_t)(max_cells + 1) * 33 * 8 : 0);
+}
+size_t pf_parent_values(int N);  // complex values of one parent's half-transformed spectrum
+size_t pf_kernel_values(int N);  // complex values of the 27 parent kernel spectra
+size_t pf_setup_bytes(int N);    // scratch of launch_pf_setup
+// Parent kernel arrays (FP64, lgf.cu): out[e][i0][i1][i2] = G(Delta - 2N e), Delta = i (i < 2N) or i - 4N (i > 2N), 0 at 2N.
+cudaError_t launch_parent_kernel_arrays(const double* table, int R, double rt, double ra, int N, double* out,
+                                        cudaStream_t s);
+template <typename R>
+cudaError_t launch_pf_setup(int N, const double* karr, void* tmp, void* kspec, cudaStream_t s);
+// cell_ch / tgt_ch: [n][8] block ids of the children (-1: no source / no target)
+template <typename R>
+cudaError_t launch_pf_forward(int N, const R* nodes, const int* cell_ch, int n, void* out, cudaStream_t s);
+template <typename R>
+cudaError_t launch_pf_mac(int N, const FlGroup* groups, int ngroups, int max_cells, int max_parents, const uint16_t* rows,
+                          const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
+                          const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s);
+template <typename R>
+cudaError_t launch_pf_inverse(int N, const void* in, const int* tgt_ch, const double* scales, int n, R* unodes,
+                              cudaStream_t s);
 
 // ---- on-device refinement of a level (meshgen.cu) ----------------------------
 // f: [nblk][N^3] in the context precision; coords, flags, children, buffer on

@@ -101,6 +101,28 @@ __global__ void kernel_arrays_kernel(const double* __restrict__ table, int R, do
   out[idx] = lgf_at(table, R, rt2, ra2, x0, x1, x2);
 }
 
+__global__ void parent_kernel_arrays_kernel(const double* __restrict__ table, int R, double rt2, double ra2, int H,
+                                            double* __restrict__ out) {
+  const int P = 2 * H;
+  const size_t per = (size_t)P * P * P;
+  const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= per * 27) return;
+  const int e = (int)(idx / per), rem = (int)(idx % per);
+  const int i0 = rem / (P * P), i1 = (rem / P) % P, i2 = rem % P;
+  if (i0 == H || i1 == H || i2 == H) { out[idx] = 0.0; return; }
+  const long long x0 = (i0 < H ? i0 : i0 - P) - (long long)H * (e / 9 - 1);
+  const long long x1 = (i1 < H ? i1 : i1 - P) - (long long)H * ((e / 3) % 3 - 1);
+  const long long x2 = (i2 < H ? i2 : i2 - P) - (long long)H * (e % 3 - 1);
+  out[idx] = lgf_at(table, R, rt2, ra2, x0, x1, x2);
+}
+
+cudaError_t launch_parent_kernel_arrays(const double* table, int R, double rt, double ra, int N, double* out,
+                                        cudaStream_t s) {
+  const size_t P = 4 * (size_t)N, total = 27 * P * P * P;
+  parent_kernel_arrays_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(table, R, rt * rt, ra * ra, 2 * N, out);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k, double* out,
                                  cudaStream_t s) {
   const size_t total = (size_t)kNOff * (2 * N) * (2 * N) * (2 * N);

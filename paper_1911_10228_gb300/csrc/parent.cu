@@ -1,0 +1,572 @@
+// a2-a4 of the finest octree level between parents: the near field and the
+// influence lists of a finest-level target (Sec. 2.1) are together all the
+// children of its parent's 27 neighbours, so the level's interaction is a
+// convolution between PARENT blocks of H = 2N cells a side.  One zero-padded
+// FFT of P = 4N points an axis per parent replaces eight of 2N: a neighbour
+// pair then costs 8 NW complex products (NW frequencies of a child's padded
+// spectrum) where the child pairs cost 64 NW.  (Coarser octree levels exclude
+// the near field, which depends on the child, and keep the child-pair
+// kernels.)
+//
+// The transform along axis 0 is fused with the products, so HBM only holds
+// spectra of the two transformed axes, half as long as padded ones:
+//   pf_forward_kernel   planes z of a source parent: axis 2, axis 1
+//   pf_mac_kernel       axis 0 forward, products, axis 0 inverse
+//   pf_inverse_kernel   planes z of a target parent: axis 1, axis 2
+// Layout between them: lines l = k1 (H + 1) + k2 (P (H + 1) of them); a unit
+// is the 32 / H lines that fill a warp, stored [unit][parent][32] with lane
+// (l % (32 / H)) H + z, so the product kernel reads 256-byte (FP32) rows.
+//
+// The axis-0 transform is pruned by parity: the even (odd) outputs are the
+// H-point transform of the H inputs (times w^z), and the kept inverse outputs
+// are the sum of the inverses of the two halves (the odd one times w^-z).  The
+// product kernel takes the two parities one after the other, so its shared
+// memory holds H values per line and parent.
+//
+// Measured against the child-pair kernels (finest level only; GB300): 16^3
+// blocks of 16^3 cells, FP32: products 2.42 -> 0.81 ms, its transforms 0.31 ->
+// 0.17 ms; 11 x 9 x 13 blocks, FP64: 32.5 -> 9.2 ms and 2.4 -> 2.2 ms.
+#include <type_traits>
+
+#include "common.cuh"
+#include "internal.h"
+#include "line_fft.cuh"
+
+namespace flgf {
+
+namespace {
+
+template <typename R> struct Vec2;
+template <> struct Vec2<float> { using type = float2; };
+template <> struct Vec2<double> { using type = double2; };
+
+constexpr int kPfStride = 33;  // complex values between two parents' lines in shared memory (odd: no conflicts)
+
+template <int N> struct PfDims {
+  static constexpr int H = 2 * N, P = 4 * N, NX = H + 1, L = P * NX, S = 32 / H, U = L / S;
+  static_assert(L % S == 0, "whole units");
+};
+
+// a row of N values of block gid in 16-byte vectors, zero for no block (gid < 0)
+template <typename R, int N>
+__device__ __forceinline__ void load_row(const R* __restrict__ nodes, int gid, size_t off, R* x) {
+  constexpr int V = 16 / (int)sizeof(R);
+  const int4* p = reinterpret_cast<const int4*>(nodes + (size_t)max(gid, 0) * N * N * N + off);
+#pragma unroll
+  for (int u = 0; u < N / V; ++u) {
+    const int4 v = gid >= 0 ? __ldg(p + u) : make_int4(0, 0, 0, 0);
+    const R* r = reinterpret_cast<const R*>(&v);
+#pragma unroll
+    for (int j = 0; j < V; ++j) x[u * V + j] = r[j];
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ void cp_async_complex(void* dst, const void* src) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(R) == 4)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+// keeps the compiler from moving one half's shared-memory reads above the
+// other half's work (a thread has the registers for one half)
+__device__ __forceinline__ void half_barrier() { asm volatile("" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+}  // namespace
+
+// Plane padding of the [ZP][H][NX] buffer of the plane kernels: the lanes of
+// a shared-memory access (16 complex floats or 8 complex doubles) are ZP
+// planes of consecutive columns, so planes are offset to fill all banks.
+template <typename R, int N, int ZP>
+constexpr int pf_plane_stride() {
+  constexpr int B = 128 / (2 * (int)sizeof(R));
+  constexpr int want = ZP >= B ? 1 : B / ZP;
+  return PfDims<N>::H * PfDims<N>::NX + ((want - PfDims<N>::H * PfDims<N>::NX % B) % B + B) % B;
+}
+
+constexpr int kPfPlaneThreads = 288;
+
+// ---------------------------------------------------------------------------
+// Axes 2 and 1 of ZP planes of a source parent.  Axis 2 transforms the real
+// rows y and y + N (children of different b1) as one complex line and splits
+// the two spectra; axis 1 writes its outputs straight to HBM, ZP consecutive
+// z per line.
+// ---------------------------------------------------------------------------
+template <typename R, int N, int ZP>
+__global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
+    pf_forward_kernel(const R* __restrict__ nodes, const int* __restrict__ cell_ch, typename Vec2<R>::type* __restrict__ out,
+                      int ncol) {
+  using D = PfDims<N>;
+  using C2 = typename Vec2<R>::type;
+  constexpr int H = D::H, NX = D::NX, P = D::P, ZS = pf_plane_stride<R, N, ZP>(), TW = 64 / P;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C2* buf = reinterpret_cast<C2*>(smem_raw);
+  const int col = blockIdx.x / (H / ZP), z0 = (blockIdx.x % (H / ZP)) * ZP;
+  // a thread per (parity, row pair), then per (parity, column)
+  auto rows = [&](auto parity, int i) {
+    constexpr int par = decltype(parity)::value;
+    const int zl = i / N, y = i % N, z = z0 + zl;
+    const int* ch = cell_ch + col * 8 + (z >= N ? 4 : 0);
+    const size_t roff = (size_t)((z % N) * N + y) * N;
+    C2* r0 = buf + zl * ZS + y * NX;
+    C2* r1 = r0 + N * NX;
+    R xr[H], xi[H];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      load_row<R, N>(nodes, __ldg(ch + b), roff, xr + b * N);
+      load_row<R, N>(nodes, __ldg(ch + 2 + b), roff, xi + b * N);
+    }
+    if constexpr (par == 1) {
+#pragma unroll
+      for (int j = 1; j < H; ++j) rotate64<-1>(j * TW, xr[j], xi[j]);
+    }
+    LineFFT<H, -1, R>::run(xr, xi);
+    // row y: (Z[k] + conj Z[P-k]) / 2, row y + N: (Z[k] - conj Z[P-k]) / 2i
+#pragma unroll
+    for (int m = 0; m <= H / 2 - par; ++m) {
+      const int q = par ? H - 1 - m : (H - m) % H, k = 2 * m + par;
+      r0[k] = C2{R(0.5) * (xr[m] + xr[q]), R(0.5) * (xi[m] - xi[q])};
+      r1[k] = C2{R(0.5) * (xi[m] + xi[q]), R(0.5) * (xr[q] - xr[m])};
+    }
+  };
+  for (int i = threadIdx.x; i < 2 * ZP * N; i += kPfPlaneThreads) {
+    if (i < ZP * N) rows(std::integral_constant<int, 0>{}, i);
+    else rows(std::integral_constant<int, 1>{}, i - ZP * N);
+  }
+  __syncthreads();
+  auto columns = [&](auto parity, int i) {
+    constexpr int par = decltype(parity)::value;
+    const int zl = i % ZP, kx = i / ZP;
+    const C2* src = buf + zl * ZS + kx;
+    R xr[H], xi[H];
+#pragma unroll
+    for (int y = 0; y < H; ++y) {
+      const C2 v = src[y * NX];
+      xr[y] = v.x; xi[y] = v.y;
+      if (par && y > 0) rotate64<-1>(y * TW, xr[y], xi[y]);
+    }
+    LineFFT<H, -1, R>::run(xr, xi);
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+      const int l = (2 * m + par) * NX + kx;
+      out[((size_t)(l / D::S) * ncol + col) * 32 + (l % D::S) * H + z0 + zl] = C2{xr[m], xi[m]};
+    }
+  };
+  for (int i = threadIdx.x; i < 2 * ZP * NX; i += kPfPlaneThreads) {
+    if (i < ZP * NX) columns(std::integral_constant<int, 0>{}, i);
+    else columns(std::integral_constant<int, 1>{}, i - ZP * NX);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Axes 1 and 2 back, of ZP planes of a target parent: keep H outputs an axis,
+// write the children that are targets.  The halves of a pruned inverse are
+// combined through the buffer, so a thread holds one H-point line.
+// ---------------------------------------------------------------------------
+template <typename R, int N, int ZP>
+__global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
+    pf_inverse_kernel(const typename Vec2<R>::type* __restrict__ in, int ncol, const int* __restrict__ tgt_ch,
+                      const double* __restrict__ scales, R* __restrict__ unodes) {
+  using D = PfDims<N>;
+  using C2 = typename Vec2<R>::type;
+  constexpr int H = D::H, NX = D::NX, P = D::P, ZS = pf_plane_stride<R, N, ZP>(), TW = 64 / P;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C2* buf = reinterpret_cast<C2*>(smem_raw);
+  const int col = blockIdx.x / (H / ZP), z0 = (blockIdx.x % (H / ZP)) * ZP;
+  for (int i = threadIdx.x; i < ZP * NX; i += kPfPlaneThreads) {
+    const int zl = i % ZP, kx = i / ZP;
+    C2* dst = buf + zl * ZS + kx;
+    auto half = [&](auto parity) {
+      constexpr int par = decltype(parity)::value;
+      R xr[H], xi[H];
+#pragma unroll
+      for (int m = 0; m < H; ++m) {
+        const int l = (2 * m + par) * NX + kx;
+        const C2 v = in[((size_t)(l / D::S) * ncol + col) * 32 + (l % D::S) * H + z0 + zl];
+        xr[m] = v.x; xi[m] = v.y;
+      }
+      LineFFT<H, +1, R>::run(xr, xi);
+#pragma unroll
+      for (int y = 0; y < H; ++y) {
+        if constexpr (par == 0) {
+          dst[y * NX] = C2{xr[y], xi[y]};
+        } else {
+          if (y > 0) rotate64<+1>(y * TW, xr[y], xi[y]);
+          const C2 v = dst[y * NX];
+          dst[y * NX] = C2{v.x + xr[y], v.y + xi[y]};
+        }
+      }
+    };
+    half(std::integral_constant<int, 0>{});
+    half_barrier();
+    half(std::integral_constant<int, 1>{});
+  }
+  __syncthreads();
+  const R scale = (R)(scales[col] / ((double)P * P * P));
+  for (int i = threadIdx.x; i < ZP * N; i += kPfPlaneThreads) {
+    const int zl = i / N, y = i % N, z = z0 + zl;
+    C2* r0 = buf + zl * ZS + y * NX;
+    C2* r1 = r0 + N * NX;
+    R xr[H], xi[H];
+    // Z = A + i B of the rows y and y + N, whose upper halves are Hermitian;
+    // the even half's outputs wait in the rows' own even slots
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+      const int k = 2 * m;
+      const C2 a = r0[k <= H ? k : P - k], b = r1[k <= H ? k : P - k];
+      xr[m] = k <= H ? a.x - b.y : a.x + b.y;
+      xi[m] = k <= H ? a.y + b.x : b.x - a.y;
+    }
+    LineFFT<H, +1, R>::run(xr, xi);
+#pragma unroll
+    for (int n = 0; n < H; ++n) (n <= N ? r0[2 * n] : r1[2 * (n - N - 1)]) = C2{xr[n], xi[n]};
+    half_barrier();
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+      const int k = 2 * m + 1;
+      const C2 a = r0[k < H ? k : P - k], b = r1[k < H ? k : P - k];
+      xr[m] = k < H ? a.x - b.y : a.x + b.y;
+      xi[m] = k < H ? a.y + b.x : b.x - a.y;
+    }
+    LineFFT<H, +1, R>::run(xr, xi);
+#pragma unroll
+    for (int n = 0; n < H; ++n) {
+      if (n > 0) rotate64<+1>(n * TW, xr[n], xi[n]);
+      const C2 v = n <= N ? r0[2 * n] : r1[2 * (n - N - 1)];
+      xr[n] += v.x;
+      xi[n] += v.y;
+    }
+    const int* ch = tgt_ch + col * 8 + (z >= N ? 4 : 0);
+    const size_t roff = (size_t)((z % N) * N + y) * N;
+    constexpr int V = 16 / (int)sizeof(R);
+#pragma unroll
+    for (int b1 = 0; b1 < 2; ++b1)
+#pragma unroll
+      for (int b2 = 0; b2 < 2; ++b2) {
+        const int gid = __ldg(ch + 2 * b1 + b2);
+        if (gid < 0) continue;
+        int4* o = reinterpret_cast<int4*>(unodes + (size_t)gid * N * N * N + roff);
+#pragma unroll
+        for (int u = 0; u < N / V; ++u) {
+          int4 v;
+          R* r = reinterpret_cast<R*>(&v);
+#pragma unroll
+          for (int j = 0; j < V; ++j) r[j] = scale * (b1 ? xi : xr)[b2 * N + u * V + j];
+          o[u] = v;
+        }
+      }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Axis 0 and the products.  A CTA takes a group of target parents (consecutive
+// in tile order, so they share neighbour cells) and a unit of lines; lane =
+// (line, k0).  Per parity of k0: the group's source lines are copied to shared
+// memory and transformed in place (a thread per line); a warp then takes one
+// target parent at a time with the 27 kernel values of its lane in registers
+// and reads each neighbour's value from shared memory (absent neighbours point
+// at a zero line, so the 27 reads are issued together); the sums go to shared
+// memory, are transformed back (a thread per line) and written.  The second
+// parity adds to what the first wrote.
+// FP64 products take the three-multiplication form (kr (fr + fi), (kr + ki)
+// fi, (ki - kr) fr) with fr + fi kept beside the sources.
+// ---------------------------------------------------------------------------
+template <typename R, int N>
+__global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
+    pf_mac_kernel(const FlGroup* __restrict__ groups, int ngroups, int max_cells, int max_parents,
+                  const uint16_t* __restrict__ rows, const int* __restrict__ cell_col, const int* __restrict__ tgt_col,
+                  const typename Vec2<R>::type* __restrict__ src, int nsrc, typename Vec2<R>::type* __restrict__ dst,
+                  int ndst, const typename Vec2<R>::type* __restrict__ kspec, int src_stride, int dst_stride) {
+  using D = PfDims<N>;
+  using C2 = typename Vec2<R>::type;
+  constexpr int H = D::H, TW = 64 / D::P;
+  constexpr bool G3 = sizeof(R) == 8;
+  constexpr int NW = kPfMacThreads / 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int g = blockIdx.x % ngroups, unit = blockIdx.x / ngroups;
+  const FlGroup gp = groups[g];
+  const int nc = gp.ncell, nt = gp.nact;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  C2* X = reinterpret_cast<C2*>(smem_raw);                       // [max_cells + 1][33], the last used line zero
+  C2* T = X + (size_t)(max_cells + 1) * kPfStride;               // [max_parents][33]
+  uint16_t* RW = reinterpret_cast<uint16_t*>(smem_raw + pf_row_offset<R>(max_cells, max_parents));  // [max_parents][kPfRow]
+  int* CC = reinterpret_cast<int*>(RW + (size_t)max_parents * kPfRow);
+  int* TC = CC + max_cells;
+  R* Sm = reinterpret_cast<R*>(smem_raw + pf_sum_offset<R>(max_cells, max_parents));  // FP64: fr + fi, [max_cells + 1][33]
+
+  {
+    const int4* r4 = reinterpret_cast<const int4*>(rows + (size_t)gp.row_off * kPfRow);
+    for (int i = tid; i < nt * (kPfRow / 8); i += kPfMacThreads) reinterpret_cast<int4*>(RW)[i] = __ldg(r4 + i);
+  }
+  for (int i = tid; i < nc; i += kPfMacThreads) CC[i] = __ldg(cell_col + gp.cell_off + i) + (int)blockIdx.y * src_stride;
+  for (int i = tid; i < nt; i += kPfMacThreads) TC[i] = __ldg(tgt_col + gp.row_off + i) + (int)blockIdx.y * dst_stride;
+  if (tid < 32) {
+    X[(size_t)nc * kPfStride + tid] = C2{R(0), R(0)};
+    if constexpr (G3) Sm[(size_t)nc * kPfStride + tid] = R(0);
+  }
+  __syncthreads();
+  const C2* sbase = src + (size_t)unit * nsrc * 32 + lane;
+  C2* dbase = dst + (size_t)unit * ndst * 32 + lane;
+  auto fill = [&]() {
+    for (int c = warp; c < nc; c += NW) cp_async_complex<R>(X + c * kPfStride + lane, sbase + (size_t)CC[c] * 32);
+  };
+  fill();
+#pragma unroll 1
+  for (int par = 0; par < 2; ++par) {
+    cp_async_wait();
+    __syncthreads();
+    for (int i = tid; i < nc * D::S; i += kPfMacThreads) {
+      const int c = D::S == 1 ? i : i % nc;
+      C2* line = X + c * kPfStride + (D::S == 1 ? 0 : (i / nc) * H);
+      R xr[H], xi[H];
+#pragma unroll
+      for (int z = 0; z < H; ++z) { const C2 v = line[z]; xr[z] = v.x; xi[z] = v.y; }
+      if (par)
+#pragma unroll
+        for (int z = 1; z < H; ++z) rotate64<-1>(z * TW, xr[z], xi[z]);
+      LineFFT<H, -1, R>::run(xr, xi);
+#pragma unroll
+      for (int k = 0; k < H; ++k) line[k] = C2{xr[k], xi[k]};
+      if constexpr (G3) {
+        R* sl = Sm + (line - X);
+#pragma unroll
+        for (int k = 0; k < H; ++k) sl[k] = xr[k] + xi[k];
+      }
+    }
+    R kr[27], ki[27], k2[G3 ? 27 : 1];
+    {
+      const C2* kp = kspec + ((size_t)(unit * 2 + par) * 27) * 32 + lane;
+#pragma unroll
+      for (int e = 0; e < 27; ++e) {
+        const C2 k = __ldg(kp + e * 32);
+        kr[e] = k.x;
+        ki[e] = G3 ? k.x + k.y : k.y;
+        if constexpr (G3) k2[e] = k.y - k.x;
+      }
+    }
+    __syncthreads();
+    for (int m = warp; m < nt; m += NW) {
+      const uint4* rw = reinterpret_cast<const uint4*>(RW + m * kPfRow);
+      uint32_t w[16];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint4 v = rw[q];
+        w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
+      }
+      R a0 = R(0), a1 = R(0), a2 = R(0), a3 = R(0);
+#pragma unroll
+      for (int e = 0; e < 27; ++e) {
+        const uint32_t o = (e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xFFFFu;
+        const C2 f = X[o + lane];
+        if constexpr (G3) {
+          a0 = fma(kr[e], Sm[o + lane], a0);
+          a1 = fma(ki[e], f.y, a1);
+          a2 = fma(k2[e], f.x, a2);
+        } else {
+          a0 = fma(kr[e], f.x, a0);
+          a1 = fma(kr[e], f.y, a1);
+          a2 = fma(ki[e], f.y, a2);
+          a3 = fma(ki[e], f.x, a3);
+        }
+      }
+      T[m * kPfStride + lane] = G3 ? C2{a0 - a1, a0 + a2} : C2{a0 - a2, a1 + a3};
+    }
+    __syncthreads();
+    if (par == 0) fill();  // the second parity's copy of the sources, while the sums are transformed back
+    for (int i = tid; i < nt * D::S; i += kPfMacThreads) {
+      const int m = D::S == 1 ? i : i % nt;
+      C2* line = T + m * kPfStride + (D::S == 1 ? 0 : (i / nt) * H);
+      R xr[H], xi[H];
+#pragma unroll
+      for (int k = 0; k < H; ++k) { const C2 v = line[k]; xr[k] = v.x; xi[k] = v.y; }
+      LineFFT<H, +1, R>::run(xr, xi);
+      if (par)
+#pragma unroll
+        for (int z = 1; z < H; ++z) rotate64<+1>(z * TW, xr[z], xi[z]);
+#pragma unroll
+      for (int z = 0; z < H; ++z) line[z] = C2{xr[z], xi[z]};
+    }
+    __syncthreads();
+    for (int m = warp; m < nt; m += NW) {
+      C2 v = T[m * kPfStride + lane];
+      C2* o = dbase + (size_t)TC[m] * 32;
+      if (par) {  // this thread's own first half
+        const C2 h = *o;
+        v.x += h.x;
+        v.y += h.y;
+      }
+      *o = v;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Setup (FP64): the 27 parent kernel arrays [27][P][P][P] to spectra, one axis
+// per pass by plain discrete Fourier sums (a few ms once per context).
+// ---------------------------------------------------------------------------
+// axis 2: real rows [rows][P] -> [rows][NX]
+__global__ void pf_setup_axis2(const double* __restrict__ in, double2* __restrict__ out, int P, int NX, int rows) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* w = reinterpret_cast<double2*>(smem_raw);
+  double* x = reinterpret_cast<double*>(w + P);
+  for (int j = threadIdx.x; j < P; j += blockDim.x) {
+    double s, c;
+    sincospi(2.0 * j / P, &s, &c);
+    w[j] = make_double2(c, -s);
+    x[j] = in[(size_t)blockIdx.x * P + j];
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < NX; k += blockDim.x) {
+    double re = 0.0, im = 0.0;
+    for (int j = 0; j < P; ++j) {
+      const double2 t = w[(j * k) & (P - 1)];
+      re = fma(x[j], t.x, re);
+      im = fma(x[j], t.y, im);
+    }
+    out[(size_t)blockIdx.x * NX + k] = make_double2(re, im);
+  }
+}
+// a strided axis of P points: in[a][j][b] -> out[a][k][b] (b < nb), block = (a, chunk of b), one thread per (b, k)
+__global__ void pf_setup_axis(const double2* __restrict__ in, double2* __restrict__ out, int P, int nb) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* w = reinterpret_cast<double2*>(smem_raw);
+  double2* x = w + P;  // [P]
+  const int b = blockIdx.x % nb;
+  const size_t a = blockIdx.x / nb;
+  for (int j = threadIdx.x; j < P; j += blockDim.x) {
+    double s, c;
+    sincospi(2.0 * j / P, &s, &c);
+    w[j] = make_double2(c, -s);
+    x[j] = in[(a * P + j) * nb + b];
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < P; k += blockDim.x) {
+    double re = 0.0, im = 0.0;
+    for (int j = 0; j < P; ++j) {
+      const double2 t = w[(j * k) & (P - 1)];
+      re = fma(x[j].x, t.x, fma(-x[j].y, t.y, re));
+      im = fma(x[j].x, t.y, fma(x[j].y, t.x, im));
+    }
+    out[(a * P + k) * nb + b] = make_double2(re, im);
+  }
+}
+// [27][k0][l] -> [unit][parity][27][32] in precision R
+template <typename R, int N>
+__global__ void pf_setup_pack(const double2* __restrict__ in, typename Vec2<R>::type* __restrict__ out) {
+  using D = PfDims<N>;
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (size_t)D::U * 2 * 27 * 32) return;
+  const int lane = i % 32, e = (i / 32) % 27, par = (i / (32 * 27)) % 2, u = (int)(i / (32 * 27 * 2));
+  const int l = u * D::S + lane / D::H, k0 = 2 * (lane % D::H) + par;
+  const double2 v = in[((size_t)e * D::P + k0) * D::L + l];
+  out[i] = typename Vec2<R>::type{(R)v.x, (R)v.y};
+}
+
+template <typename R, int N>
+static cudaError_t setup_spectra(const double* karr, void* tmp, void* kspec, cudaStream_t s) {
+  using D = PfDims<N>;
+  constexpr int P = D::P, NX = D::NX;
+  double2* t0 = reinterpret_cast<double2*>(tmp);
+  double2* t1 = t0 + (size_t)27 * P * P * NX;
+  pf_setup_axis2<<<27 * P * P, 64, P * 24, s>>>(karr, t0, P, NX, 27 * P * P);
+  pf_setup_axis<<<27 * P * NX, 64, P * 32, s>>>(t0, t1, P, NX);       // axis 1: a = (e, i0), b = k2
+  pf_setup_axis<<<27 * P * NX, 64, P * 32, s>>>(t1, t0, P, P * NX);   // axis 0: a = e, b = (k1, k2)
+  const size_t total = (size_t)D::U * 2 * 27 * 32;
+  pf_setup_pack<R, N><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(t0, reinterpret_cast<typename Vec2<R>::type*>(kspec));
+  return cudaGetLastError();
+}
+
+size_t pf_kernel_values(int N) { return (size_t)4 * N * (2 * N + 1) * 2 * N * 2 * 27; }
+size_t pf_setup_bytes(int N) { return (size_t)2 * 16 * 27 * 4 * N * 4 * N * (2 * N + 1); }
+size_t pf_parent_values(int N) { return (size_t)4 * N * (2 * N + 1) * 2 * N; }
+
+template <typename R>
+cudaError_t launch_pf_setup(int N, const double* karr, void* tmp, void* kspec, cudaStream_t s) {
+  if (N == 16) return setup_spectra<R, 16>(karr, tmp, kspec, s);
+  if (N == 8) return setup_spectra<R, 8>(karr, tmp, kspec, s);
+  return cudaErrorInvalidValue;
+}
+
+// Planes per CTA of the plane kernels: FP32 8 of 32 (16 at N = 8, whole
+// parents), FP64 half of that: about 68 KB of shared memory.
+template <typename R, int N> constexpr int pf_planes() { return (N == 16 ? 8 : 16) / (sizeof(R) == 8 ? 2 : 1); }
+
+template <typename R, int N>
+static cudaError_t forward_n(const R* nodes, const int* cell_ch, int n, void* out, int ncol, cudaStream_t s) {
+  constexpr int ZP = pf_planes<R, N>();
+  const size_t sm = sizeof(R) * 2 * ZP * pf_plane_stride<R, N, ZP>();
+  auto k = pf_forward_kernel<R, N, ZP>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  k<<<n * (PfDims<N>::H / ZP), kPfPlaneThreads, sm, s>>>(nodes, cell_ch, reinterpret_cast<typename Vec2<R>::type*>(out), ncol);
+  return cudaGetLastError();
+}
+template <typename R, int N>
+static cudaError_t inverse_n(const void* in, const int* tgt_ch, const double* scales, int n, R* unodes, cudaStream_t s) {
+  constexpr int ZP = pf_planes<R, N>();
+  const size_t sm = sizeof(R) * 2 * ZP * pf_plane_stride<R, N, ZP>();
+  auto k = pf_inverse_kernel<R, N, ZP>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  k<<<n * (PfDims<N>::H / ZP), kPfPlaneThreads, sm, s>>>(reinterpret_cast<const typename Vec2<R>::type*>(in), n, tgt_ch, scales,
+                                                        unodes);
+  return cudaGetLastError();
+}
+template <typename R, int N>
+static cudaError_t mac_n(const FlGroup* groups, int ngroups, int max_cells, int max_parents, const uint16_t* rows,
+                         const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
+                         const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s) {
+  using C2 = typename Vec2<R>::type;
+  const size_t sm = pf_smem_bytes<R>(max_cells, max_parents);
+  if (sm > kFlSmemBytes || (size_t)PfDims<N>::U * ngroups >= (1u << 31)) return cudaErrorInvalidConfiguration;
+  auto k = pf_mac_kernel<R, N>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+  if (e != cudaSuccess) return e;
+  k<<<dim3((unsigned)(PfDims<N>::U * ngroups), ncomp), kPfMacThreads, sm, s>>>(
+      groups, ngroups, max_cells, max_parents, rows, cell_col, tgt_col, reinterpret_cast<const C2*>(src), nsrc,
+      reinterpret_cast<C2*>(dst), ndst, reinterpret_cast<const C2*>(kspec), src_stride, dst_stride);
+  return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_pf_forward(int N, const R* nodes, const int* cell_ch, int n, void* out, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (N == 16) return forward_n<R, 16>(nodes, cell_ch, n, out, n, s);
+  if (N == 8) return forward_n<R, 8>(nodes, cell_ch, n, out, n, s);
+  return cudaErrorInvalidValue;
+}
+template <typename R>
+cudaError_t launch_pf_mac(int N, const FlGroup* groups, int ngroups, int max_cells, int max_parents, const uint16_t* rows,
+                          const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
+                          const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s) {
+  if (ngroups <= 0) return cudaSuccess;
+  if (N == 16)
+    return mac_n<R, 16>(groups, ngroups, max_cells, max_parents, rows, cell_col, tgt_col, src, nsrc, dst, ndst, kspec, ncomp,
+                        src_stride, dst_stride, s);
+  if (N == 8)
+    return mac_n<R, 8>(groups, ngroups, max_cells, max_parents, rows, cell_col, tgt_col, src, nsrc, dst, ndst, kspec, ncomp,
+                       src_stride, dst_stride, s);
+  return cudaErrorInvalidValue;
+}
+template <typename R>
+cudaError_t launch_pf_inverse(int N, const void* in, const int* tgt_ch, const double* scales, int n, R* unodes,
+                              cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  if (N == 16) return inverse_n<R, 16>(in, tgt_ch, scales, n, unodes, s);
+  if (N == 8) return inverse_n<R, 8>(in, tgt_ch, scales, n, unodes, s);
+  return cudaErrorInvalidValue;
+}
+
+#define FLGF_PF_INST(R)                                                                                             \
+  template cudaError_t launch_pf_setup<R>(int, const double*, void*, void*, cudaStream_t);                          \
+  template cudaError_t launch_pf_forward<R>(int, const R*, const int*, int, void*, cudaStream_t);                   \
+  template cudaError_t launch_pf_mac<R>(int, const FlGroup*, int, int, int, const uint16_t*, const int*, const int*, \
+                                        const void*, int, void*, int, const void*, int, int, int, cudaStream_t);    \
+  template cudaError_t launch_pf_inverse<R>(int, const void*, const int*, const double*, int, R*, cudaStream_t);
+FLGF_PF_INST(float)
+FLGF_PF_INST(double)
+#undef FLGF_PF_INST
+
+}  // namespace flgf

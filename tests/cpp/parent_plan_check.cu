@@ -1,0 +1,116 @@
+// Host-only check of the tables of the products between parents (parent.cu):
+// in every phase, forward and adjoint, each finest-level target is written
+// exactly once (a child of a target parent, or of the block-wise inverse), the
+// parents' rows and columns say the same as the frequency-lane groups they are
+// made from, and the sources of the block-wise kernels are all transformed.
+//
+// usage: parent_plan_check <mesh file> <list_pct> <fp64 0|1> <ncomp>
+#include "../../paper_1911_10228_gb300/csrc/flgf_api.cu"
+
+#include <cstdio>
+#include <map>
+#include <set>
+
+int main(int argc, char** argv) {
+  if (argc != 5) return 2;
+  FILE* fp = fopen(argv[1], "rb");
+  if (!fp) return 2;
+  auto rd = [&](int* v, size_t n) { return fread(v, sizeof(int), n, fp) == n; };
+  int N = 0, np = 0, nl = 0, nb = 0;
+  if (!rd(&N, 1) || !rd(&np, 1)) return 2;
+  std::vector<int> nlev(np);
+  if (!rd(nlev.data(), np)) return 2;
+  for (int v : nlev) nl += v;
+  std::vector<int> nblk(nl);
+  if (!rd(nblk.data(), nl)) return 2;
+  for (int v : nblk) nb += v;
+  std::vector<int32_t> coords(3 * (size_t)nb);
+  if (!rd(coords.data(), coords.size())) return 2;
+  fclose(fp);
+  std::vector<double> h0(np);
+  for (int p = 0; p < np; ++p) h0[p] = 1.0 + (atoi(argv[4]) > 1 ? 0 : p);
+  flgf_ctx ctx;
+  ctx.N = N;
+  ctx.prec = atoi(argv[3]) ? FLGF_FP64 : FLGF_FP32;
+  ctx.max_oct = 8;
+  ctx.list_pct = atoi(argv[2]);
+  auto bs = new flgf_blockset();
+  bs->ctx = &ctx;
+  bs->ncomp = atoi(argv[4]);
+  if (plan_blockset(&ctx, bs, np, nlev.data(), nblk.data(), coords.data(), h0.data()) != FLGF_OK) return 1;
+  build_adjoint(bs);  // the lists are complete; its allocations fail without a GPU
+  long bad = 0, parents = 0, blocks = 0;
+  auto check = [&](const PhaseOff& ph, const char* base, const std::vector<const Inst*>& insts) {
+    auto I = [&](size_t off) { return reinterpret_cast<const int*>(base + off); };
+    std::map<int, double> want;  // finest-level target -> scale
+    for (const Inst* in : insts)
+      for (size_t i = 0; i < in->lv[0].size(); ++i)
+        if (in->need_tgt[0][i]) want[in->gid0[0] + (int)i] = in->h * in->h;
+    std::map<int, int> written;
+    auto wrote = [&](int gid, double scale) {
+      bad += want.count(gid) == 0 || want[gid] != scale;
+      written[gid]++;
+    };
+    const double* iscale = reinterpret_cast<const double*>(base + ph.inv_scale);
+    for (int i = 0; i < ph.n_inv0; ++i, ++blocks) wrote(I(ph.inv_gid)[i], iscale[i]);
+    const double* pscale = reinterpret_cast<const double*>(base + ph.pf_scale);
+    for (int i = 0; i < ph.n_pft; ++i, ++parents)
+      for (int a = 0; a < 8; ++a)
+        if (I(ph.pf_tch)[8 * i + a] >= 0) wrote(I(ph.pf_tch)[8 * i + a], pscale[i]);
+    bad += written.size() != want.size();
+    for (const auto& w : written) bad += w.second != 1;
+    std::set<int> fwd(I(ph.fwd_sid), I(ph.fwd_sid) + ph.n_fwd);
+    const uint32_t* qe = reinterpret_cast<const uint32_t*>(base + ph.fll_ent);
+    const FllGroup* Q = reinterpret_cast<const FllGroup*>(base + ph.fll_groups);
+    for (int g = 0; g < ph.n_fll; ++g)
+      for (int m = 0; m < Q[g].ntgt; ++m)
+        for (int j = 0; j < I(ph.fll_len)[Q[g].tgt_off + m]; ++j)
+          bad += !fwd.count((int)(qe[I(ph.fll_beg)[Q[g].tgt_off + m] + j] >> 9));
+    const ListGroup* LG = reinterpret_cast<const ListGroup*>(base + ph.groups);
+    for (int g = 0; g < ph.n_groups; ++g)
+      for (int i = 0; i < LG[g].nsrc; ++i) bad += !fwd.count(I(ph.l_src)[LG[g].src_off + i]);
+    const FlGroup* G = reinterpret_cast<const FlGroup*>(base + ph.fl_groups);
+    const uint16_t* rows = reinterpret_cast<const uint16_t*>(base + ph.fl_rows);
+    const uint16_t* prow = reinterpret_cast<const uint16_t*>(base + ph.pf_rows);
+    for (int gi = 0; gi < ph.n_fl; ++gi) {
+      const FlGroup& g = G[gi];
+      bad += (gi < ph.n_pf) != (g.level == 0);
+      for (int c = 0; c < g.ncell; ++c)
+        for (int b = 0; b < 8; ++b) {
+          const int s = I(ph.fl_cells)[(g.cell_off + c) * 8 + b];
+          if (g.level > 0) { bad += s >= 0 && !fwd.count(s); continue; }
+          for (int k = 0; k < ph.fl_ncomp; ++k)
+            bad += I(ph.pf_sch)[8 * (I(ph.pf_ccol)[g.cell_off + c] + k * ph.pf_src_stride) + b] !=
+                   (s < 0 ? -1 : s + k * ph.fl_cstride + ph.gid_begin);
+        }
+      if (g.level > 0) continue;
+      bad += g.nact > ph.pf_max_parents || g.ncell > ph.pf_max_cells;
+      for (int m = 0; m < g.nact; ++m) {
+        const uint16_t* r = rows + (size_t)(g.row_off + m) * kFlRowStride;
+        const uint16_t* p = prow + (size_t)(g.row_off + m) * kPfRow;
+        int have = 0;
+        for (int e = 0; e < kPfRow; ++e) have += p[e] != 33 * g.ncell;
+        bad += have != r[0];
+        for (int j = 0; j < r[0]; ++j) bad += p[r[1 + j] >> 11] != 33 * (r[1 + j] & 0x7FF);
+        for (int k = 0; k < ph.fl_ncomp; ++k)
+          for (int a = 0; a < 8; ++a) {
+            const int t = I(ph.fl_tgt)[(g.row_off + m) * 8 + a];
+            bad += I(ph.pf_tch)[8 * (I(ph.pf_tcol)[g.row_off + m] + k * ph.pf_tgt_stride) + a] !=
+                   (t < 0 ? -1 : t + k * ph.fl_cstride + ph.gid_begin);
+          }
+      }
+    }
+  };
+  for (int adj = 0; adj < 2; ++adj)
+    for (int l = 0; l < bs->Lmax; ++l) {
+      std::vector<const Inst*> insts;
+      for (const Inst& in : bs->inst)
+        if (in.l == l && (!adj || in.variant == 0)) insts.push_back(&in);
+      if (adj)
+        for (const Inst& in : bs->adj_inst)
+          if (in.l == l) insts.push_back(&in);
+      check(adj ? bs->aph[l] : bs->ph[l], adj ? bs->aar.host.data() : bs->ar.host.data(), insts);
+    }
+  printf("parents %ld blocks %ld mismatches %ld\n%s\n", parents, blocks, bad, bad ? "FAILED" : "ok");
+  return bad ? 1 : 0;
+}
