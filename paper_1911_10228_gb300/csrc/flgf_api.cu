@@ -166,10 +166,11 @@ struct PhaseOff {  // arena offsets and counts of one phase's launch lists
   int fl_ncomp = 1, fl_cstride = 0;  // components sharing the frequency-lane groups, their column stride
   bool fl_split = false;              // rows nearly all full: the two-path product form
   // the finest octree level between parents (parent.cu): the first n_pf
-  // frequency-lane groups, their row and column tables, and the children of
+  // frequency-lane groups, their items and column tables, and the children of
   // the source and target parents (one component's; the others follow in order)
-  int n_pf = 0, pf_max_cells = 0, pf_max_parents = 0, n_pfs = 0, n_pft = 0, pf_src_stride = 0, pf_tgt_stride = 0;
-  size_t pf_rows = 0, pf_ccol = 0, pf_tcol = 0, pf_sch = 0, pf_tch = 0, pf_scale = 0;
+  int n_pf = 0, n_pfs = 0, n_pft = 0, pf_src_stride = 0, pf_tgt_stride = 0;
+  PfLimits pf_lim;
+  size_t pf_groups = 0, pf_items = 0, pf_ccol = 0, pf_tcol = 0, pf_sch = 0, pf_tch = 0, pf_scale = 0;
   int n_fll = 0; size_t fll_groups = 0, fll_tgt = 0, fll_beg = 0, fll_len = 0, fll_ent = 0;
   int n_inv = 0, n_inv0 = 0; size_t inv_sid = 0, inv_gid = 0, inv_scale = 0;  // finest octree level first (n_inv0)
   std::vector<int> n_itp; std::vector<size_t> itp_ch, itp_par, itp_cpos;
@@ -620,7 +621,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
           int64_t dense = 0;  // complex MACs per frequency of the parent-group kernel
           for (int p0 = 0; p0 < tl.P[0]; ++p0)
             for (int p1 = 0; p1 < tl.P[1]; ++p1)
-              for (int p2 = 0; p2 < tl.P[2]; ++p2) {
+              for (int p2 = 0, last_p2 = -2; p2 < tl.P[2]; ++p2) {
                 ParentRec r;
                 bool has = false;
                 for (int a = 0; a < 8; ++a) {
@@ -645,6 +646,8 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
                   }
                   dense += any_src ? per_cell : 0;
                 }
+                r.follows = last_p2 == p2 - 1;
+                last_p2 = p2;
                 recs.push_back(r);
               }
           if (useful * 100 < (int64_t)list_pct * dense) {
@@ -769,8 +772,6 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       const bool f64 = ctx->prec == FLGF_FP64;
       pack_fl_groups(0, dpool[0], fll, pf_max_parents(f64), pf_max_cells(f64));
       ph.n_pf = (int)fll.groups.size();
-      ph.pf_max_cells = fll.max_cells;
-      ph.pf_max_parents = fll.max_parents;
     } else if (fl)
       pack_fl_groups(k, dpool[k], fll);
     else
@@ -783,7 +784,8 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     std::unordered_map<int, int> col_of;  // first source child of a parent -> its column
     std::vector<int> ccol, tcol, sch, tch;
     std::vector<double> pscale;
-    std::vector<uint16_t> prow;
+    std::vector<PfGroup> pgroups;
+    std::vector<uint16_t> items;  // [items][kPfItem]
     for (int gi = 0; gi < ph.n_pf; ++gi) {
       const FlGroup& g = fll.groups[gi];
       for (int c = 0; c < g.ncell; ++c) {
@@ -804,11 +806,37 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
           if (t[b] >= 0) sc = scale_of[t[b]];
         }
         pscale.push_back(sc);
-        const uint16_t* row = &fll.rows[(size_t)(g.row_off + m) * kFlRowStride];
-        const size_t r0 = prow.size();
-        prow.resize(r0 + kPfRow, (uint16_t)(33 * g.ncell));
-        for (int j = 0; j < row[0]; ++j) prow[r0 + (row[1 + j] >> 11)] = (uint16_t)(33 * (row[1 + j] & 0x7FF));
       }
+      PfGroup pg{g.ncell, g.nact, 0, g.cell_off, g.row_off, (int)(items.size() / kPfItem)};
+      // pairs first, then single parents, so the warps' round-robin ends together
+      auto add_item = [&](int m, int n) {
+        uint16_t it[kPfItem] = {0};
+        for (int i = 0; i < 36; ++i) it[i] = (uint16_t)(33 * g.ncell);
+        it[36] = (uint16_t)m;
+        it[37] = (uint16_t)n;
+        for (int p = 0; p < n; ++p) {
+          const uint16_t* row = &fll.rows[(size_t)(g.row_off + m + p) * kFlRowStride];
+          for (int j = 0; j < row[0]; ++j) {
+            const int e = row[1 + j] >> 11;
+            it[9 * (e % 3 + p) + e / 3] = (uint16_t)(33 * (row[1 + j] & 0x7FF));
+            it[38] |= (uint16_t)(1 << (e / 9));
+          }
+        }
+        items.insert(items.end(), it, it + kPfItem);
+        ++pg.nitem;
+      };
+      std::vector<int> single;
+      for (int m = 0; m < g.nact;) {
+        const bool pair = m + 1 < g.nact && dpool[0][g.row_off + m + 1].follows;
+        if (pair) add_item(m, 2);
+        else single.push_back(m);
+        m += pair ? 2 : 1;
+      }
+      for (int m : single) add_item(m, 1);
+      ph.pf_lim.cells = std::max(ph.pf_lim.cells, pg.ncell);
+      ph.pf_lim.parents = std::max(ph.pf_lim.parents, pg.nact);
+      ph.pf_lim.items = std::max(ph.pf_lim.items, pg.nitem);
+      pgroups.push_back(pg);
     }
     // the components of a vector block set: the same parents, shifted blocks
     ph.pf_src_stride = (int)sch.size() / 8;
@@ -822,7 +850,8 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     }
     ph.n_pfs = (int)sch.size() / 8;
     ph.n_pft = (int)tch.size() / 8;
-    ph.pf_rows = ar.add(prow);
+    ph.pf_groups = ar.add(pgroups);
+    ph.pf_items = ar.add(items);
     ph.pf_ccol = ar.add(ccol);
     ph.pf_tcol = ar.add(tcol);
     ph.pf_sch = ar.add(sch);
@@ -1594,9 +1623,9 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
   }
   {
     StageScope sc(bs, 3);
-    KRUN(ph.n_pf, launch_pf_mac<R>(N, ar.at<FlGroup>(ph.fl_groups), ph.n_pf, ph.pf_max_cells, ph.pf_max_parents,
-                                   ar.at<uint16_t>(ph.pf_rows), ar.at<int>(ph.pf_ccol), ar.at<int>(ph.pf_tcol), pf_src,
-                                   ph.n_pfs, pf_dst, ph.n_pft, c->d_pspec, ph.fl_ncomp, ph.pf_src_stride,
+    KRUN(ph.n_pf, launch_pf_mac<R>(N, ar.at<PfGroup>(ph.pf_groups), ph.n_pf, ph.pf_lim, ar.at<uint16_t>(ph.pf_items),
+                                   ar.at<int>(ph.pf_ccol), ar.at<int>(ph.pf_tcol), pf_src, ph.n_pfs,
+                                   pf_dst, ph.n_pft, c->d_pspec, ph.fl_ncomp, ph.pf_src_stride,
                                    ph.pf_tgt_stride, s));
     KRUN(ph.n_work, launch_hadamard<R>(N, ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
                                        ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),

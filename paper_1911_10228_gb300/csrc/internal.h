@@ -80,9 +80,11 @@ constexpr uint16_t kNbEnd = 0xFFFF;           // no neighbour cell (cells < 2048
 // One parent with targets: its 8 children (spectrum column or -1) and, per
 // neighbour e (e = 9 (e0+1) + 3 (e1+1) + (e2+1)), the 8 children of parent
 // p + e that are sources (all -1 when there are none or the pair is excluded).
+// follows: the record before it is its neighbour along axis 2, one down.
 struct ParentRec {
   int tgt[8];
   int cell[27][8];
+  bool follows = false;
 };
 // Launch lists of the dense MAC, appended to by pack_parent_groups.
 struct HadLists {
@@ -201,34 +203,44 @@ cudaError_t launch_hadamard_fll(int N, const FllGroup* groups, int ngroups, cons
                                 const void* kspec, size_t kspec_level_stride, cudaStream_t s);
 
 // ---- the finest octree level between parents (parent.cu) ---------------------
-// The groups are the frequency-lane groups of octree level 0.  Per parent of a
-// group a row of kPfRow uint16: entry e < 27 = 33 x (index of neighbour e's
-// cell in the group), or 33 x ncell (a zero line) where it has no sources; per
-// cell the column of its parent in the source spectra, per target parent its
-// column in the result.  Spectra: [unit][column][32] complex (see parent.cu).
-constexpr int kPfRow = 32;
+// The groups are the frequency-lane groups of octree level 0.  Their parents
+// are taken in items of two neighbours along axis 2 (consecutive in the group)
+// or one.  Item: uint16 entries; 9 q + c (q < 4, c = 3 (e0 + 1) + e1 + 1) = 33 x
+// (index in the group) of the neighbour cell (e0, e1) one down of the first
+// parent (q = 0), at it (1), one up (2) and two up (3, pairs only), or 33 x ncell
+// (a zero line) where it has no sources; entry 36 the first parent (index in
+// the group), 37 the parents, 38 bit e0 + 1 set when cells of that e0 exist.
+// Per cell the column of its parent in the source spectra, per target parent
+// its column in the result.  Spectra: [unit][column][32] complex (parent.cu).
+struct PfGroup {
+  int ncell, nact, nitem;
+  int cell_off, row_off, item_off;
+};
+constexpr int kPfItem = 40;  // uint16 per item: five 16-byte vectors
 constexpr int kPfMacThreads = 256;
 // Cost of a neighbour pair of parents, its share of the parents' transforms
 // included, in child pairs of the pair lists (the rule of FLGF_CTX_LIST_PCT).
 constexpr int pf_pairs(bool fp64) { return fp64 ? 32 : 16; }
-// Group limits: FP32 two CTAs of at most 113 KB per SM, FP64 one.
+// Group limits: FP32 two CTAs of at most 113 KB per SM, FP64 one of 227 KB.
 constexpr int pf_max_cells(bool fp64) { return fp64 ? 192 : 256; }
 constexpr int pf_max_parents(bool fp64) { return fp64 ? 64 : 128; }
+struct PfLimits {  // the largest group of a launch
+  int cells = 0, parents = 0, items = 0;
+};
 // Shared memory of the product kernel: lines of the cells (and a zero one) and
-// of the parents, then (16-byte aligned) the rows and columns, then for FP64
-// the real and imaginary parts' sums of the cells' lines.
+// of the parents (FP64: per parity); for FP64 the sums of the cells' real and
+// imaginary parts; then the items and columns.
 template <typename R>
-constexpr size_t pf_row_offset(int max_cells, int max_parents) {
-  return ((size_t)(max_cells + 1 + max_parents) * 33 * 2 * sizeof(R) + 15) / 16 * 16;
+constexpr size_t pf_sum_offset(const PfLimits& l) {
+  return (size_t)(l.cells + 1 + (sizeof(R) == 8 ? 2 : 1) * l.parents) * 33 * 2 * sizeof(R);
 }
 template <typename R>
-constexpr size_t pf_sum_offset(int max_cells, int max_parents) {
-  return (pf_row_offset<R>(max_cells, max_parents) + (size_t)max_parents * (kPfRow * 2 + 4) + (size_t)max_cells * 4 + 15) /
-         16 * 16;
+constexpr size_t pf_table_offset(const PfLimits& l) {
+  return (pf_sum_offset<R>(l) + (sizeof(R) == 8 ? (size_t)(l.cells + 1) * 33 * 8 : 0) + 15) / 16 * 16;
 }
 template <typename R>
-constexpr size_t pf_smem_bytes(int max_cells, int max_parents) {
-  return pf_sum_offset<R>(max_cells, max_parents) + (sizeof(R) == 8 ? (size_t)(max_cells + 1) * 33 * 8 : 0);
+constexpr size_t pf_smem_bytes(const PfLimits& l) {
+  return pf_table_offset<R>(l) + (size_t)l.items * kPfItem * 2 + (size_t)(l.cells + l.parents) * 4;
 }
 size_t pf_parent_values(int N);  // complex values of one parent's half-transformed spectrum
 size_t pf_kernel_values(int N);  // complex values of the 27 parent kernel spectra
@@ -242,9 +254,9 @@ cudaError_t launch_pf_setup(int N, const double* karr, void* tmp, void* kspec, c
 template <typename R>
 cudaError_t launch_pf_forward(int N, const R* nodes, const int* cell_ch, int n, void* out, cudaStream_t s);
 template <typename R>
-cudaError_t launch_pf_mac(int N, const FlGroup* groups, int ngroups, int max_cells, int max_parents, const uint16_t* rows,
-                          const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
-                          const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s);
+cudaError_t launch_pf_mac(int N, const PfGroup* groups, int ngroups, const PfLimits& lim, const uint16_t* items,
+                          const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst,
+                          int ndst, const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s);
 template <typename R>
 cudaError_t launch_pf_inverse(int N, const void* in, const int* tgt_ch, const double* scales, int n, R* unodes,
                               cudaStream_t s);

@@ -2,8 +2,8 @@
 // with twiddles known at compile time, and the pieces of the pruned transforms
 // of length 2H whose second half of the inputs is zero (forward) or of the
 // outputs is not kept (inverse): the even outputs of the forward transform are
-// the length-H transform of the inputs, the odd ones that of the inputs times
-// w^j; the kept outputs of the inverse are E + w^-j O with E and O the
+// the length-H transform of the inputs, the odd ones the same at frequencies
+// k + 1/2; the kept outputs of the inverse are E + w^-j O with E and O the
 // transforms of the even and odd inputs.
 #pragma once
 #include <cuda_runtime.h>
@@ -45,9 +45,30 @@ __device__ __forceinline__ void rotate64(int j, R& xr, R& xi) {
   xr = tr;
 }
 
+// (u, v) -> (u + w v, u - w v), w = e^{-2 pi i j / 64} (DIR < 0) or its
+// conjugate: six fused multiply-adds with tan or cot, whichever is at most 1,
+// factored out of w v.
+template <int DIR, typename R>
+__device__ __forceinline__ void butterfly64(int j, R ur, R ui, R vr, R vi, R& ar, R& ai, R& br, R& bi) {
+  const double c = cos64(j), s = DIR < 0 ? -sin64(j) : sin64(j);  // w = c + i s
+  if (s == 0.0 || c == 0.0) {                                      // +-1, +-i
+    const R tr = s == 0.0 ? (c > 0 ? vr : -vr) : (s > 0 ? -vi : vi);
+    const R ti = s == 0.0 ? (c > 0 ? vi : -vi) : (s > 0 ? vr : -vr);
+    ar = ur + tr; ai = ui + ti;
+    br = ur - tr; bi = ui - ti;
+    return;
+  }
+  const bool big = c * c >= s * s;
+  const R t = (R)(big ? s / c : c / s), f = (R)(big ? c : s);
+  const R p = big ? fma(-t, vi, vr) : fma(t, vr, -vi), q = big ? fma(t, vr, vi) : fma(t, vi, vr);
+  ar = fma(f, p, ur); ai = fma(f, q, ui);
+  br = fma(-f, p, ur); bi = fma(-f, q, ui);
+}
+
 // In-register FFT of length L (a power of two up to 32), natural order in and
-// out, unnormalised; DIR = -1 forward, +1 inverse.
-template <int L, int DIR, typename R>
+// out, unnormalised; DIR = -1 forward, +1 inverse.  ODD: the odd outputs of the
+// transform of length 2L whose inputs L.. are zero (frequencies k + 1/2).
+template <int L, int DIR, typename R, bool ODD = false>
 struct LineFFT {
   static __device__ __forceinline__ void run(R* re, R* im) {
     constexpr int H = L / 2;
@@ -57,24 +78,15 @@ struct LineFFT {
       er[j] = re[2 * j]; ei[j] = im[2 * j];
       odr[j] = re[2 * j + 1]; odi[j] = im[2 * j + 1];
     }
-    LineFFT<H, DIR, R>::run(er, ei);
-    LineFFT<H, DIR, R>::run(odr, odi);
+    LineFFT<H, DIR, R, ODD>::run(er, ei);
+    LineFFT<H, DIR, R, ODD>::run(odr, odi);
 #pragma unroll
-    for (int k = 0; k < H; ++k) {
-      R tr = odr[k], ti = odi[k];
-      if (4 * k == L) {  // w = -i (forward) or +i (inverse)
-        tr = DIR < 0 ? odi[k] : -odi[k];
-        ti = DIR < 0 ? -odr[k] : odr[k];
-      } else if (k > 0) {
-        rotate64<DIR>(k * (64 / L), tr, ti);
-      }
-      re[k] = er[k] + tr; im[k] = ei[k] + ti;
-      re[k + H] = er[k] - tr; im[k + H] = ei[k] - ti;
-    }
+    for (int k = 0; k < H; ++k)
+      butterfly64<DIR>((2 * k + ODD) * (32 / L), er[k], ei[k], odr[k], odi[k], re[k], im[k], re[k + H], im[k + H]);
   }
 };
-template <int DIR, typename R>
-struct LineFFT<1, DIR, R> {
+template <int DIR, typename R, bool ODD>
+struct LineFFT<1, DIR, R, ODD> {
   static __device__ __forceinline__ void run(R*, R*) {}
 };
 

@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
                       int ncol) {
   using D = PfDims<N>;
   using C2 = typename Vec2<R>::type;
-  constexpr int H = D::H, NX = D::NX, P = D::P, ZS = pf_plane_stride<R, N, ZP>(), TW = 64 / P;
+  constexpr int H = D::H, NX = D::NX, ZS = pf_plane_stride<R, N, ZP>();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2* buf = reinterpret_cast<C2*>(smem_raw);
   const int col = blockIdx.x / (H / ZP), z0 = (blockIdx.x % (H / ZP)) * ZP;
@@ -118,11 +118,7 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
       load_row<R, N>(nodes, __ldg(ch + b), roff, xr + b * N);
       load_row<R, N>(nodes, __ldg(ch + 2 + b), roff, xi + b * N);
     }
-    if constexpr (par == 1) {
-#pragma unroll
-      for (int j = 1; j < H; ++j) rotate64<-1>(j * TW, xr[j], xi[j]);
-    }
-    LineFFT<H, -1, R>::run(xr, xi);
+    LineFFT<H, -1, R, par == 1>::run(xr, xi);
     // row y: (Z[k] + conj Z[P-k]) / 2, row y + N: (Z[k] - conj Z[P-k]) / 2i
 #pragma unroll
     for (int m = 0; m <= H / 2 - par; ++m) {
@@ -145,9 +141,8 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
     for (int y = 0; y < H; ++y) {
       const C2 v = src[y * NX];
       xr[y] = v.x; xi[y] = v.y;
-      if (par && y > 0) rotate64<-1>(y * TW, xr[y], xi[y]);
     }
-    LineFFT<H, -1, R>::run(xr, xi);
+    LineFFT<H, -1, R, par == 1>::run(xr, xi);
 #pragma unroll
     for (int m = 0; m < H; ++m) {
       const int l = (2 * m + par) * NX + kx;
@@ -263,20 +258,22 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 // ---------------------------------------------------------------------------
 // Axis 0 and the products.  A CTA takes a group of target parents (consecutive
 // in tile order, so they share neighbour cells) and a unit of lines; lane =
-// (line, k0).  Per parity of k0: the group's source lines are copied to shared
-// memory and transformed in place (a thread per line); a warp then takes one
-// target parent at a time with the 27 kernel values of its lane in registers
-// and reads each neighbour's value from shared memory (absent neighbours point
-// at a zero line, so the 27 reads are issued together); the sums go to shared
-// memory, are transformed back (a thread per line) and written.  The second
-// parity adds to what the first wrote.
+// (line, k0).  Per parity of k0 the group's source lines are copied to shared
+// memory and transformed in place (a thread per line); a warp then takes two
+// parents that are neighbours along axis 2 (or one) at a time, its lane's 27
+// kernel values in registers: the pair's 36 distinct source values feed 54
+// products (shared-memory bandwidth bounds the kernel with 27 reads each, and
+// longer runs lost more to their short parts than they saved: 20 sparse
+// problems 7.6 ms with single parents, 8.2 ms with runs).  The sums are
+// transformed back (a thread per line) and the two parities added.
 // FP64 products take the three-multiplication form (kr (fr + fi), (kr + ki)
-// fi, (ki - kr) fr) with fr + fi kept beside the sources.
+// fi, (ki - kr) fr) with fr + fi kept beside the sources, and skip absent cells
+// one by one: the FP64 pipe is the bound.
 // ---------------------------------------------------------------------------
 template <typename R, int N>
 __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
-    pf_mac_kernel(const FlGroup* __restrict__ groups, int ngroups, int max_cells, int max_parents,
-                  const uint16_t* __restrict__ rows, const int* __restrict__ cell_col, const int* __restrict__ tgt_col,
+    pf_mac_kernel(const PfGroup* __restrict__ groups, int ngroups, const PfLimits lim,
+                  const uint16_t* __restrict__ items, const int* __restrict__ cell_col, const int* __restrict__ tgt_col,
                   const typename Vec2<R>::type* __restrict__ src, int nsrc, typename Vec2<R>::type* __restrict__ dst,
                   int ndst, const typename Vec2<R>::type* __restrict__ kspec, int src_stride, int dst_stride) {
   using D = PfDims<N>;
@@ -286,33 +283,51 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
   constexpr int NW = kPfMacThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int g = blockIdx.x % ngroups, unit = blockIdx.x / ngroups;
-  const FlGroup gp = groups[g];
+  const PfGroup gp = groups[g];
   const int nc = gp.ncell, nt = gp.nact;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  C2* X = reinterpret_cast<C2*>(smem_raw);                       // [max_cells + 1][33], the last used line zero
-  C2* T = X + (size_t)(max_cells + 1) * kPfStride;               // [max_parents][33]
-  uint16_t* RW = reinterpret_cast<uint16_t*>(smem_raw + pf_row_offset<R>(max_cells, max_parents));  // [max_parents][kPfRow]
-  int* CC = reinterpret_cast<int*>(RW + (size_t)max_parents * kPfRow);
-  int* TC = CC + max_cells;
-  R* Sm = reinterpret_cast<R*>(smem_raw + pf_sum_offset<R>(max_cells, max_parents));  // FP64: fr + fi, [max_cells + 1][33]
+  C2* X = reinterpret_cast<C2*>(smem_raw);                      // [cells + 1][33], line nc is zero
+  C2* T = X + (size_t)(lim.cells + 1) * kPfStride;              // [FP64: 2][parents][33]
+  R* Sm = reinterpret_cast<R*>(smem_raw + pf_sum_offset<R>(lim));  // FP64: fr + fi, [cells + 1][33]
+  uint4* IT = reinterpret_cast<uint4*>(smem_raw + pf_table_offset<R>(lim));  // [items][5]
+  int* CC = reinterpret_cast<int*>(IT + (size_t)lim.items * (kPfItem / 8));
+  int* TC = CC + lim.cells;
 
-  {
-    const int4* r4 = reinterpret_cast<const int4*>(rows + (size_t)gp.row_off * kPfRow);
-    for (int i = tid; i < nt * (kPfRow / 8); i += kPfMacThreads) reinterpret_cast<int4*>(RW)[i] = __ldg(r4 + i);
-  }
   for (int i = tid; i < nc; i += kPfMacThreads) CC[i] = __ldg(cell_col + gp.cell_off + i) + (int)blockIdx.y * src_stride;
-  for (int i = tid; i < nt; i += kPfMacThreads) TC[i] = __ldg(tgt_col + gp.row_off + i) + (int)blockIdx.y * dst_stride;
   if (tid < 32) {
     X[(size_t)nc * kPfStride + tid] = C2{R(0), R(0)};
     if constexpr (G3) Sm[(size_t)nc * kPfStride + tid] = R(0);
   }
   __syncthreads();
   const C2* sbase = src + (size_t)unit * nsrc * 32 + lane;
-  C2* dbase = dst + (size_t)unit * ndst * 32 + lane;
   auto fill = [&]() {
     for (int c = warp; c < nc; c += NW) cp_async_complex<R>(X + c * kPfStride + lane, sbase + (size_t)CC[c] * 32);
   };
   fill();
+  for (int i = tid; i < nt; i += kPfMacThreads) TC[i] = __ldg(tgt_col + gp.row_off + i) + (int)blockIdx.y * dst_stride;
+  for (int i = tid; i < gp.nitem * (kPfItem / 8); i += kPfMacThreads)
+    IT[i] = __ldg(reinterpret_cast<const uint4*>(items) + (size_t)gp.item_off * (kPfItem / 8) + i);
+  C2* dbase = dst + (size_t)unit * ndst * 32 + lane;
+  // FP64 keeps both parities' sums and transforms them back at once (few lines
+  // a group: more of them in flight); FP32 transforms and writes each parity's,
+  // the second adding to the first, which leaves room for larger groups
+  constexpr bool kBoth = G3;
+  auto inverse = [&](int last) {
+    for (int i = tid; i < (kBoth ? 2 : 1) * nt * D::S; i += kPfMacThreads) {
+      const int par = kBoth ? i / (nt * D::S) : last, r = kBoth ? i % (nt * D::S) : i;
+      const int m = D::S == 1 ? r : r % nt;
+      C2* line = T + ((kBoth ? (size_t)par * lim.parents : 0) + m) * kPfStride + (D::S == 1 ? 0 : (r / nt) * H);
+      R xr[H], xi[H];
+#pragma unroll
+      for (int k = 0; k < H; ++k) { const C2 v = line[k]; xr[k] = v.x; xi[k] = v.y; }
+      LineFFT<H, +1, R>::run(xr, xi);
+      if (par)
+#pragma unroll
+        for (int z = 1; z < H; ++z) rotate64<+1>(z * TW, xr[z], xi[z]);
+#pragma unroll
+      for (int z = 0; z < H; ++z) line[z] = C2{xr[z], xi[z]};
+    }
+  };
 #pragma unroll 1
   for (int par = 0; par < 2; ++par) {
     cp_async_wait();
@@ -324,9 +339,9 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll
       for (int z = 0; z < H; ++z) { const C2 v = line[z]; xr[z] = v.x; xi[z] = v.y; }
       if (par)
-#pragma unroll
-        for (int z = 1; z < H; ++z) rotate64<-1>(z * TW, xr[z], xi[z]);
-      LineFFT<H, -1, R>::run(xr, xi);
+        LineFFT<H, -1, R, true>::run(xr, xi);
+      else
+        LineFFT<H, -1, R>::run(xr, xi);
 #pragma unroll
       for (int k = 0; k < H; ++k) line[k] = C2{xr[k], xi[k]};
       if constexpr (G3) {
@@ -335,73 +350,101 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
         for (int k = 0; k < H; ++k) sl[k] = xr[k] + xi[k];
       }
     }
-    R kr[27], ki[27], k2[G3 ? 27 : 1];
+    R k0[27], k1[27], k2[G3 ? 27 : 1];
     {
       const C2* kp = kspec + ((size_t)(unit * 2 + par) * 27) * 32 + lane;
 #pragma unroll
       for (int e = 0; e < 27; ++e) {
         const C2 k = __ldg(kp + e * 32);
-        kr[e] = k.x;
-        ki[e] = G3 ? k.x + k.y : k.y;
+        k0[e] = k.x;
+        k1[e] = G3 ? k.x + k.y : k.y;
         if constexpr (G3) k2[e] = k.y - k.x;
       }
     }
     __syncthreads();
-    for (int m = warp; m < nt; m += NW) {
-      const uint4* rw = reinterpret_cast<const uint4*>(RW + m * kPfRow);
-      uint32_t w[16];
+    C2* Tp = T + (G3 ? (size_t)par * lim.parents * kPfStride : 0) + lane;
+    constexpr int NA = G3 ? 3 : 4;
+    auto product = [&](R (&s)[NA], int e, const C2& f, const R& sum) {
+      if constexpr (G3) {
+        s[0] = fma(k0[e], sum, s[0]);
+        s[1] = fma(k1[e], f.y, s[1]);
+        s[2] = fma(k2[e], f.x, s[2]);
+      } else {
+        s[0] = fma(k0[e], f.x, s[0]);
+        s[1] = fma(k0[e], f.y, s[1]);
+        s[2] = fma(k1[e], f.y, s[2]);
+        s[3] = fma(k1[e], f.x, s[3]);
+      }
+    };
+    auto result = [&](const R (&s)[NA]) {
+      return G3 ? C2{s[0] - s[1], s[0] + s[2]} : C2{s[0] - s[2], s[1] + s[NA - 1]};
+    };
+    const C2* Xl = X + lane;
+    const R* Sl = Sm + lane;
+    for (int it = warp; it < gp.nitem; it += NW) {
+      uint32_t w[kPfItem / 2];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint4 v = rw[q];
+      for (int q = 0; q < kPfItem / 8; ++q) {
+        const uint4 v = IT[it * (kPfItem / 8) + q];
         w[4 * q] = v.x; w[4 * q + 1] = v.y; w[4 * q + 2] = v.z; w[4 * q + 3] = v.w;
       }
-      R a0 = R(0), a1 = R(0), a2 = R(0), a3 = R(0);
+      auto entry = [&](int i) { return (i & 1) ? w[i / 2] >> 16 : w[i / 2] & 0xFFFFu; };
+      const uint32_t m0 = entry(36), flags = entry(38);
+      R a[2][NA];
 #pragma unroll
-      for (int e = 0; e < 27; ++e) {
-        const uint32_t o = (e & 1) ? w[e / 2] >> 16 : w[e / 2] & 0xFFFFu;
-        const C2 f = X[o + lane];
-        if constexpr (G3) {
-          a0 = fma(kr[e], Sm[o + lane], a0);
-          a1 = fma(ki[e], f.y, a1);
-          a2 = fma(k2[e], f.x, a2);
-        } else {
-          a0 = fma(kr[e], f.x, a0);
-          a1 = fma(kr[e], f.y, a1);
-          a2 = fma(ki[e], f.y, a2);
-          a3 = fma(ki[e], f.x, a3);
+      for (int t = 0; t < NA; ++t) a[0][t] = a[1][t] = R(0);
+      // both forms take a parent's 27 products in the same order
+      if (entry(37) == 2) {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          if (!(flags >> r & 1)) continue;  // no sources at this e0 (uniform)
+#pragma unroll
+          for (int c = 3 * r; c < 3 * r + 3; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t o = entry(9 * q + c);
+              if (G3 && o == (uint32_t)nc * kPfStride) continue;
+              const C2 f = Xl[o];
+              const R s = G3 ? Sl[o] : R(0);
+              if (q < 3) product(a[0], 3 * c + q, f, s);
+              if (q > 0) product(a[1], 3 * c + q - 1, f, s);
+            }
+        }
+        Tp[(m0 + 1) * kPfStride] = result(a[1]);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          if (!(flags >> r & 1)) continue;
+#pragma unroll
+          for (int c = 3 * r; c < 3 * r + 3; ++c)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              const uint32_t o = entry(9 * q + c);
+              if (G3 && o == (uint32_t)nc * kPfStride) continue;
+              product(a[0], 3 * c + q, Xl[o], G3 ? Sl[o] : R(0));
+            }
         }
       }
-      T[m * kPfStride + lane] = G3 ? C2{a0 - a1, a0 + a2} : C2{a0 - a2, a1 + a3};
+      Tp[m0 * kPfStride] = result(a[0]);
     }
     __syncthreads();
-    if (par == 0) fill();  // the second parity's copy of the sources, while the sums are transformed back
-    for (int i = tid; i < nt * D::S; i += kPfMacThreads) {
-      const int m = D::S == 1 ? i : i % nt;
-      C2* line = T + m * kPfStride + (D::S == 1 ? 0 : (i / nt) * H);
-      R xr[H], xi[H];
-#pragma unroll
-      for (int k = 0; k < H; ++k) { const C2 v = line[k]; xr[k] = v.x; xi[k] = v.y; }
-      LineFFT<H, +1, R>::run(xr, xi);
-      if (par)
-#pragma unroll
-        for (int z = 1; z < H; ++z) rotate64<+1>(z * TW, xr[z], xi[z]);
-#pragma unroll
-      for (int z = 0; z < H; ++z) line[z] = C2{xr[z], xi[z]};
-    }
-    __syncthreads();
-    for (int m = warp; m < nt; m += NW) {
-      C2 v = T[m * kPfStride + lane];
-      C2* o = dbase + (size_t)TC[m] * 32;
-      if (par) {  // this thread's own first half
-        const C2 h = *o;
-        v.x += h.x;
-        v.y += h.y;
+    if (par == 0) fill();  // the second parity's copy of the sources
+    if (!kBoth || par == 1) {
+      inverse(par);
+      __syncthreads();
+      for (int m = warp; m < nt; m += NW) {
+        C2 v = T[m * kPfStride + lane];
+        C2* o = dbase + (size_t)TC[m] * 32;
+        if (par) {  // the first parity's part: beside this one, or written by this thread
+          const C2 h = kBoth ? T[((size_t)lim.parents + m) * kPfStride + lane] : *o;
+          v.x += h.x;
+          v.y += h.y;
+        }
+        *o = v;
       }
-      *o = v;
     }
   }
 }
-
 // ---------------------------------------------------------------------------
 // Setup (FP64): the 27 parent kernel arrays [27][P][P][P] to spectra, one axis
 // per pass by plain discrete Fourier sums (a few ms once per context).
@@ -515,18 +558,17 @@ static cudaError_t inverse_n(const void* in, const int* tgt_ch, const double* sc
   return cudaGetLastError();
 }
 template <typename R, int N>
-static cudaError_t mac_n(const FlGroup* groups, int ngroups, int max_cells, int max_parents, const uint16_t* rows,
-                         const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
+static cudaError_t mac_n(const PfGroup* groups, int ngroups, const PfLimits& lim, const uint16_t* items, const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
                          const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s) {
   using C2 = typename Vec2<R>::type;
-  const size_t sm = pf_smem_bytes<R>(max_cells, max_parents);
+  const size_t sm = pf_smem_bytes<R>(lim);
   if (sm > kFlSmemBytes || (size_t)PfDims<N>::U * ngroups >= (1u << 31)) return cudaErrorInvalidConfiguration;
   auto k = pf_mac_kernel<R, N>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
   k<<<dim3((unsigned)(PfDims<N>::U * ngroups), ncomp), kPfMacThreads, sm, s>>>(
-      groups, ngroups, max_cells, max_parents, rows, cell_col, tgt_col, reinterpret_cast<const C2*>(src), nsrc,
-      reinterpret_cast<C2*>(dst), ndst, reinterpret_cast<const C2*>(kspec), src_stride, dst_stride);
+      groups, ngroups, lim, items, cell_col, tgt_col, reinterpret_cast<const C2*>(src), nsrc, reinterpret_cast<C2*>(dst),
+      ndst, reinterpret_cast<const C2*>(kspec), src_stride, dst_stride);
   return cudaGetLastError();
 }
 
@@ -538,16 +580,16 @@ cudaError_t launch_pf_forward(int N, const R* nodes, const int* cell_ch, int n, 
   return cudaErrorInvalidValue;
 }
 template <typename R>
-cudaError_t launch_pf_mac(int N, const FlGroup* groups, int ngroups, int max_cells, int max_parents, const uint16_t* rows,
-                          const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
-                          const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s) {
+cudaError_t launch_pf_mac(int N, const PfGroup* groups, int ngroups, const PfLimits& lim, const uint16_t* items,
+                          const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst,
+                          int ndst, const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s) {
   if (ngroups <= 0) return cudaSuccess;
   if (N == 16)
-    return mac_n<R, 16>(groups, ngroups, max_cells, max_parents, rows, cell_col, tgt_col, src, nsrc, dst, ndst, kspec, ncomp,
-                        src_stride, dst_stride, s);
+    return mac_n<R, 16>(groups, ngroups, lim, items, cell_col, tgt_col, src, nsrc, dst, ndst, kspec, ncomp, src_stride,
+                        dst_stride, s);
   if (N == 8)
-    return mac_n<R, 8>(groups, ngroups, max_cells, max_parents, rows, cell_col, tgt_col, src, nsrc, dst, ndst, kspec, ncomp,
-                       src_stride, dst_stride, s);
+    return mac_n<R, 8>(groups, ngroups, lim, items, cell_col, tgt_col, src, nsrc, dst, ndst, kspec, ncomp, src_stride,
+                       dst_stride, s);
   return cudaErrorInvalidValue;
 }
 template <typename R>
@@ -562,8 +604,9 @@ cudaError_t launch_pf_inverse(int N, const void* in, const int* tgt_ch, const do
 #define FLGF_PF_INST(R)                                                                                             \
   template cudaError_t launch_pf_setup<R>(int, const double*, void*, void*, cudaStream_t);                          \
   template cudaError_t launch_pf_forward<R>(int, const R*, const int*, int, void*, cudaStream_t);                   \
-  template cudaError_t launch_pf_mac<R>(int, const FlGroup*, int, int, int, const uint16_t*, const int*, const int*, \
-                                        const void*, int, void*, int, const void*, int, int, int, cudaStream_t);    \
+  template cudaError_t launch_pf_mac<R>(int, const PfGroup*, int, const PfLimits&, const uint16_t*, const int*,       \
+                                        const int*, const void*, int, void*, int, const void*, int, int, \
+                                        int, cudaStream_t);                                                         \
   template cudaError_t launch_pf_inverse<R>(int, const void*, const int*, const double*, int, R*, cudaStream_t);
 FLGF_PF_INST(float)
 FLGF_PF_INST(double)

@@ -1,7 +1,7 @@
 // Host-only check of the tables of the products between parents (parent.cu):
 // in every phase, forward and adjoint, each finest-level target is written
 // exactly once (a child of a target parent, or of the block-wise inverse), the
-// parents' rows and columns say the same as the frequency-lane groups they are
+// parents' items and columns say the same as the frequency-lane groups they are
 // made from, and the sources of the block-wise kernels are all transformed.
 //
 // usage: parent_plan_check <mesh file> <list_pct> <fp64 0|1> <ncomp>
@@ -71,7 +71,8 @@ int main(int argc, char** argv) {
       for (int i = 0; i < LG[g].nsrc; ++i) bad += !fwd.count(I(ph.l_src)[LG[g].src_off + i]);
     const FlGroup* G = reinterpret_cast<const FlGroup*>(base + ph.fl_groups);
     const uint16_t* rows = reinterpret_cast<const uint16_t*>(base + ph.fl_rows);
-    const uint16_t* prow = reinterpret_cast<const uint16_t*>(base + ph.pf_rows);
+    const PfGroup* PG = reinterpret_cast<const PfGroup*>(base + ph.pf_groups);
+    const uint16_t* items = reinterpret_cast<const uint16_t*>(base + ph.pf_items);
     for (int gi = 0; gi < ph.n_fl; ++gi) {
       const FlGroup& g = G[gi];
       bad += (gi < ph.n_pf) != (g.level == 0);
@@ -84,14 +85,29 @@ int main(int argc, char** argv) {
                    (s < 0 ? -1 : s + k * ph.fl_cstride + ph.gid_begin);
         }
       if (g.level > 0) continue;
-      bad += g.nact > ph.pf_max_parents || g.ncell > ph.pf_max_cells;
+      const PfGroup& pg = PG[gi];
+      bad += pg.ncell != g.ncell || pg.nact != g.nact || pg.cell_off != g.cell_off || pg.row_off != g.row_off ||
+             g.nact > ph.pf_lim.parents || g.ncell > ph.pf_lim.cells || pg.nitem > ph.pf_lim.items;
+      std::vector<int> seen(g.nact, 0);
+      for (int i = 0; i < pg.nitem; ++i) {
+        const uint16_t* it = items + (size_t)(pg.item_off + i) * kPfItem;
+        if (it[37] < 1 || it[37] > 2 || it[36] + it[37] > g.nact) { ++bad; continue; }
+        for (int p = 0; p < it[37]; ++p) {
+          const int m = it[36] + p;
+          seen[m]++;
+          // the 27 cells that the kernel multiplies for the parent
+          const uint16_t* row = rows + (size_t)(g.row_off + m) * kFlRowStride;
+          int want_cell[27];
+          std::fill(want_cell, want_cell + 27, g.ncell);
+          for (int j = 0; j < row[0]; ++j) want_cell[row[1 + j] >> 11] = row[1 + j] & 0x7FF;
+          for (int e = 0; e < 27; ++e) {
+            bad += it[9 * (e % 3 + p) + e / 3] != 33 * want_cell[e];
+            bad += want_cell[e] != g.ncell && !((it[38] >> (e / 9)) & 1);
+          }
+        }
+      }
       for (int m = 0; m < g.nact; ++m) {
-        const uint16_t* r = rows + (size_t)(g.row_off + m) * kFlRowStride;
-        const uint16_t* p = prow + (size_t)(g.row_off + m) * kPfRow;
-        int have = 0;
-        for (int e = 0; e < kPfRow; ++e) have += p[e] != 33 * g.ncell;
-        bad += have != r[0];
-        for (int j = 0; j < r[0]; ++j) bad += p[r[1 + j] >> 11] != 33 * (r[1 + j] & 0x7FF);
+        bad += seen[m] != 1;
         for (int k = 0; k < ph.fl_ncomp; ++k)
           for (int a = 0; a < 8; ++a) {
             const int t = I(ph.fl_tgt)[(g.row_off + m) * 8 + a];
