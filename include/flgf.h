@@ -236,8 +236,8 @@ int flgf_get_potential(flgf_blockset* bs, int problem, int level, void* u, int w
  * are not blocks of the level, each once.  Both lists are in Morton order: by
  * the key interleaving the bits of (x, y, z) + 2^20 (bit i of x at key bit
  * 3i + 2, of y at 3i + 1, of z at 3i).  counts (host): {children, buffer}.
- * The call allocates its scratch (about 560 bytes per block) for its duration
- * and synchronises the context stream.  FLGF_EINVAL for a bad argument, a
+ * The call uses scratch of the context (about 560 bytes per block, kept for the
+ * next call up to 64 MB) and synchronises the context stream.  FLGF_EINVAL for a bad argument, a
  * coordinate out of range or nblk > 645277; FLGF_ENOMEM when the scratch
  * cannot be allocated.  The octree and interaction lists are still built on
  * the host by flgf_blockset_create. */

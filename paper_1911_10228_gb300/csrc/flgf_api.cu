@@ -37,6 +37,7 @@ struct flgf_ctx {
   size_t kstride = 0;  // complex elements per octree level
   void* d_pspec = nullptr;  // the 27 parent kernel spectra of the finest octree level (parent.cu)
   std::vector<double> J1;
+  MgScratch mg_scratch;  // flgf_refine_level
   // whether dense tiles of the finest octree level run between parents (all
   // but the FP32 parent-group form, FLGF_CTX_MAC = 0)
   bool parent_form() const { return prec == FLGF_FP64 || mac >= 1; }
@@ -271,6 +272,7 @@ extern "C" void flgf_destroy(flgf_ctx* ctx) {
   cudaFree(ctx->d_J1);
   cudaFree(ctx->d_kspec);
   cudaFree(ctx->d_pspec);
+  cudaFree(ctx->mg_scratch.ptr);
   delete ctx;
 }
 
@@ -2040,7 +2042,7 @@ extern "C" int flgf_refine_level(flgf_ctx* ctx, const void* f, int nblk, const i
     return fail(ctx, FLGF_EINVAL, "refine_level: bad arguments");
   counts[0] = counts[1] = 0;
   const cudaError_t e = launch_refine_level(ctx->N, ctx->prec == FLGF_FP64, f, nblk, coords, rel, flags, children,
-                                            buffer, counts, ctx->stream);
+                                            buffer, counts, ctx->mg_scratch, ctx->stream);
   if (e == cudaErrorInvalidValue)
     return fail(ctx, FLGF_EINVAL, "refine_level: a coordinate outside (-2^19, 2^19) or more than 645277 blocks");
   if (e == cudaErrorMemoryAllocation) return fail(ctx, FLGF_ENOMEM, "refine_level: scratch allocation");
@@ -2059,6 +2061,7 @@ bool ctx_view(const flgf_ctx* c, CtxView* v) {
   v->stream = c->stream;
   v->kspec = c->d_kspec;
   v->kstride = c->kstride;
+  v->pspec = c->d_pspec;
   return true;
 }
 void ctx_set_error(flgf_ctx* c, const char* msg) {

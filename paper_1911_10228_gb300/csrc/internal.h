@@ -20,6 +20,7 @@ struct CtxView {
   cudaStream_t stream;
   const void* kspec;  // [octree level][chunk][343][T]
   size_t kstride;     // complex elements per octree level
+  const void* pspec;  // parent kernel spectra (parent.cu)
 };
 bool ctx_view(const flgf_ctx* c, CtxView* v);
 void ctx_set_error(flgf_ctx* c, const char* msg);
@@ -265,8 +266,14 @@ cudaError_t launch_pf_inverse(int N, const void* in, const int* tgt_ch, const do
 // f: [nblk][N^3] in the context precision; coords, flags, children, buffer on
 // the device, counts on the host (see flgf_refine_level).  cudaErrorInvalidValue
 // for a coordinate outside (-2^19, 2^19) or more than 2^24 / 26 blocks.
+// keep: scratch of the context, grown as needed and given back above 64 MB.
+struct MgScratch {
+  void* ptr = nullptr;
+  size_t bytes = 0;
+};
 cudaError_t launch_refine_level(int N, int prec_fp64, const void* f, int nblk, const int32_t* coords, double rel,
-                                uint8_t* flags, int32_t* children, int32_t* buffer, int* counts, cudaStream_t s);
+                                uint8_t* flags, int32_t* children, int32_t* buffer, int* counts, MgScratch& keep,
+                                cudaStream_t s);
 
 // ---- a1/a5 and multi-resolution stencils (stencil.cu) ----------------------
 // J1: dense 1-D Lagrange matrix [2N][N] (row = child node of the two children, column = parent node).

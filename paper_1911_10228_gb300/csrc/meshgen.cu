@@ -7,12 +7,21 @@
 //
 // Morton order: blocks compare by the key that interleaves the bits of
 // (x + 2^20, y + 2^20, z + 2^20), bit i of x at key bit 3i + 2, of y at 3i + 1,
-// of z at 3i (|coordinates| < 2^20, 21 bits per axis).  Keys are sorted by a
-// stable least-significant-bit-first split per bit, run only for the bits that
-// vary among the keys (their OR differs from their AND).
+// of z at 3i (|coordinates| < 2^20, 21 bits per axis).  Bit 63 carries a
+// block's flag.
+//
+// The step is bound by launches and host round trips, not by its data (16^3
+// blocks: the 67 MB of source are read in 10 us), so: the level's keys are
+// sorted once, by a radix sort of 8 bits a pass over the bits that can vary;
+// the children of the sorted flagged blocks are then in order as they are
+// (halving the coordinates keeps the order of the keys); of the neighbours only
+// those missing from the level are listed and sorted.  4096 blocks with 459
+// flagged, a call: 1.6 ms with a stable split of five launches per varying bit of
+// three sorts, 459 x 26 candidates sorted and an allocation per scratch array;
+// 0.18 ms (84 us of kernels, three round trips).
+#include <algorithm>
 #include <cstdint>
 #include <utility>
-#include <vector>
 
 #include "flgf.h"
 #include "internal.h"
@@ -21,9 +30,15 @@ namespace flgf {
 
 namespace {
 
-constexpr int kMgThreads = 1024;         // scan tile
+constexpr int kMgThreads = 1024;
+// keys per CTA of a radix pass: 1024 for lists of up to 2^18 keys (more CTAs:
+// the passes are latency-bound), 4096 beyond (fewer digit counts to scan)
+constexpr int mg_tile(size_t n) { return n <= (1u << 18) ? 1024 : 4096; }
+constexpr size_t kMgKeepBytes = 64u << 20;  // scratch kept by the context between calls
+constexpr int kMgDigits = 256;
 constexpr int kMgCoordBias = 1 << 20;    // coordinates + bias are in [0, 2^21)
-constexpr int kMgMaxKeys = 1 << 24;      // one-CTA scan of tile sums: <= 16384 tiles
+constexpr int kMgMaxKeys = 1 << 24;
+constexpr uint64_t kMgFlag = 1ull << 63;
 
 __host__ __device__ inline uint64_t spread3(uint32_t v) {
   uint64_t x = v & 0x1fffffu;
@@ -53,316 +68,337 @@ __device__ inline void morton_decode(uint64_t k, int32_t* c) {
   c[2] = (int32_t)compact3(k) - kMgCoordBias;
 }
 
-// max |f| over each block (one CTA per block)
-template <typename R>
-__global__ void block_absmax_kernel(const R* __restrict__ f, int n3, R* __restrict__ bmax) {
-  __shared__ R red[256];
-  const R* b = f + (size_t)blockIdx.x * n3;
-  R m = R(0);
-  for (int i = threadIdx.x; i < n3; i += blockDim.x) m = fmax(m, fabs(b[i]));
-  red[threadIdx.x] = m;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) bmax[blockIdx.x] = red[0];
-}
-
-// one CTA: the level maximum, then the flags (comparison in FP64)
-template <typename R>
-__global__ void flag_kernel(const R* __restrict__ bmax, int n, double rel, uint8_t* __restrict__ flags,
-                            uint32_t* __restrict__ nflag) {
-  __shared__ double red[kMgThreads];
-  __shared__ uint32_t cnt;
-  double m = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmax(m, (double)bmax[i]);
-  red[threadIdx.x] = m;
-  if (threadIdx.x == 0) cnt = 0;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  const double thr = rel * red[0];
-  const bool any = red[0] > 0.0;
-  uint32_t local = 0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const uint8_t v = any && (double)bmax[i] > thr;
-    flags[i] = v;
-    local += v;
-  }
-  atomicAdd(&cnt, local);
-  __syncthreads();
-  if (threadIdx.x == 0) *nflag = cnt;
-}
-
-// candidates of the flagged blocks: 8 children keys or 26 neighbour keys each
-// (written at slot rank * per + j; rank = exclusive prefix of the flags)
-__global__ void emit_kernel(const int32_t* __restrict__ coords, const uint8_t* __restrict__ flags,
-                            const uint32_t* __restrict__ rank, int n, int children, uint64_t* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || !flags[i]) return;
-  const int x = coords[3 * i], y = coords[3 * i + 1], z = coords[3 * i + 2];
-  if (children) {
-    for (int a = 0; a < 8; ++a)
-      out[(size_t)rank[i] * 8 + a] = morton_key(2 * x + (a >> 2), 2 * y + ((a >> 1) & 1), 2 * z + (a & 1));
-  } else {
-    int j = 0;
-    for (int e = 0; e < 27; ++e) {
-      if (e == 13) continue;
-      out[(size_t)rank[i] * 26 + j++] = morton_key(x + e / 9 - 1, y + (e / 3) % 3 - 1, z + e % 3 - 1);
-    }
-  }
-}
-
-// 1 in *bad when a coordinate is outside (-2^19, 2^19) (children must fit the keys)
-__global__ void check_coords_kernel(const int32_t* __restrict__ coords, int n, uint32_t* __restrict__ bad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 3 * n) return;
-  const int v = coords[i];
-  if (v <= -(kMgCoordBias >> 1) || v >= (kMgCoordBias >> 1)) atomicOr(bad, 1u);
-}
-
-__global__ void level_keys_kernel(const int32_t* __restrict__ coords, int n, uint64_t* __restrict__ keys) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) keys[i] = morton_key(coords[3 * i], coords[3 * i + 1], coords[3 * i + 2]);
-}
-
-// OR and AND of all keys (one CTA): the bits that vary
-__global__ void key_bits_kernel(const uint64_t* __restrict__ keys, int n, uint64_t* __restrict__ out) {
-  __shared__ unsigned long long o, a;
-  if (threadIdx.x == 0) { o = 0ull; a = ~0ull; }
-  __syncthreads();
-  unsigned long long lo = 0ull, la = ~0ull;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) { lo |= keys[i]; la &= keys[i]; }
-  atomicOr(&o, lo);
-  atomicAnd(&a, la);
-  __syncthreads();
-  if (threadIdx.x == 0) { out[0] = o; out[1] = a; }
-}
-
-// keep[i] for a predicate; rank by exclusive scan
-// (a) per-tile scan of 0/1 values, tile sums
-__global__ void scan_tiles_kernel(const uint8_t* __restrict__ keep, int n, uint32_t* __restrict__ rank,
-                                  uint32_t* __restrict__ tile_sum) {
-  __shared__ uint32_t s[kMgThreads];
-  const int i = blockIdx.x * kMgThreads + threadIdx.x;
-  const uint32_t v = i < n ? keep[i] : 0u;
-  s[threadIdx.x] = v;
-  __syncthreads();
-  for (int w = 1; w < kMgThreads; w <<= 1) {  // Hillis-Steele inclusive scan
-    const uint32_t t = threadIdx.x >= (unsigned)w ? s[threadIdx.x - w] : 0u;
-    __syncthreads();
-    s[threadIdx.x] += t;
-    __syncthreads();
-  }
-  if (i < n) rank[i] = s[threadIdx.x] - v;
-  if (threadIdx.x == kMgThreads - 1) tile_sum[blockIdx.x] = s[threadIdx.x];
-}
-// (b) one CTA: exclusive scan of the tile sums in place, total at [ntiles]
-__global__ void scan_sums_kernel(uint32_t* __restrict__ tile_sum, int ntiles) {
-  __shared__ uint32_t s[kMgThreads];
-  __shared__ uint32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < ntiles; base += kMgThreads) {
-    const int i = base + threadIdx.x;
-    const uint32_t v = i < ntiles ? tile_sum[i] : 0u;
-    s[threadIdx.x] = v;
-    __syncthreads();
-    for (int w = 1; w < kMgThreads; w <<= 1) {
-      const uint32_t t = threadIdx.x >= (unsigned)w ? s[threadIdx.x - w] : 0u;
-      __syncthreads();
-      s[threadIdx.x] += t;
-      __syncthreads();
-    }
-    if (i < ntiles) tile_sum[i] = carry + s[threadIdx.x] - v;
-    __syncthreads();
-    if (threadIdx.x == kMgThreads - 1) carry += s[threadIdx.x];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) tile_sum[ntiles] = carry;
-}
-// (c) rank += tile offset
-__global__ void scan_add_kernel(uint32_t* __restrict__ rank, int n, const uint32_t* __restrict__ tile_off) {
-  const int i = blockIdx.x * kMgThreads + threadIdx.x;
-  if (i < n) rank[i] += tile_off[blockIdx.x];
-}
-
-// stable split on one bit: zeros first (in order), then ones
-__global__ void bit_kernel(const uint64_t* __restrict__ keys, int n, int bit, uint8_t* __restrict__ zero) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) zero[i] = !((keys[i] >> bit) & 1ull);
-}
-__global__ void split_scatter_kernel(const uint64_t* __restrict__ in, int n, const uint8_t* __restrict__ zero,
-                                     const uint32_t* __restrict__ rank, const uint32_t* __restrict__ nzero,
-                                     uint64_t* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t z = *nzero;
-  out[zero[i] ? rank[i] : z + ((uint32_t)i - rank[i])] = in[i];
-}
-
-// keep[i]: first of its run of equal sorted keys, and (when lvl != null) not a
-// key of the sorted level list
-__global__ void select_kernel(const uint64_t* __restrict__ keys, int n, const uint64_t* __restrict__ lvl, int nl,
-                              uint8_t* __restrict__ keep) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t k = keys[i];
-  bool v = i == 0 || keys[i - 1] != k;
-  if (v && lvl) {
-    int lo = 0, hi = nl;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (lvl[mid] < k) lo = mid + 1; else hi = mid;
-    }
-    v = !(lo < nl && lvl[lo] == k);
-  }
-  keep[i] = v;
-}
-__global__ void compact_decode_kernel(const uint64_t* __restrict__ keys, int n, const uint8_t* __restrict__ keep,
-                                      const uint32_t* __restrict__ rank, int32_t* __restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && keep[i]) morton_decode(keys[i], out + 3 * (size_t)rank[i]);
-}
-
-// scratch for lists of up to n keys
-struct MgWork {
-  uint64_t *k0 = nullptr, *k1 = nullptr, *lvl = nullptr, *bits = nullptr;
-  uint8_t* f8 = nullptr;
-  uint32_t *rank = nullptr, *tiles = nullptr, *cnt = nullptr;
+// What the host needs to know of a level.
+struct MgInfo {
+  unsigned long long maxbits;  // largest |f| (bits of a non-negative number order like it)
+  int lo[3], hi[3];            // range of the coordinates
+  uint32_t bad, nflag, nparent, ncand, nbuf;  // nparent: flagged blocks, each coordinate once
 };
 
-inline int nblk_of(size_t n, int t) { return (int)((n + t - 1) / t); }
-
-cudaError_t exclusive_scan(const uint8_t* keep, int n, uint32_t* rank, uint32_t* tiles, cudaStream_t s) {
-  const int nt = nblk_of((size_t)n, kMgThreads);
-  scan_tiles_kernel<<<nt, kMgThreads, 0, s>>>(keep, n, rank, tiles);
-  scan_sums_kernel<<<1, kMgThreads, 0, s>>>(tiles, nt);
-  scan_add_kernel<<<nt, kMgThreads, 0, s>>>(rank, n, tiles);
-  return cudaGetLastError();  // total at tiles[nt]
+__global__ void info_init_kernel(MgInfo* info) {
+  *info = MgInfo{0ull, {1 << 20, 1 << 20, 1 << 20}, {-(1 << 20), -(1 << 20), -(1 << 20)}, 0u, 0u, 0u, 0u, 0u};
 }
 
-// stable sort of keys[0..n) (result in *keys; *other is scratch)
-cudaError_t sort_keys(uint64_t** keys, uint64_t** other, int n, MgWork& w, cudaStream_t s) {
-  if (n <= 1) return cudaSuccess;
-  key_bits_kernel<<<1, kMgThreads, 0, s>>>(*keys, n, w.bits);
-  uint64_t hb[2];
-  cudaError_t e = cudaMemcpyAsync(hb, w.bits, sizeof(hb), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return e;
-  const uint64_t vary = hb[0] & ~hb[1];
-  const int nt = nblk_of((size_t)n, kMgThreads);
-  for (int b = 0; b < 64; ++b) {
-    if (!((vary >> b) & 1ull)) continue;
-    bit_kernel<<<nt, kMgThreads, 0, s>>>(*keys, n, b, w.f8);
-    if ((e = exclusive_scan(w.f8, n, w.rank, w.tiles, s)) != cudaSuccess) return e;
-    split_scatter_kernel<<<nt, kMgThreads, 0, s>>>(*keys, n, w.f8, w.rank, w.tiles + nt, *other);
+__device__ __forceinline__ unsigned long long abs_bits(float v) { return (unsigned long long)__float_as_uint(v); }
+__device__ __forceinline__ unsigned long long abs_bits(double v) { return (unsigned long long)__double_as_longlong(v); }
+template <typename R> __device__ __forceinline__ double from_bits(unsigned long long b);
+template <> __device__ __forceinline__ double from_bits<float>(unsigned long long b) { return (double)__uint_as_float((unsigned)b); }
+template <> __device__ __forceinline__ double from_bits<double>(unsigned long long b) { return __longlong_as_double((long long)b); }
+
+// max |f| over each block (one CTA per block; NaN counts as absent, as in fmax),
+// the level's maximum and coordinate range, the block's key; bad = 1 when a
+// coordinate is outside (-2^19, 2^19) (children must fit the keys)
+template <typename R>
+__global__ void __launch_bounds__(256) block_kernel(const R* __restrict__ f, int n3, const int32_t* __restrict__ coords,
+                                                    R* __restrict__ bmax, uint64_t* __restrict__ keys, MgInfo* info) {
+  __shared__ R red[8];
+  const R* b = f + (size_t)blockIdx.x * n3;
+  R m = R(0);
+  if (reinterpret_cast<uintptr_t>(f) % 16 == 0) {  // a block is a multiple of 16 bytes
+    constexpr int V = 16 / (int)sizeof(R);
+    for (int i = threadIdx.x; i < n3 / V; i += 256) {
+      const int4 q = __ldg(reinterpret_cast<const int4*>(b) + i);
+      const R* r = reinterpret_cast<const R*>(&q);
+#pragma unroll
+      for (int j = 0; j < V; ++j) m = fmax(m, fabs(r[j]));
+    }
+  } else {
+    for (int i = threadIdx.x; i < n3; i += 256) m = fmax(m, fabs(b[i]));
+  }
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) m = fmax(m, red[w]);
+    bmax[blockIdx.x] = m;
+    if (m > R(0)) atomicMax(&info->maxbits, abs_bits(m));
+    int c[3];
+    for (int a = 0; a < 3; ++a) {
+      c[a] = coords[3 * (size_t)blockIdx.x + a];
+      if (c[a] <= -(kMgCoordBias >> 1) || c[a] >= (kMgCoordBias >> 1)) {
+        info->bad = 1u;
+        c[a] = 0;
+      }
+      if (c[a] < info->lo[a]) atomicMin(&info->lo[a], c[a]);
+      if (c[a] > info->hi[a]) atomicMax(&info->hi[a], c[a]);
+    }
+    keys[blockIdx.x] = morton_key(c[0], c[1], c[2]);
+  }
+}
+
+// the flags (compared in FP64), also into bit 63 of the keys, and their number
+template <typename R>
+__global__ void flag_kernel(const R* __restrict__ bmax, int n, double rel, uint8_t* __restrict__ flags,
+                            uint64_t* __restrict__ keys, MgInfo* info) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const double top = from_bits<R>(info->maxbits);
+  const bool v = i < n && top > 0.0 && (double)bmax[i] > rel * top;
+  if (i < n) {
+    flags[i] = v;
+    if (v) keys[i] |= kMgFlag;
+  }
+  const unsigned w = __ballot_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0 && w) atomicAdd(&info->nflag, (uint32_t)__popc(w));
+}
+
+// Exclusive scan over the CTA (kMgThreads threads, one value each, replaced by
+// its prefix); returns the total.
+__device__ __forceinline__ uint32_t block_scan(uint32_t& v, uint32_t* ws) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t x = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += t;
+  }
+  if (lane == 31) ws[warp] = x;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t y = ws[lane];
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xffffffffu, y, o);
+      if (lane >= o) y += t;
+    }
+    ws[32 + lane] = y;
+  }
+  __syncthreads();
+  const uint32_t total = ws[63];
+  v = x - v + (warp ? ws[32 + warp - 1] : 0u);
+  __syncthreads();
+  return total;
+}
+
+__device__ __forceinline__ uint32_t radix_digit(uint64_t k, int shift) {
+  return (uint32_t)((k & ~kMgFlag) >> shift) & (kMgDigits - 1);
+}
+
+// Radix pass, 8 bits at `shift`: digit counts per tile [digit][tile], one CTA's
+// exclusive scan of them, stable scatter.
+__global__ void __launch_bounds__(kMgThreads) radix_count_kernel(const uint64_t* __restrict__ keys, int n, int shift,
+                                                                 uint32_t* __restrict__ counts, int ntiles, int tile) {
+  __shared__ uint32_t h[kMgDigits];
+  if (threadIdx.x < kMgDigits) h[threadIdx.x] = 0;
+  __syncthreads();
+  for (int j = 0; j < tile; j += kMgThreads) {
+    const int i = blockIdx.x * tile + j + threadIdx.x;
+    if (i < n) atomicAdd(&h[radix_digit(keys[i], shift)], 1u);
+  }
+  __syncthreads();
+  if (threadIdx.x < kMgDigits) counts[(size_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+}
+__global__ void __launch_bounds__(kMgThreads) scan_kernel(uint32_t* __restrict__ v, int n, uint32_t* __restrict__ total) {
+  __shared__ uint32_t ws[64];
+  uint32_t carry = 0;
+  for (int base = 0; base < n; base += 4 * kMgThreads) {
+    uint32_t x[4], sum = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = base + 4 * (int)threadIdx.x + j;
+      x[j] = i < n ? v[i] : 0u;
+      sum += x[j];
+    }
+    uint32_t at = sum;
+    const uint32_t t = block_scan(at, ws);
+    at += carry;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = base + 4 * (int)threadIdx.x + j;
+      if (i < n) v[i] = at;
+      at += x[j];
+    }
+    carry += t;
+  }
+  if (total && threadIdx.x == 0) *total = carry;
+}
+__global__ void __launch_bounds__(kMgThreads) radix_scatter_kernel(const uint64_t* __restrict__ in, int n, int shift,
+                                                                   const uint32_t* __restrict__ offs, int ntiles, int tile,
+                                                                   uint64_t* __restrict__ out) {
+  __shared__ uint32_t at[kMgDigits];           // next slot of each digit
+  __shared__ uint16_t cnt[32][kMgDigits];      // per warp, then its exclusive prefix over the warps
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < kMgDigits) at[threadIdx.x] = offs[(size_t)threadIdx.x * ntiles + blockIdx.x];
+  for (int j = 0; j < tile; j += kMgThreads) {
+    const int i = blockIdx.x * tile + j + threadIdx.x;
+    if (blockIdx.x * tile + j >= n) break;  // uniform
+    for (int q = threadIdx.x; q < 32 * kMgDigits; q += kMgThreads) cnt[0][q] = 0;
+    __syncthreads();
+    const uint64_t k = i < n ? in[i] : 0ull;
+    const uint32_t d = i < n ? radix_digit(k, shift) : kMgDigits;  // 256: past the end
+    const unsigned same = __match_any_sync(0xffffffffu, d);
+    const uint32_t rank = __popc(same & ((1u << lane) - 1u));
+    if (d < kMgDigits && rank == 0) cnt[warp][d] = (uint16_t)__popc(same);
+    __syncthreads();
+    if (threadIdx.x < kMgDigits) {
+      uint32_t run = 0;
+      for (int w = 0; w < 32; ++w) {
+        const uint32_t c = cnt[w][threadIdx.x];
+        cnt[w][threadIdx.x] = (uint16_t)run;
+        run += c;
+      }
+      cnt[0][threadIdx.x] = (uint16_t)run;  // warp 0's prefix is zero: its slot carries the total
+    }
+    __syncthreads();
+    if (d < kMgDigits) out[at[d] + (warp ? cnt[warp][d] : 0u) + rank] = k;
+    __syncthreads();
+    if (threadIdx.x < kMgDigits) at[threadIdx.x] += cnt[0][threadIdx.x];
+    __syncthreads();
+  }
+}
+
+// mark[i] = 1 where sorted key i carries the flag as the first flagged one of
+// its coordinates (flagged = 1: the parents of the children), or is the first of
+// its run of equal keys (flagged = 0: neighbours)
+__device__ __forceinline__ bool marked(const uint64_t* __restrict__ keys, int i, int flagged) {
+  const uint64_t k = keys[i];
+  if (!flagged) return i == 0 || keys[i - 1] != k;
+  if (!(k & kMgFlag)) return false;
+  for (int j = i - 1; j >= 0 && ((keys[j] ^ k) & ~kMgFlag) == 0; --j)
+    if (keys[j] & kMgFlag) return false;
+  return true;
+}
+__global__ void mark_kernel(const uint64_t* __restrict__ keys, int n, int flagged, uint32_t* __restrict__ mark) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) mark[i] = marked(keys, i, flagged);
+}
+
+// children of the flagged blocks in the order of their sorted keys
+__global__ void children_kernel(const uint64_t* __restrict__ keys, int n, const uint32_t* __restrict__ rank,
+                                int32_t* __restrict__ out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t / 8, a = t % 8;
+  if (i >= n || !marked(keys, i, 1)) return;
+  int32_t c[3];
+  morton_decode(keys[i] & ~kMgFlag, c);
+  int32_t* o = out + 3 * ((size_t)rank[i] * 8 + a);
+  o[0] = 2 * c[0] + (a >> 2);
+  o[1] = 2 * c[1] + ((a >> 1) & 1);
+  o[2] = 2 * c[2] + (a & 1);
+}
+
+// keys of the flagged blocks' neighbours that are not blocks of the level (any order)
+__global__ void missing_kernel(const uint64_t* __restrict__ keys, int n, uint64_t* __restrict__ out, MgInfo* info) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t / 32, e = t % 32;  // a warp per block
+  if (i >= n || !(keys[i] & kMgFlag)) return;                                   // uniform
+  bool miss = e < 27 && e != 13;
+  uint64_t k = 0;
+  if (miss) {
+    int32_t c[3];
+    morton_decode(keys[i] & ~kMgFlag, c);
+    k = morton_key(c[0] + e / 9 - 1, c[1] + (e / 3) % 3 - 1, c[2] + e % 3 - 1);
+    int lo = 0, hi = n;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((keys[mid] & ~kMgFlag) < k) lo = mid + 1; else hi = mid;
+    }
+    miss = !(lo < n && (keys[lo] & ~kMgFlag) == k);
+  }
+  const unsigned w = __ballot_sync(0xffffffffu, miss);
+  if (!w) return;
+  uint32_t base = 0;
+  if (e == 0) base = atomicAdd(&info->ncand, (uint32_t)__popc(w));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (miss) out[base + __popc(w & ((1u << e) - 1u))] = k;
+}
+
+__global__ void unique_kernel(const uint64_t* __restrict__ keys, int n, const uint32_t* __restrict__ rank,
+                              int32_t* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n && marked(keys, i, 0)) morton_decode(keys[i], out + 3 * (size_t)rank[i]);
+}
+
+inline int ceil_div(size_t n, int t) { return (int)((n + t - 1) / t); }
+
+// stable sort of keys[0..n) by their low `bits` bits (result in *keys; *other and counts are scratch)
+void sort_keys(uint64_t** keys, uint64_t** other, int n, int bits, uint32_t* counts, cudaStream_t s) {
+  if (n <= 1) return;
+  const int tile = mg_tile(n), nt = ceil_div((size_t)n, tile);
+  for (int shift = 0; shift < bits; shift += 8) {
+    radix_count_kernel<<<nt, kMgThreads, 0, s>>>(*keys, n, shift, counts, nt, tile);
+    scan_kernel<<<1, kMgThreads, 0, s>>>(counts, kMgDigits * nt, nullptr);
+    radix_scatter_kernel<<<nt, kMgThreads, 0, s>>>(*keys, n, shift, counts, nt, tile, *other);
     std::swap(*keys, *other);
   }
-  return cudaGetLastError();
-}
-
-// sorted, deduplicated (and, with lvl, not in the level) keys -> coordinates;
-// returns the count through *count (host)
-cudaError_t finish_list(uint64_t** keys, uint64_t** other, int n, const uint64_t* lvl, int nl, int32_t* out,
-                        int* count, MgWork& w, cudaStream_t s) {
-  *count = 0;
-  if (n == 0) return cudaSuccess;
-  cudaError_t e = sort_keys(keys, other, n, w, s);
-  if (e != cudaSuccess) return e;
-  const int nt = nblk_of((size_t)n, kMgThreads);
-  select_kernel<<<nt, kMgThreads, 0, s>>>(*keys, n, lvl, nl, w.f8);
-  if ((e = exclusive_scan(w.f8, n, w.rank, w.tiles, s)) != cudaSuccess) return e;
-  compact_decode_kernel<<<nt, kMgThreads, 0, s>>>(*keys, n, w.f8, w.rank, out);
-  uint32_t c = 0;
-  e = cudaMemcpyAsync(&c, w.tiles + nt, sizeof(c), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  *count = (int)c;
-  return e;
 }
 
 }  // namespace
 
 template <typename R>
 static cudaError_t refine_level(int N, const R* f, int nblk, const int32_t* coords, double rel, uint8_t* flags,
-                                int32_t* children, int32_t* buffer, int* counts, cudaStream_t s) {
-  const size_t nmax = (size_t)nblk * 26;
-  MgWork w;
-  std::vector<void*> owned;
+                                int32_t* children, int32_t* buffer, int* counts, MgScratch& keep, cudaStream_t s) {
+  counts[0] = counts[1] = 0;
+  // one array: level keys (two), neighbour keys (two), ranks, digit counts, block maxima, info
+  const size_t n = (size_t)nblk, ncap = 26 * n;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t o_lvl0 = 0, o_lvl1 = o_lvl0 + up(8 * n), o_c0 = o_lvl1 + up(8 * n), o_c1 = o_c0 + up(8 * ncap);
+  const size_t o_rank = o_c1 + up(8 * ncap), o_cnt = o_rank + up(4 * ncap);
+  const size_t o_max = o_cnt + up(4 * (size_t)kMgDigits * std::max(ceil_div(ncap, mg_tile(ncap)), ceil_div(std::min<size_t>(ncap, 1u << 18), 1024))), o_info = o_max + up(sizeof(R) * n);
   cudaError_t e = cudaSuccess;
-  auto get = [&](void** p, size_t bytes) {
-    if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-    if (e == cudaSuccess) owned.push_back(*p);
+  if (keep.bytes < o_info + 256) {
+    cudaFree(keep.ptr);
+    keep = MgScratch();
+    e = cudaMalloc(&keep.ptr, o_info + 256);
+    if (e != cudaSuccess) return e;
+    keep.bytes = o_info + 256;
+  }
+  char* base = (char*)keep.ptr;
+  uint64_t* lvl = (uint64_t*)(base + o_lvl0);
+  uint64_t* lvl1 = (uint64_t*)(base + o_lvl1);
+  uint64_t* cand = (uint64_t*)(base + o_c0);
+  uint64_t* cand1 = (uint64_t*)(base + o_c1);
+  uint32_t* rank = (uint32_t*)(base + o_rank);
+  uint32_t* cnt = (uint32_t*)(base + o_cnt);
+  R* bmax = (R*)(base + o_max);
+  MgInfo* info = (MgInfo*)(base + o_info);
+  MgInfo h{};
+  auto read_info = [&]() {
+    cudaError_t r = cudaGetLastError();
+    if (r == cudaSuccess) r = cudaMemcpyAsync(&h, info, sizeof(h), cudaMemcpyDeviceToHost, s);
+    return r == cudaSuccess ? cudaStreamSynchronize(s) : r;
   };
-  R* bmax = nullptr;
-  get((void**)&bmax, sizeof(R) * nblk);
-  get((void**)&w.k0, sizeof(uint64_t) * nmax);
-  get((void**)&w.k1, sizeof(uint64_t) * nmax);
-  get((void**)&w.lvl, sizeof(uint64_t) * nblk);
-  get((void**)&w.bits, sizeof(uint64_t) * 2);
-  get((void**)&w.f8, nmax);
-  get((void**)&w.rank, sizeof(uint32_t) * nmax);
-  get((void**)&w.tiles, sizeof(uint32_t) * (nblk_of(nmax, kMgThreads) + 1));
-  get((void**)&w.cnt, sizeof(uint32_t) * 2);
-  uint32_t nflag = 0;
-  if (e == cudaSuccess) {
-    uint32_t bad = 0;
-    e = cudaMemsetAsync(w.cnt + 1, 0, sizeof(uint32_t), s);
-    check_coords_kernel<<<nblk_of((size_t)3 * nblk, 256), 256, 0, s>>>(coords, nblk, w.cnt + 1);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, w.cnt + 1, sizeof(bad), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess && bad) e = cudaErrorInvalidValue;
-  }
-  if (e == cudaSuccess) {
-    const int nb = nblk_of((size_t)nblk, kMgThreads);
-    block_absmax_kernel<R><<<nblk, 256, 0, s>>>(f, N * N * N, bmax);
-    flag_kernel<R><<<1, kMgThreads, 0, s>>>(bmax, nblk, rel, flags, w.cnt);
-    e = exclusive_scan(flags, nblk, w.rank, w.tiles, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&nflag, w.cnt, sizeof(nflag), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    // children of the flagged blocks (distinct for distinct parents)
-    if (e == cudaSuccess && nflag > 0) {
-      emit_kernel<<<nb, kMgThreads, 0, s>>>(coords, flags, w.rank, nblk, 1, w.k0);
-      e = finish_list(&w.k0, &w.k1, (int)(8 * nflag), nullptr, 0, children, &counts[0], w, s);
-    } else {
-      counts[0] = 0;
+  info_init_kernel<<<1, 1, 0, s>>>(info);
+  block_kernel<R><<<nblk, 256, 0, s>>>(f, N * N * N, coords, bmax, lvl, info);
+  flag_kernel<R><<<ceil_div(n, 256), 256, 0, s>>>(bmax, nblk, rel, flags, lvl, info);
+  e = read_info();
+  if (e == cudaSuccess && h.bad) e = cudaErrorInvalidValue;
+  if (e == cudaSuccess && h.nflag > 0) {
+    // key bits that can vary among the level's blocks and their neighbours
+    int bits = 1;
+    for (int a = 0; a < 3; ++a) {
+      const uint32_t x = (uint32_t)(h.lo[a] - 1 + kMgCoordBias) ^ (uint32_t)(h.hi[a] + 1 + kMgCoordBias);
+      int b = 0;
+      while (x >> b) ++b;
+      bits = std::max(bits, 3 * b);
     }
-    // the level's keys, sorted, then the neighbours missing from the level
-    if (e == cudaSuccess && nflag > 0) {
-      level_keys_kernel<<<nb, kMgThreads, 0, s>>>(coords, nblk, w.lvl);
-      uint64_t* lvl = w.lvl;
-      uint64_t* tmp = w.k1;
-      e = sort_keys(&lvl, &tmp, nblk, w, s);
-      if (e == cudaSuccess && lvl != w.lvl)
-        e = cudaMemcpyAsync(w.lvl, lvl, sizeof(uint64_t) * nblk, cudaMemcpyDeviceToDevice, s);
-      if (e == cudaSuccess) {
-        e = exclusive_scan(flags, nblk, w.rank, w.tiles, s);  // ranks again (the sorts reused the scratch)
-        emit_kernel<<<nb, kMgThreads, 0, s>>>(coords, flags, w.rank, nblk, 0, w.k0);
-        e = finish_list(&w.k0, &w.k1, (int)(26 * nflag), w.lvl, nblk, buffer, &counts[1], w, s);
-      }
-    } else {
-      counts[1] = 0;
+    sort_keys(&lvl, &lvl1, nblk, bits, cnt, s);
+    mark_kernel<<<ceil_div(n, 256), 256, 0, s>>>(lvl, nblk, 1, rank);
+    scan_kernel<<<1, kMgThreads, 0, s>>>(rank, nblk, &info->nparent);
+    children_kernel<<<ceil_div(8 * n, 256), 256, 0, s>>>(lvl, nblk, rank, children);
+    missing_kernel<<<ceil_div(32 * n, 256), 256, 0, s>>>(lvl, nblk, cand, info);
+    e = read_info();
+    const int nc = (int)h.ncand;
+    if (e == cudaSuccess && nc > 0) {
+      sort_keys(&cand, &cand1, nc, bits, cnt, s);
+      mark_kernel<<<ceil_div((size_t)nc, 256), 256, 0, s>>>(cand, nc, 0, rank);
+      scan_kernel<<<1, kMgThreads, 0, s>>>(rank, nc, &info->nbuf);
+      unique_kernel<<<ceil_div((size_t)nc, 256), 256, 0, s>>>(cand, nc, rank, buffer);
+      e = read_info();
+    }
+    if (e == cudaSuccess) {
+      counts[0] = 8 * (int)h.nparent;
+      counts[1] = (int)h.nbuf;
     }
   }
-  if (e == cudaSuccess) e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  for (void* p : owned) cudaFree(p);
+  if (keep.bytes > kMgKeepBytes) {
+    cudaFree(keep.ptr);
+    keep = MgScratch();
+  }
   return e;
 }
 
-template cudaError_t refine_level<float>(int, const float*, int, const int32_t*, double, uint8_t*, int32_t*, int32_t*,
-                                         int*, cudaStream_t);
-template cudaError_t refine_level<double>(int, const double*, int, const int32_t*, double, uint8_t*, int32_t*,
-                                          int32_t*, int*, cudaStream_t);
-
 cudaError_t launch_refine_level(int N, int prec_fp64, const void* f, int nblk, const int32_t* coords, double rel,
-                                uint8_t* flags, int32_t* children, int32_t* buffer, int* counts, cudaStream_t s) {
+                                uint8_t* flags, int32_t* children, int32_t* buffer, int* counts, MgScratch& keep,
+                                cudaStream_t s) {
   if ((size_t)nblk * 26 > (size_t)kMgMaxKeys) return cudaErrorInvalidValue;
-  return prec_fp64 ? refine_level<double>(N, (const double*)f, nblk, coords, rel, flags, children, buffer, counts, s)
-                   : refine_level<float>(N, (const float*)f, nblk, coords, rel, flags, children, buffer, counts, s);
+  return prec_fp64 ? refine_level<double>(N, (const double*)f, nblk, coords, rel, flags, children, buffer, counts, keep, s)
+                   : refine_level<float>(N, (const float*)f, nblk, coords, rel, flags, children, buffer, counts, keep, s);
 }
 
 }  // namespace flgf
