@@ -13,8 +13,9 @@
 // It computes u = h^2 (G * f) over at most kStaticMaxBlocks blocks whose
 // octree has a single level (all blocks within a 4 x 4 x 4 box aligned to
 // even coordinates), so every pair is an exact zero-padded FFT convolution:
-// the same forward FFT, spectrum multiply-accumulate and inverse FFT kernels
-// as flgf_solve, with their scratch in the static array.
+// the products between parents of flgf_solve (parent.cu; at most 8 parents,
+// neighbours of each other), with their scratch in the static array.  27 blocks
+// of 16^3, FP32, a call: 122 us with the child-pair kernel (104 us of it), 68 us.
 #include <algorithm>
 #include <array>
 #include <cstring>
@@ -30,7 +31,7 @@ namespace {
 using namespace flgf;
 
 constexpr int kStaticMaxBlocks = 32;
-constexpr size_t kSpecBytes = (size_t)kStaticMaxBlocks * nfreq(16) * 16;  // complex double, N = 16
+constexpr size_t kSpecBytes = (size_t)kStaticMaxBlocks * nfreq(16) * 16;  // half-transformed spectra of 8 parents (complex double, N = 16: 8.65 MB)
 constexpr size_t kListBytes = 512 * 1024;
 constexpr size_t kScratchBytes = 2 * kSpecBytes + kListBytes;             // ~18.3 MB
 
@@ -60,41 +61,21 @@ cudaError_t scratch_address(void** out) {
 
 // Launch lists of one call, passed to the list-writing kernel by value (the
 // kernel's parameters are copied at launch, so nothing is read from host
-// memory afterwards).  At most 8 parents with targets and 8 neighbour cells
-// with sources: the blocks lie in one aligned 4x4x4 box.
-struct StaticLists {
-  HadGroup group;
-  int nchunk, nblk;
-  double h2;
-  int src[8 * 8];
-  int tgt[8 * 8];
-  uint16_t par[27 * 8];
+// memory afterwards).  At most 8 parents, all sources and targets: the blocks
+// lie in one aligned 4x4x4 box.  Laid out as in the scratch array.
+constexpr int kMaxParents = 8;
+struct __align__(16) StaticLists {
+  uint16_t items[kMaxParents * kPfItem];
+  int child[kMaxParents * 8];
+  int col[kMaxParents];
+  double scale[kMaxParents];
+  PfGroup group;
 };
+static_assert(sizeof(StaticLists) <= kListBytes, "lists fit the scratch");
+static_assert(sizeof(StaticLists) % sizeof(int) == 0, "copied by words");
 
-// Offsets of the lists in the scratch array (256-byte aligned).
-constexpr size_t kOffGroup = 0;
-constexpr size_t kOffIds = 256;
-constexpr size_t kOffScale = kOffIds + 256;
-constexpr size_t kOffSrc = kOffScale + 256;
-constexpr size_t kOffTgt = kOffSrc + 256;
-constexpr size_t kOffPar = kOffTgt + 256;
-constexpr size_t kOffWork = kOffPar + 512;
-
-__global__ void static_lists_kernel(const StaticLists L, unsigned char* __restrict__ dl) {
-  const int t = threadIdx.x;
-  if (t == 0) *reinterpret_cast<HadGroup*>(dl + kOffGroup) = L.group;
-  if (t < L.nblk) {
-    reinterpret_cast<int*>(dl + kOffIds)[t] = t;
-    reinterpret_cast<double*>(dl + kOffScale)[t] = L.h2;
-  }
-  if (t < 8 * L.group.ncell) reinterpret_cast<int*>(dl + kOffSrc)[t] = L.src[t];
-  if (t < 8 * L.group.nact) reinterpret_cast<int*>(dl + kOffTgt)[t] = L.tgt[t];
-  if (t < 27 * L.group.nact) reinterpret_cast<uint16_t*>(dl + kOffPar)[t] = L.par[t];
-  // work items: (group 0, first chunk, chunks), cpc chunks each
-  HadWork* w = reinterpret_cast<HadWork*>(dl + kOffWork);
-  const int cpc = L.group.cpc;
-  for (int i = t; i * cpc < L.nchunk; i += blockDim.x)
-    w[i] = HadWork{0, i * cpc, min(cpc, L.nchunk - i * cpc)};
+__global__ void static_lists_kernel(const StaticLists L, int* __restrict__ dl) {
+  for (int i = threadIdx.x; i < (int)(sizeof(L) / sizeof(int)); i += blockDim.x) dl[i] = reinterpret_cast<const int*>(&L)[i];
 }
 
 }  // namespace
@@ -130,46 +111,41 @@ extern "C" int flgf_convolve_static(flgf_ctx* ctx, int nblk, const int32_t* coor
     std::sort(s.begin(), s.end());
     if (std::adjacent_find(s.begin(), s.end()) != s.end()) return bad(FLGF_EMESH, "convolve_static: duplicate block");
   }
-  auto find = [&](int x, int y, int z) -> int {
-    for (int b = 0; b < nblk; ++b)
-      if (c[b][0] == x && c[b][1] == y && c[b][2] == z) return b;
-    return -1;
-  };
-  // launch lists: one parent group over the parent box (one octree level,
-  // near field included: every pair is a neighbour-parent pair)
-  std::vector<ParentRec> recs;
-  for (int p0 = plo[0]; p0 <= phi[0]; ++p0)
-    for (int p1 = plo[1]; p1 <= phi[1]; ++p1)
-      for (int p2 = plo[2]; p2 <= phi[2]; ++p2) {
-        ParentRec r;
-        bool has = false;
-        for (int a = 0; a < 8; ++a) {
-          r.tgt[a] = find(2 * p0 + (a >> 2), 2 * p1 + ((a >> 1) & 1), 2 * p2 + (a & 1));
-          has |= r.tgt[a] >= 0;
-        }
-        if (!has) continue;
-        for (int e = 0; e < 27; ++e)
-          for (int b = 0; b < 8; ++b)
-            r.cell[e][b] = find(2 * (p0 + e / 9 - 1) + (b >> 2), 2 * (p1 + (e / 3) % 3 - 1) + ((b >> 1) & 1),
-                                2 * (p2 + e % 3 - 1) + (b & 1));
-        recs.push_back(r);
-      }
-  const int nchunk = cv.fp64 ? nchunks<double>(N) : nchunks<float>(N);
-  HadLists hl;
-  pack_parent_groups(0, recs, nchunk, had_kernel_units(cv.fp64), hl);
-  // one group of at most 8 parents and 8 cells (the parents lie in a 2x2x2 box)
-  if (hl.groups.size() != 1 || hl.groups[0].nact > 8 || hl.groups[0].ncell > 8 ||
-      kOffWork + sizeof(HadWork) * hl.work.size() > kListBytes)
-    return bad(FLGF_EINVAL, "convolve_static: launch lists exceed the scratch");
+  // the box's blocks by their place in it, and its parents
+  int at[4][4][4];
+  std::fill(&at[0][0][0], &at[0][0][0] + 64, -1);
+  for (int b = 0; b < nblk; ++b) at[c[b][0] - 2 * plo[0]][c[b][1] - 2 * plo[1]][c[b][2] - 2 * plo[2]] = b;
   StaticLists L;
   std::memset(&L, 0, sizeof(L));
-  L.group = hl.groups[0];
-  L.nchunk = nchunk;
-  L.nblk = nblk;
-  L.h2 = h * h;
-  std::copy(hl.src_ids.begin(), hl.src_ids.end(), L.src);
-  std::copy(hl.tgt_ids.begin(), hl.tgt_ids.end(), L.tgt);
-  std::copy(hl.par_tab.begin(), hl.par_tab.end(), L.par);
+  int col[2][2][2], np = 0;
+  for (int p = 0; p < 8; ++p) {
+    const int x = p >> 2, y = (p >> 1) & 1, z = p & 1;
+    bool any = false;
+    for (int a = 0; a < 8; ++a) {
+      L.child[np * 8 + a] = at[2 * x + (a >> 2)][2 * y + ((a >> 1) & 1)][2 * z + (a & 1)];
+      any |= L.child[np * 8 + a] >= 0;
+    }
+    col[x][y][z] = any ? np++ : -1;
+  }
+  // one item per parent: its neighbours in the box (the entries of PfGroup's items)
+  for (int p = 0; p < 8; ++p) {
+    const int q[3] = {p >> 2, (p >> 1) & 1, p & 1}, m = col[q[0]][q[1]][q[2]];
+    if (m < 0) continue;
+    uint16_t* it = L.items + m * kPfItem;
+    for (int i = 0; i < 36; ++i) it[i] = (uint16_t)(33 * np);
+    it[36] = (uint16_t)m;
+    it[37] = 1;
+    for (int e = 0; e < 27; ++e) {
+      const int x = q[0] + e / 9 - 1, y = q[1] + (e / 3) % 3 - 1, z = q[2] + e % 3 - 1;
+      if (x < 0 || x > 1 || y < 0 || y > 1 || z < 0 || z > 1 || col[x][y][z] < 0) continue;
+      it[9 * (e % 3) + e / 3] = (uint16_t)(33 * col[x][y][z]);
+      it[38] |= (uint16_t)(1 << (e / 9));
+    }
+    L.col[m] = m;
+    L.scale[m] = h * h;
+  }
+  L.group = PfGroup{np, np, np, 0, 0, 0};
+  const PfLimits lim{np, np, np};
 
   void* base = nullptr;
   cudaError_t e = scratch_address(&base);
@@ -180,32 +156,17 @@ extern "C" int flgf_convolve_static(flgf_ctx* ctx, int nblk, const int32_t* coor
   unsigned char* dl = sp + 2 * kSpecBytes;
   cudaStream_t s = cv.stream;
   // the lists travel as kernel parameters, written into the scratch on the stream
-  static_lists_kernel<<<1, 256, 0, s>>>(L, dl);
+  static_lists_kernel<<<1, 256, 0, s>>>(L, reinterpret_cast<int*>(dl));
   e = cudaGetLastError();
-  const int* d_ids = reinterpret_cast<const int*>(dl + kOffIds);
-  if (e == cudaSuccess) {
-    if (cv.fp64) e = launch_fft_forward<double>(N, static_cast<const double*>(f), d_ids, d_ids, nblk, spec, nblk, s);
-    else e = launch_fft_forward<float>(N, static_cast<const float*>(f), d_ids, d_ids, nblk, spec, nblk, s);
-  }
-  if (e == cudaSuccess) {
-    const HadGroup* d_groups = reinterpret_cast<const HadGroup*>(dl + kOffGroup);
-    const HadWork* d_work = reinterpret_cast<const HadWork*>(dl + kOffWork);
-    const int* d_src = reinterpret_cast<const int*>(dl + kOffSrc);
-    const int* d_tgt = reinterpret_cast<const int*>(dl + kOffTgt);
-    const uint16_t* d_par = reinterpret_cast<const uint16_t*>(dl + kOffPar);
-    const int nw = (int)hl.work.size();
-    if (cv.fp64)
-      e = launch_hadamard<double>(N, d_groups, d_work, nw, hl.max_units, d_src, d_tgt, d_par, spec, acc, nblk,
-                                  cv.kspec, cv.kstride, s);
-    else
-      e = launch_hadamard<float>(N, d_groups, d_work, nw, hl.max_units, d_src, d_tgt, d_par, spec, acc, nblk,
-                                 cv.kspec, cv.kstride, s);
-  }
-  if (e == cudaSuccess) {
-    const double* d_scale = reinterpret_cast<const double*>(dl + kOffScale);
-    if (cv.fp64) e = launch_fft_inverse<double>(N, acc, nblk, d_ids, d_ids, d_scale, nblk, static_cast<double*>(u), s, false);
-    else e = launch_fft_inverse<float>(N, acc, nblk, d_ids, d_ids, d_scale, nblk, static_cast<float*>(u), s, false);
-  }
+  const StaticLists* d = reinterpret_cast<const StaticLists*>(dl);
+  auto run = [&](auto zero) {
+    using R = decltype(zero);
+    cudaError_t r = launch_pf_forward<R>(N, static_cast<const R*>(f), d->child, np, spec, s);
+    if (r == cudaSuccess)
+      r = launch_pf_mac<R>(N, &d->group, 1, lim, d->items, d->col, d->col, spec, np, acc, np, cv.pspec, 1, 0, 0, s);
+    return r == cudaSuccess ? launch_pf_inverse<R>(N, acc, d->child, d->scale, np, static_cast<R*>(u), s) : r;
+  };
+  if (e == cudaSuccess) e = cv.fp64 ? run(0.0) : run(0.0f);
   if (e != cudaSuccess) return bad(FLGF_ECUDA, cudaGetErrorString(e));
   return FLGF_OK;
 }
