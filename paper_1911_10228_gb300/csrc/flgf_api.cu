@@ -226,6 +226,8 @@ struct flgf_blockset {
   void* lap_in = nullptr;
   void* lap_out = nullptr;
   int* d_err = nullptr;
+  int* h_err = nullptr;       // pinned: where the device flag is read to
+  bool err_known = false;     // *h_err is the flag of the last solve (forward or adjoint)
   // host source loads run on their own stream: they wait only until the
   // solve in flight has copied the source buffer (ev_fuser_free), so they
   // overlap the rest of that solve; the next solve waits for ev_loaded
@@ -460,6 +462,7 @@ extern "C" void flgf_blockset_destroy(flgf_blockset* bs) {
   cudaFree(bs->lap_in);
   cudaFree(bs->lap_out);
   cudaFree(bs->d_err);
+  if (bs->h_err) cudaFreeHost(bs->h_err);
   if (bs->ev_fuser_free) cudaEventDestroy(bs->ev_fuser_free);
   if (bs->ev_loaded) cudaEventDestroy(bs->ev_loaded);
   if (bs->ev_dev_load) cudaEventDestroy(bs->ev_dev_load);
@@ -1319,6 +1322,7 @@ static int blockset_create(flgf_ctx* ctx, int n_problems, const int* n_levels, c
   if (e == cudaSuccess) e = cudaMemset(bs->fuser, 0, rs * N3 * bs->B);
   if (e == cudaSuccess) e = cudaMemset(bs->unodes, 0, rs * N3 * bs->G);
   if (e == cudaSuccess) e = cudaMemset(bs->d_err, 0, sizeof(int));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&bs->h_err, sizeof(int));
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&bs->cstream, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bs->ev_fuser_free, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&bs->ev_loaded, cudaEventDisableTiming);
@@ -1897,6 +1901,7 @@ extern "C" int flgf_solve(flgf_blockset* bs) {
   flgf_ctx* ctx = bs->ctx;
   collect_times(bs);
   cudaError_t e;
+  bs->err_known = false;
   if (bs->load_pending) {  // a host load on the copy stream feeds this solve
     CK(cudaStreamWaitEvent(ctx->stream, bs->ev_loaded, 0));
     bs->load_pending = false;
@@ -1946,10 +1951,11 @@ namespace {
 // kernels of the last solve (forward or adjoint) raise on a missing halo block.
 int check_device_flag(flgf_blockset* bs, const char* what) {
   flgf_ctx* ctx = bs->ctx;
+  // one round trip: the flag is read behind the caller's copy, once per solve
+  if (!bs->err_known) CK(cudaMemcpyAsync(bs->h_err, bs->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
-  int herr = 0;
-  CK(cudaMemcpy(&herr, bs->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (herr) return fail(ctx, FLGF_EDEVICE, std::string(what) + ": a coarse-fine interpolation met a missing halo block");
+  bs->err_known = true;
+  if (*bs->h_err) return fail(ctx, FLGF_EDEVICE, std::string(what) + ": a coarse-fine interpolation met a missing halo block");
   return FLGF_OK;
 }
 }  // namespace
@@ -1978,6 +1984,7 @@ extern "C" int flgf_solve_adjoint(flgf_blockset* bs) {
   }
   collect_times(bs);
   bs->ev_used = 0;
+  bs->err_known = false;
   cudaError_t e = ctx->prec == FLGF_FP64 ? enqueue_adjoint<double>(bs) : enqueue_adjoint<float>(bs);
   if (e != cudaSuccess) return fail(ctx, FLGF_ECUDA, std::string("solve_adjoint: ") + cudaGetErrorString(e));
   bs->ev_pending = bs->timing && bs->ev_used > 0;

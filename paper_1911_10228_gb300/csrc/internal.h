@@ -228,20 +228,21 @@ constexpr int pf_max_parents(bool fp64) { return fp64 ? 64 : 128; }
 struct PfLimits {  // the largest group of a launch
   int cells = 0, parents = 0, items = 0;
 };
-// Shared memory of the product kernel: lines of the cells (and a zero one) and
-// of the parents (FP64: per parity); for FP64 the sums of the cells' real and
-// imaginary parts; then the items and columns.
+// Shared memory of the product kernel with upc units a CTA: per unit the lines
+// of the cells (and a zero one) and of the parents (FP64: per parity), for FP64
+// also the sums of the cells' real and imaginary parts; then the items and
+// columns.
 template <typename R>
-constexpr size_t pf_sum_offset(const PfLimits& l) {
-  return (size_t)(l.cells + 1 + (sizeof(R) == 8 ? 2 : 1) * l.parents) * 33 * 2 * sizeof(R);
+constexpr size_t pf_sum_offset(const PfLimits& l, int upc) {
+  return (size_t)upc * (l.cells + 1 + (sizeof(R) == 8 ? 2 : 1) * l.parents) * 33 * 2 * sizeof(R);
 }
 template <typename R>
-constexpr size_t pf_table_offset(const PfLimits& l) {
-  return (pf_sum_offset<R>(l) + (sizeof(R) == 8 ? (size_t)(l.cells + 1) * 33 * 8 : 0) + 15) / 16 * 16;
+constexpr size_t pf_table_offset(const PfLimits& l, int upc) {
+  return (pf_sum_offset<R>(l, upc) + (sizeof(R) == 8 ? (size_t)upc * (l.cells + 1) * 33 * 8 : 0) + 15) / 16 * 16;
 }
 template <typename R>
-constexpr size_t pf_smem_bytes(const PfLimits& l) {
-  return pf_table_offset<R>(l) + (size_t)l.items * kPfItem * 2 + (size_t)(l.cells + l.parents) * 4;
+constexpr size_t pf_smem_bytes(const PfLimits& l, int upc) {
+  return pf_table_offset<R>(l, upc) + (size_t)l.items * kPfItem * 2 + (size_t)(l.cells + l.parents) * 4;
 }
 size_t pf_parent_values(int N);  // complex values of one parent's half-transformed spectrum
 size_t pf_kernel_values(int N);  // complex values of the 27 parent kernel spectra

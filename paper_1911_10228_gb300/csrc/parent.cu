@@ -257,8 +257,8 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 
 // ---------------------------------------------------------------------------
 // Axis 0 and the products.  A CTA takes a group of target parents (consecutive
-// in tile order, so they share neighbour cells) and a unit of lines; lane =
-// (line, k0).  Per parity of k0 the group's source lines are copied to shared
+// in tile order, so they share neighbour cells) and upc units of lines (one,
+// unless the groups are small: mac_units); lane = (line, k0).  Per parity of k0 the group's source lines are copied to shared
 // memory and transformed in place (a thread per line); a warp then takes two
 // parents that are neighbours along axis 2 (or one) at a time, its lane's 27
 // kernel values in registers: the pair's 36 distinct source values feed 54
@@ -270,33 +270,41 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 // fi, (ki - kr) fr) with fr + fi kept beside the sources, and skip absent cells
 // one by one: the FP64 pipe is the bound.
 // ---------------------------------------------------------------------------
-template <typename R, int N>
+// kOne: one unit a CTA (known at compile time: 703 us against 735 for 16^3
+// blocks of 16^3, FP32).
+template <typename R, int N, bool kOne>
 __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
     pf_mac_kernel(const PfGroup* __restrict__ groups, int ngroups, const PfLimits lim,
                   const uint16_t* __restrict__ items, const int* __restrict__ cell_col, const int* __restrict__ tgt_col,
                   const typename Vec2<R>::type* __restrict__ src, int nsrc, typename Vec2<R>::type* __restrict__ dst,
-                  int ndst, const typename Vec2<R>::type* __restrict__ kspec, int src_stride, int dst_stride) {
+                  int ndst, const typename Vec2<R>::type* __restrict__ kspec, int src_stride, int dst_stride, int units) {
   using D = PfDims<N>;
   using C2 = typename Vec2<R>::type;
   constexpr int H = D::H, TW = 64 / D::P;
   constexpr bool G3 = sizeof(R) == 8;
-  constexpr int NW = kPfMacThreads / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int g = blockIdx.x % ngroups, unit = blockIdx.x / ngroups;
+  const int upc = kOne ? 1 : units, NW = kPfMacThreads / 32 / upc;  // warps per unit
+  const int g = blockIdx.x % ngroups, sub = kOne ? 0 : threadIdx.x / 32 / NW, unit = blockIdx.x / ngroups * upc + sub;
   const PfGroup gp = groups[g];
   const int nc = gp.ncell, nt = gp.nact;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  C2* X = reinterpret_cast<C2*>(smem_raw);                      // [cells + 1][33], line nc is zero
-  C2* T = X + (size_t)(lim.cells + 1) * kPfStride;              // [FP64: 2][parents][33]
-  R* Sm = reinterpret_cast<R*>(smem_raw + pf_sum_offset<R>(lim));  // FP64: fr + fi, [cells + 1][33]
-  uint4* IT = reinterpret_cast<uint4*>(smem_raw + pf_table_offset<R>(lim));  // [items][5]
+  const int tid = threadIdx.x, lane = tid & 31, warp = (tid >> 5) % NW;
+  // per unit: the cells' lines (line nc is zero) and the parents' (FP64: of both parities); FP64: fr + fi
+  constexpr int kT = G3 ? 2 : 1;
+  const int xs = (lim.cells + 1) * kPfStride, ts = kT * lim.parents * kPfStride;
+  C2* const X0 = reinterpret_cast<C2*>(smem_raw);                   // [upc][cells + 1][33]
+  C2* const T0 = X0 + (size_t)upc * xs;                             // [upc][kT][parents][33]
+  R* const S0 = reinterpret_cast<R*>(smem_raw + pf_sum_offset<R>(lim, upc));  // [upc][cells + 1][33]
+  C2* const X = X0 + sub * xs;
+  C2* const T = T0 + sub * ts;
+  R* const Sm = S0 + (G3 ? sub * xs : 0);
+  uint4* IT = reinterpret_cast<uint4*>(smem_raw + pf_table_offset<R>(lim, upc));  // [items][5]
   int* CC = reinterpret_cast<int*>(IT + (size_t)lim.items * (kPfItem / 8));
   int* TC = CC + lim.cells;
 
   for (int i = tid; i < nc; i += kPfMacThreads) CC[i] = __ldg(cell_col + gp.cell_off + i) + (int)blockIdx.y * src_stride;
-  if (tid < 32) {
-    X[(size_t)nc * kPfStride + tid] = C2{R(0), R(0)};
-    if constexpr (G3) Sm[(size_t)nc * kPfStride + tid] = R(0);
+  if (warp == 0) {
+    X[(size_t)nc * kPfStride + lane] = C2{R(0), R(0)};
+    if constexpr (G3) Sm[(size_t)nc * kPfStride + lane] = R(0);
   }
   __syncthreads();
   const C2* sbase = src + (size_t)unit * nsrc * 32 + lane;
@@ -313,10 +321,9 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
   // the second adding to the first, which leaves room for larger groups
   constexpr bool kBoth = G3;
   auto inverse = [&](int last) {
-    for (int i = tid; i < (kBoth ? 2 : 1) * nt * D::S; i += kPfMacThreads) {
-      const int par = kBoth ? i / (nt * D::S) : last, r = kBoth ? i % (nt * D::S) : i;
-      const int m = D::S == 1 ? r : r % nt;
-      C2* line = T + ((kBoth ? (size_t)par * lim.parents : 0) + m) * kPfStride + (D::S == 1 ? 0 : (r / nt) * H);
+    for (int i = tid; i < upc * kT * nt * D::S; i += kPfMacThreads) {
+      const int j = kOne && kT * D::S == 1 ? 0 : i / nt, m = i - j * nt, par = kBoth ? j / D::S % 2 : last;  // j: (unit, parity, line of the unit)
+      C2* line = T0 + (j / D::S / kT) * ts + ((kBoth ? par * lim.parents : 0) + m) * kPfStride + (j % D::S) * H;
       R xr[H], xi[H];
 #pragma unroll
       for (int k = 0; k < H; ++k) { const C2 v = line[k]; xr[k] = v.x; xi[k] = v.y; }
@@ -332,9 +339,9 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
   for (int par = 0; par < 2; ++par) {
     cp_async_wait();
     __syncthreads();
-    for (int i = tid; i < nc * D::S; i += kPfMacThreads) {
-      const int c = D::S == 1 ? i : i % nc;
-      C2* line = X + c * kPfStride + (D::S == 1 ? 0 : (i / nc) * H);
+    for (int i = tid; i < upc * nc * D::S; i += kPfMacThreads) {
+      const int j = kOne && D::S == 1 ? 0 : i / nc, c = i - j * nc;
+      C2* line = X0 + (j / D::S) * xs + c * kPfStride + (j % D::S) * H;
       R xr[H], xi[H];
 #pragma unroll
       for (int z = 0; z < H; ++z) { const C2 v = line[z]; xr[z] = v.x; xi[z] = v.y; }
@@ -345,7 +352,7 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll
       for (int k = 0; k < H; ++k) line[k] = C2{xr[k], xi[k]};
       if constexpr (G3) {
-        R* sl = Sm + (line - X);
+        R* sl = S0 + (line - X0);
 #pragma unroll
         for (int k = 0; k < H; ++k) sl[k] = xr[k] + xi[k];
       }
@@ -557,18 +564,32 @@ static cudaError_t inverse_n(const void* in, const int* tgt_ch, const double* sc
                                                         unodes);
   return cudaGetLastError();
 }
+// Units per CTA of the product kernel: small groups leave most threads without
+// a line to transform, so up to 8 units share a CTA while every line has a
+// thread, the shared memory stays below half an SM's, and every SM gets a CTA.
 template <typename R, int N>
-static cudaError_t mac_n(const PfGroup* groups, int ngroups, const PfLimits& lim, const uint16_t* items, const int* cell_col, const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
+static int mac_units(int ngroups, int ncomp, const PfLimits& lim) {
+  int upc = 1;
+  while (upc < 8 && 2 * upc * lim.cells * PfDims<N>::S <= kPfMacThreads && pf_smem_bytes<R>(lim, 2 * upc) <= 100 * 1024 &&
+         (long long)PfDims<N>::U / (2 * upc) * ngroups * ncomp >= 152)
+    upc *= 2;
+  return upc;
+}
+template <typename R, int N>
+static cudaError_t mac_n(const PfGroup* groups, int ngroups, const PfLimits& lim, const uint16_t* items, const int* cell_col,
+                         const int* tgt_col, const void* src, int nsrc, void* dst, int ndst,
                          const void* kspec, int ncomp, int src_stride, int dst_stride, cudaStream_t s) {
   using C2 = typename Vec2<R>::type;
-  const size_t sm = pf_smem_bytes<R>(lim);
+  static_assert(PfDims<N>::U % 8 == 0, "whole CTAs of 8 units");
+  const int upc = mac_units<R, N>(ngroups, ncomp, lim);
+  const size_t sm = pf_smem_bytes<R>(lim, upc);
   if (sm > kFlSmemBytes || (size_t)PfDims<N>::U * ngroups >= (1u << 31)) return cudaErrorInvalidConfiguration;
-  auto k = pf_mac_kernel<R, N>;
+  auto k = upc == 1 ? pf_mac_kernel<R, N, true> : pf_mac_kernel<R, N, false>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k<<<dim3((unsigned)(PfDims<N>::U * ngroups), ncomp), kPfMacThreads, sm, s>>>(
+  k<<<dim3((unsigned)(PfDims<N>::U / upc * ngroups), ncomp), kPfMacThreads, sm, s>>>(
       groups, ngroups, lim, items, cell_col, tgt_col, reinterpret_cast<const C2*>(src), nsrc, reinterpret_cast<C2*>(dst),
-      ndst, reinterpret_cast<const C2*>(kspec), src_stride, dst_stride);
+      ndst, reinterpret_cast<const C2*>(kspec), src_stride, dst_stride, upc);
   return cudaGetLastError();
 }
 
