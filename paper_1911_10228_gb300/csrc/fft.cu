@@ -265,14 +265,17 @@ __global__ void __launch_bounds__(N * N) fft_fwd_kernel(const R* __restrict__ no
 // ---------------------------------------------------------------------------
 // Inverse transform of accumulated spectra; keeps the first N^3 outputs.
 // ---------------------------------------------------------------------------
+// Blocks from index `assign` on add to what stands in the output (FP64: the
+// parents' part of a coarser octree level's target).
 // TH threads per block.  With N (N + 1) threads the 2N (N + 1) lines of the
 // first axis take exactly two rounds and the N (N + 1) of the second one (N^2
 // threads leave the last round of each nearly empty).
 template <typename R, int N, typename C, int TH>
 __global__ void __launch_bounds__(TH) fft_inv_kernel(const cplx<R>* __restrict__ acc, int spec_blocks,
                                                         const int* __restrict__ sids, const int* __restrict__ gids,
-                                                        const double* __restrict__ scales, R* __restrict__ out) {
+                                                        const double* __restrict__ scales, int assign, R* __restrict__ out) {
   constexpr int P = 2 * N, NX = N + 1;
+  constexpr bool kAdd = sizeof(R) == 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<C>* buf = reinterpret_cast<cplx<C>*>(smem_raw);  // [N z][P y][NX kx]
   const int sid = sids[blockIdx.x], gid = gids[blockIdx.x];
@@ -329,6 +332,11 @@ __global__ void __launch_bounds__(TH) fft_inv_kernel(const cplx<R>* __restrict__
       R* r = reinterpret_cast<R*>(&v);
 #pragma unroll
       for (int j = 0; j < V; ++j) r[j] = Arith<C>::template to<R>(scale * xr[u * V + j]);
+      if (kAdd && (int)blockIdx.x >= assign) {
+        const int4 w = orow[u];
+#pragma unroll
+        for (int j = 0; j < V; ++j) r[j] += reinterpret_cast<const R*>(&w)[j];
+      }
       orow[u] = v;
     }
   }
@@ -555,7 +563,8 @@ constexpr int kInv2Threads = 512;
 
 template <typename R, typename C>
 static cudaError_t launch_inv(int N, const cplx<R>* ac, int spec_blocks, const int* sids, const int* gids,
-                              const double* scales, int count, R* out, cudaStream_t s) {
+                              const double* scales, int count, int n_add, R* out, cudaStream_t s) {
+  if (n_add > 0 && sizeof(R) != 8) return cudaErrorInvalidValue;
   if (N == 16) {
     const size_t sm = sizeof(cplx<C>) * 16 * 32 * 17;
     if constexpr (std::is_same<C, ff>::value) {
@@ -567,12 +576,12 @@ static cudaError_t launch_inv(int N, const cplx<R>* ac, int spec_blocks, const i
       constexpr int TH = inv_threads<C, 16>();
       cudaError_t e = set_smem(fft_inv_kernel<R, 16, C, TH>, sm);
       if (e != cudaSuccess) return e;
-      fft_inv_kernel<R, 16, C, TH><<<count, TH, sm, s>>>(ac, spec_blocks, sids, gids, scales, out);
+      fft_inv_kernel<R, 16, C, TH><<<count, TH, sm, s>>>(ac, spec_blocks, sids, gids, scales, count - n_add, out);
     }
   } else if (N == 8) {
     const size_t sm = sizeof(cplx<C>) * 8 * 16 * 9;
     constexpr int TH = inv_threads<C, 8>();
-    fft_inv_kernel<R, 8, C, TH><<<count, TH, sm, s>>>(ac, spec_blocks, sids, gids, scales, out);
+    fft_inv_kernel<R, 8, C, TH><<<count, TH, sm, s>>>(ac, spec_blocks, sids, gids, scales, count - n_add, out);
   } else {
     return cudaErrorInvalidValue;
   }
@@ -588,13 +597,13 @@ cudaError_t launch_fft_forward(int N, const R* nodes, const int* gids, const int
 
 template <typename R>
 cudaError_t launch_fft_inverse(int N, const void* acc, int spec_blocks, const int* sids, const int* gids,
-                               const double* scales, int count, R* out, cudaStream_t s, bool compensated) {
+                               const double* scales, int count, int n_add, R* out, cudaStream_t s, bool compensated) {
   if (count <= 0) return cudaSuccess;
   const cplx<R>* ac = reinterpret_cast<const cplx<R>*>(acc);
   if constexpr (sizeof(R) == 4) {
-    if (compensated) return launch_inv<R, ff>(N, ac, spec_blocks, sids, gids, scales, count, out, s);
+    if (compensated) return launch_inv<R, ff>(N, ac, spec_blocks, sids, gids, scales, count, n_add, out, s);
   }
-  return launch_inv<R, R>(N, ac, spec_blocks, sids, gids, scales, count, out, s);
+  return launch_inv<R, R>(N, ac, spec_blocks, sids, gids, scales, count, n_add, out, s);
 }
 
 template <typename R>
@@ -624,9 +633,9 @@ cudaError_t launch_kernel_spectra(int N, const double* karr, void* kspec_level, 
 template cudaError_t launch_fft_forward<float>(int, const float*, const int*, const int*, int, void*, int, cudaStream_t);
 template cudaError_t launch_fft_forward<double>(int, const double*, const int*, const int*, int, void*, int,
                                                 cudaStream_t);
-template cudaError_t launch_fft_inverse<float>(int, const void*, int, const int*, const int*, const double*, int, float*,
+template cudaError_t launch_fft_inverse<float>(int, const void*, int, const int*, const int*, const double*, int, int, float*,
                                                cudaStream_t, bool);
-template cudaError_t launch_fft_inverse<double>(int, const void*, int, const int*, const int*, const double*, int,
+template cudaError_t launch_fft_inverse<double>(int, const void*, int, const int*, const int*, const double*, int, int,
                                                 double*, cudaStream_t, bool);
 template cudaError_t launch_kernel_spectra<float>(int, const double*, void*, double*, int, cudaStream_t);
 template cudaError_t launch_kernel_spectra<double>(int, const double*, void*, double*, int, cudaStream_t);

@@ -35,12 +35,16 @@ struct flgf_ctx {
   double* d_J1 = nullptr;
   void* d_kspec = nullptr;
   size_t kstride = 0;  // complex elements per octree level
-  void* d_pspec = nullptr;  // the 27 parent kernel spectra of the finest octree level (parent.cu)
+  void* d_pspec = nullptr;  // the 27 parent kernel spectra (parent.cu) of every level that runs between parents
   std::vector<double> J1;
   MgScratch mg_scratch;  // flgf_refine_level
   // whether dense tiles of the finest octree level run between parents (all
   // but the FP32 parent-group form, FLGF_CTX_MAC = 0)
   bool parent_form() const { return prec == FLGF_FP64 || mac >= 1; }
+  // whether the coarser levels' do too, their near pairs taken out block by
+  // block: FP64 (the FP32 child-pair kernels stay: their spectra go through the
+  // float-float inverse transforms of FLGF_OPT_COMPENSATED)
+  bool parent_form_coarse() const { return prec == FLGF_FP64; }
 };
 
 namespace {
@@ -161,19 +165,20 @@ struct PhaseOff {  // arena offsets and counts of one phase's launch lists
   int n_fwd = 0; size_t fwd_gid = 0, fwd_sid = 0;
   int n_groups_dense = 0, n_work = 0, max_units = 0;
   size_t hgroups = 0, work = 0, src_ids = 0, tgt_ids = 0, par_tab = 0;
-  int n_groups = 0, max_group_src = 0; size_t groups = 0, l_tgt = 0, l_len = 0, l_ent = 0, l_src = 0;
+  int n_groups = 0, n_groups_out = 0, max_group_src = 0; size_t groups = 0, l_tgt = 0, l_len = 0, l_ent = 0, l_src = 0;
   int n_fl = 0, fl_max_cells = 0, fl_max_parents = 0;
   size_t fl_groups = 0, fl_rows = 0, fl_dlms = 0, fl_tgt = 0, fl_cells = 0;
   int fl_ncomp = 1, fl_cstride = 0;  // components sharing the frequency-lane groups, their column stride
   bool fl_split = false;              // rows nearly all full: the two-path product form
-  // the finest octree level between parents (parent.cu): the first n_pf
+  // the octree levels between parents (parent.cu): the first n_pf
   // frequency-lane groups, their items and column tables, and the children of
   // the source and target parents (one component's; the others follow in order)
   int n_pf = 0, n_pfs = 0, n_pft = 0, pf_src_stride = 0, pf_tgt_stride = 0;
   PfLimits pf_lim;
   size_t pf_groups = 0, pf_items = 0, pf_ccol = 0, pf_tcol = 0, pf_sch = 0, pf_tch = 0, pf_scale = 0;
   int n_fll = 0; size_t fll_groups = 0, fll_tgt = 0, fll_beg = 0, fll_len = 0, fll_ent = 0;
-  int n_inv = 0, n_inv0 = 0; size_t inv_sid = 0, inv_gid = 0, inv_scale = 0;  // finest octree level first (n_inv0)
+  // finest octree level first (n_inv0); the last n_inv_add add to what the parents' inverse wrote
+  int n_inv = 0, n_inv0 = 0, n_inv_add = 0; size_t inv_sid = 0, inv_gid = 0, inv_scale = 0;
   std::vector<int> n_itp; std::vector<size_t> itp_ch, itp_par, itp_cpos;
   int n_sel = 0; size_t sel_src = 0, sel_dst = 0;
   int n_selw = 0; size_t selw_src = 0, selw_dst = 0;
@@ -327,20 +332,25 @@ extern "C" int flgf_create(flgf_ctx** out, const flgf_opts* o) {
   const size_t csz = ctx->prec == FLGF_FP64 ? 16 : 8;
   ctx->kstride = (size_t)kNOff * NW;
   STEP(cudaMalloc(&ctx->d_kspec, csz * ctx->kstride * ctx->max_oct));
-  STEP(cudaMalloc(&ctx->d_pspec, csz * pf_kernel_values(N)));
-  STEP(cudaMalloc(&karr, sizeof(double) * (size_t)kNOff * P * P * P));  // also the 27 parent arrays of 8 P^3
+  const int npl = ctx->parent_form_coarse() ? ctx->max_oct : 1;
+  STEP(cudaMalloc(&ctx->d_pspec, csz * pf_kernel_values(N) * npl));
+  STEP(cudaMalloc(&karr, sizeof(double) * (size_t)kNOff * P * P * P));  // also 8 parent arrays of 8 P^3
   STEP(cudaMalloc(&tmp, std::max<size_t>(2 * 16 * (size_t)kNOff * NW, pf_setup_bytes(N))));
-  STEP(launch_parent_kernel_arrays(ctx->d_table, R, (double)R, (double)ctx->RA, N, karr, ctx->stream));
-  if (ctx->prec == FLGF_FP64) {
-    STEP(launch_pf_setup<double>(N, karr, tmp, ctx->d_pspec, ctx->stream));
-  } else {
-    STEP(launch_pf_setup<float>(N, karr, tmp, ctx->d_pspec, ctx->stream));
+  for (int k = 0; k < npl; ++k) {
+    STEP(launch_parent_kernel_arrays(ctx->d_table, R, (double)R, (double)ctx->RA, N, k, karr, ctx->stream));
+    void* lvl = (char*)ctx->d_pspec + csz * pf_kernel_values(N) * k;
+    if (ctx->prec == FLGF_FP64) {
+      STEP(launch_pf_setup<double>(N, karr, tmp, lvl, ctx->stream));
+    } else {
+      STEP(launch_pf_setup<float>(N, karr, tmp, lvl, ctx->stream));
+    }
   }
   for (int k = 0; k < ctx->max_oct; ++k) {
-    STEP(launch_kernel_arrays(ctx->d_table, R, (double)R, (double)ctx->RA, N, k, karr, ctx->stream));
+    STEP(launch_kernel_arrays(ctx->d_table, R, (double)R, (double)ctx->RA, N, k, k >= 1 && ctx->parent_form_coarse(), karr,
+                              ctx->stream));
     void* lvl = (char*)ctx->d_kspec + csz * ctx->kstride * k;
     if (ctx->prec == FLGF_FP64) {
-      STEP(launch_kernel_spectra<double>(N, karr, lvl, tmp, k >= 1 ? 1 : 0, ctx->stream));
+      STEP(launch_kernel_spectra<double>(N, karr, lvl, tmp, 0, ctx->stream));
     } else {
       STEP(launch_kernel_spectra<float>(N, karr, lvl, tmp, k >= 1 ? 1 : 0, ctx->stream));
     }
@@ -375,6 +385,9 @@ extern "C" int flgf_kernel_spectrum(flgf_ctx* ctx, int k, int d0, int d1, int d2
   const int N = ctx->N, NW = nfreq(N);
   const int d = off_index(d0, d1, d2);
   const bool f64 = ctx->prec == FLGF_FP64;
+  // near pairs do not interact above the finest level (FP64 keeps the spectra
+  // that take them out of the parents' products there)
+  const bool zero = k >= 1 && std::abs(d0) <= 1 && std::abs(d1) <= 1 && std::abs(d2) <= 1;
   const int T = f64 ? 2 : 4;
   const size_t csz = f64 ? 16 : 8;
   std::vector<char> lvl(csz * ctx->kstride);
@@ -392,6 +405,7 @@ extern "C" int flgf_kernel_spectrum(flgf_ctx* ctx, int k, int d0, int d1, int d2
       out[2 * w] = v[0];
       out[2 * w + 1] = v[1];
     }
+    if (zero) out[2 * w] = out[2 * w + 1] = 0.0;
   }
   return FLGF_OK;
 }
@@ -471,6 +485,23 @@ extern "C" void flgf_blockset_destroy(flgf_blockset* bs) {
   delete bs;
 }
 
+// The near pairs (|d|_inf <= 1) of a target parent's children and those of its
+// neighbour cell e: f(a, b, kernel offset index) of each; returns their number.
+template <typename F>
+static int near_pairs(int e, const int* tgt, const int* src, F&& f) {
+  int n = 0;
+  for (int a = 0; a < 8; ++a)
+    for (int b = 0; b < 8; ++b) {
+      if (tgt[a] < 0 || src[b] < 0) continue;
+      const int d0 = (a >> 2) - (b >> 2) - 2 * (e / 9 - 1), d1 = (a >> 1 & 1) - (b >> 1 & 1) - 2 * ((e / 3) % 3 - 1),
+                d2 = (a & 1) - (b & 1) - 2 * (e % 3 - 1);
+      if (std::abs(d0) > 1 || std::abs(d1) > 1 || std::abs(d2) > 1) continue;
+      f(a, b, off_index(d0, d1, d2));
+      ++n;
+    }
+  return n;
+}
+
 // FMM launch lists of phase l for the given instances (their is_src /
 // need_tgt masks select sources and targets), appended to arena ar.
 static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<const Inst*>& insts, PhaseOff& ph, bool count,
@@ -487,9 +518,12 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   // inverse FFT list: finest octree level, then the coarser ones (their own launch)
   std::vector<int> fwd_gid, fwd_sid, inv_sid, inv_gid, inv_sid_c, inv_gid_c;
   std::vector<double> inv_scale, inv_scale_c;
-  // sources and targets (with the squared spacing) of the finest octree level
+  // sources and targets (octree level, squared spacing) of the levels that run between parents
+  struct Tgt { int gid, k; double scale; };
   std::vector<int> src0;
-  std::vector<std::pair<int, double>> tgt0;
+  std::vector<Tgt> tgt0;
+  const bool pform = ctx->parent_form(), pcoarse = ctx->parent_form_coarse();
+  auto by_parents = [&](size_t k) { return k == 0 ? pform : pcoarse; };
   // parents with targets of dense tiles per octree level, in tile order
   std::vector<std::vector<ParentRec>> dpool;
   std::vector<ListGroup> groups;
@@ -556,7 +590,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     // products of a neighbour cell in the dense kernel, in units of a child
     // pair's: 64 of the child-pair kernels; the parent form's cost (8 products
     // and its share of the parents' transforms) is that of kPfPairs pairs
-    const int per_cell = k == 0 && ctx->parent_form() ? pf_pairs(ctx->prec == FLGF_FP64) : 64;
+    const int per_cell = by_parents(k) ? pf_pairs(ctx->prec == FLGF_FP64) : 64;
     for (int t0 = lo[0]; t0 <= hi[0]; t0 += TP[0])
       for (int t1 = lo[1]; t1 <= hi[1]; t1 += TP[1])
         for (int t2 = lo[2]; t2 <= hi[2]; t2 += TP[2]) {
@@ -624,6 +658,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
           // parent records of the tile's parents that have targets
           std::vector<ParentRec> recs;
           int64_t dense = 0;  // complex MACs per frequency of the parent-group kernel
+          int64_t out = 0;    // near pairs to take out of the parents' products, on the pair lists themselves
           for (int p0 = 0; p0 < tl.P[0]; ++p0)
             for (int p1 = 0; p1 < tl.P[1]; ++p1)
               for (int p2 = 0, last_p2 = -2; p2 < tl.P[2]; ++p2) {
@@ -650,12 +685,14 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
                     any_src |= r.cell[e][b] >= 0;
                   }
                   dense += any_src ? per_cell : 0;
+                  if (any_src && excl && by_parents(k)) out += near_pairs(e, r.tgt, r.cell[e], [](int, int, int) {});
                 }
                 r.follows = last_p2 == p2 - 1;
                 last_p2 = p2;
                 recs.push_back(r);
               }
-          if (useful * 100 < (int64_t)list_pct * dense) {
+          // (the near pairs to take out run on the list kernel at its own cost)
+          if (list_pct > 0 && useful * 100 < (int64_t)list_pct * dense + 100 * out) {
             // sparse tile: its targets join the pair-list pool of octree level k
             for (int ti = 0; ti < (int)tg.size(); ++ti)
               if (tg[ti] >= 0) job.lrecs.push_back({tg[ti], std::move(plist[ti])});
@@ -686,10 +723,10 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     for (size_t k = 0; k < in.lv.size(); ++k) {
       for (size_t i = 0; i < in.lv[k].size(); ++i) {
         const int gid = in.gid0[k] + (int)i;
-        if (in.is_src[k][i]) (k == 0 ? src0 : fwd_gid).push_back(gid);
+        if (in.is_src[k][i]) (k == 0 || by_parents(k) ? src0 : fwd_gid).push_back(gid);
         if (in.need_tgt[k][i]) {
-          if (k == 0) {
-            tgt0.push_back({gid, in.h * in.h});
+          if (k == 0 || by_parents(k)) {
+            tgt0.push_back({gid, (int)k, in.h * in.h});
           } else {
             inv_sid_c.push_back(gid - ph.gid_begin);
             inv_gid_c.push_back(gid);
@@ -739,43 +776,16 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       for (auto& r : job.lrecs) lpool[job.k].push_back(std::move(r));
     }
   }
-  // block spectra and inverse transforms of the finest octree level: where it
-  // runs between parents, only the blocks of the pair lists
-  if (count) {
-    bs->n_fwd += (int64_t)(fwd_gid.size() + src0.size());
-    bs->n_inv += (int64_t)(inv_gid_c.size() + tgt0.size());
-    for (int k = 0; k <= maxtop; ++k) bs->n_koff += kNOff;
-  }
-  const bool pform = ctx->parent_form();
-  {
-    std::vector<uint8_t> lsrc(ph.nblocks, !pform), ltgt(ph.nblocks, !pform);
-    if (pform && !lpool.empty())
-      for (const auto& r : lpool[0]) {
-        ltgt[r.first] = 1;
-        for (int w : r.second) lsrc[w >> 9] = 1;
-      }
-    for (int gid : src0)
-      if (lsrc[gid - ph.gid_begin]) fwd_gid.push_back(gid);
-    for (const auto& t : tgt0)
-      if (ltgt[t.first - ph.gid_begin]) {
-        inv_sid.push_back(t.first - ph.gid_begin);
-        inv_gid.push_back(t.first);
-        inv_scale.push_back(t.second);
-      }
-    for (int gid : fwd_gid) fwd_sid.push_back(gid - ph.gid_begin);
-  }
-  const int n_inv0 = (int)inv_gid.size();
-  inv_gid.insert(inv_gid.end(), inv_gid_c.begin(), inv_gid_c.end());
-  inv_sid.insert(inv_sid.end(), inv_sid_c.begin(), inv_sid_c.end());
-  inv_scale.insert(inv_scale.end(), inv_scale_c.begin(), inv_scale_c.end());
   // dense MAC: parent groups of every octree level (or frequency-lane groups;
-  // the finest level's are those of the products between parents)
+  // those of the levels between parents come first)
   HadLists hl;
   FlLists fll;
+  std::vector<uint8_t> follows;  // of the parents of these levels, in the order of the groups
   for (int k = 0; k < (int)dpool.size(); ++k) {
-    if (k == 0 && pform) {
+    if (by_parents(k)) {
       const bool f64 = ctx->prec == FLGF_FP64;
-      pack_fl_groups(0, dpool[0], fll, pf_max_parents(f64), pf_max_cells(f64));
+      pack_fl_groups(k, dpool[k], fll, pf_max_parents(f64), pf_max_cells(f64), true);
+      for (const ParentRec& r : dpool[k]) follows.push_back(r.follows);
       ph.n_pf = (int)fll.groups.size();
     } else if (fl)
       pack_fl_groups(k, dpool[k], fll);
@@ -783,9 +793,68 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       pack_parent_groups(k, dpool[k], nchunk, had_kernel_units(ctx->prec == FLGF_FP64), hl, ctx->order_by_list);
   }
   ph.n_fl = (int)fll.groups.size();
+  // the near pairs of the coarser levels that the parents' products contain:
+  // pair lists of their own, whose results are added to the parents'
+  std::vector<std::vector<std::pair<int, std::vector<int>>>> opool(dpool.size());
+  for (int gi = 0; gi < ph.n_pf; ++gi) {
+    const FlGroup& g = fll.groups[gi];
+    if (g.level == 0) continue;
+    for (int m = 0; m < g.nact; ++m) {
+      const int* tgt = &fll.tgt_ids[(size_t)(g.row_off + m) * 8];
+      const uint16_t* row = &fll.rows[(size_t)(g.row_off + m) * kFlRowStride];
+      std::vector<int> list[8];
+      for (int j = 0; j < row[0]; ++j) {
+        const int* src = &fll.cells[(size_t)(g.cell_off + (row[1 + j] & 0x7FF)) * 8];
+        near_pairs(row[1 + j] >> 11, tgt, src, [&](int a, int b, int off) { list[a].push_back((src[b] << 9) | off); });
+      }
+      for (int a = 0; a < 8; ++a)
+        if (!list[a].empty()) opool[g.level].push_back({tgt[a], std::move(list[a])});
+    }
+  }
+  // block spectra and inverse transforms: of the levels between parents, only
+  // the blocks of the pair lists
+  if (count) {
+    bs->n_fwd += (int64_t)(fwd_gid.size() + src0.size());
+    bs->n_inv += (int64_t)(inv_gid_c.size() + tgt0.size());
+    for (int k = 0; k <= maxtop; ++k) bs->n_koff += kNOff;
+  }
+  {
+    enum : uint8_t { kNone, kAssign, kAdd };
+    std::vector<uint8_t> lsrc(ph.nblocks, !pform), ltgt(ph.nblocks, pform ? kNone : kAssign);
+    auto mark = [&](const std::vector<std::pair<int, std::vector<int>>>& pool, uint8_t how) {
+      for (const auto& r : pool) {
+        ltgt[r.first] = how;
+        for (int w : r.second) lsrc[w >> 9] = 1;
+      }
+    };
+    if (pform)
+      for (size_t k = 0; k < lpool.size(); ++k)
+        if (by_parents(k)) mark(lpool[k], kAssign);
+    for (const auto& pool : opool) mark(pool, kAdd);
+    for (int gid : src0)
+      if (lsrc[gid - ph.gid_begin]) fwd_gid.push_back(gid);
+    for (int gid : fwd_gid) fwd_sid.push_back(gid - ph.gid_begin);
+    auto inverse_of = [&](auto&& which) {
+      for (const Tgt& t : tgt0)
+        if (which(t, ltgt[t.gid - ph.gid_begin])) {
+          inv_sid.push_back(t.gid - ph.gid_begin);
+          inv_gid.push_back(t.gid);
+          inv_scale.push_back(t.scale);
+        }
+    };
+    inverse_of([](const Tgt& t, uint8_t how) { return t.k == 0 && how == kAssign; });
+    ph.n_inv0 = (int)inv_gid.size();
+    inv_gid.insert(inv_gid.end(), inv_gid_c.begin(), inv_gid_c.end());
+    inv_sid.insert(inv_sid.end(), inv_sid_c.begin(), inv_sid_c.end());
+    inv_scale.insert(inv_scale.end(), inv_scale_c.begin(), inv_scale_c.end());
+    inverse_of([](const Tgt& t, uint8_t how) { return t.k > 0 && how == kAssign; });
+    const size_t assigned = inv_gid.size();
+    inverse_of([](const Tgt&, uint8_t how) { return how == kAdd; });
+    ph.n_inv_add = (int)(inv_gid.size() - assigned);
+  }
   if (ph.n_pf > 0) {
     std::vector<double> scale_of(ph.nblocks, 0.0);
-    for (const auto& t : tgt0) scale_of[t.first - ph.gid_begin] = t.second;
+    for (const Tgt& t : tgt0) scale_of[t.gid - ph.gid_begin] = t.scale;
     std::unordered_map<int, int> col_of;  // first source child of a parent -> its column
     std::vector<int> ccol, tcol, sch, tch;
     std::vector<double> pscale;
@@ -812,7 +881,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
         }
         pscale.push_back(sc);
       }
-      PfGroup pg{g.ncell, g.nact, 0, g.cell_off, g.row_off, (int)(items.size() / kPfItem)};
+      PfGroup pg{g.ncell, g.nact, 0, g.cell_off, g.row_off, (int)(items.size() / kPfItem), g.level};
       // pairs first, then single parents, so the warps' round-robin ends together
       auto add_item = [&](int m, int n) {
         uint16_t it[kPfItem] = {0};
@@ -832,7 +901,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       };
       std::vector<int> single;
       for (int m = 0; m < g.nact;) {
-        const bool pair = m + 1 < g.nact && dpool[0][g.row_off + m + 1].follows;
+        const bool pair = m + 1 < g.nact && follows[g.row_off + m + 1];
         if (pair) add_item(m, 2);
         else single.push_back(m);
         m += pair ? 2 : 1;
@@ -895,8 +964,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   ph.fll_ent = ar.add(fq.ent);
   // pair-list groups: consecutive pool targets (spatially close, so their
   // source sets overlap) up to kListTargets targets or kListMaxSrc sources
-  for (int k = 0; k < (int)lpool.size(); ++k) {
-    const auto& pool = lpool[k];
+  auto pack_lists = [&](int k, const std::vector<std::pair<int, std::vector<int>>>& pool) {
     size_t pos = 0;
     while (pos < pool.size()) {
       std::unordered_map<int, int> slot;
@@ -937,7 +1005,11 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       max_group_src = std::max(max_group_src, g.nsrc);
       groups.push_back(g);
     }
-  }
+  };
+  for (int k = 0; k < (int)lpool.size(); ++k) pack_lists(k, lpool[k]);
+  ph.n_groups = (int)groups.size();
+  for (int k = 0; k < (int)opool.size(); ++k) pack_lists(k, opool[k]);
+  ph.n_groups_out = (int)groups.size() - ph.n_groups;
   ph.n_prep = (int)prep_src.size();
   ph.prep_src = ar.add(prep_src);
   ph.prep_dst = ar.add(prep_dst);
@@ -990,7 +1062,6 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   ph.src_ids = ar.add(hl.src_ids);
   ph.tgt_ids = ar.add(hl.tgt_ids);
   ph.par_tab = ar.add(hl.par_tab);
-  ph.n_groups = (int)groups.size();
   ph.max_group_src = max_group_src;
   ph.groups = ar.add(groups);
   ph.l_tgt = ar.add(l_tgt);
@@ -998,7 +1069,6 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   ph.l_ent = ar.add(l_ent);
   ph.l_src = ar.add(l_src);
   ph.n_inv = (int)inv_gid.size();
-  ph.n_inv0 = n_inv0;
   ph.inv_sid = ar.add(inv_sid);
   ph.inv_gid = ar.add(inv_gid);
   ph.inv_scale = ar.add(inv_scale);
@@ -1633,7 +1703,8 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
                                    ar.at<int>(ph.pf_ccol), ar.at<int>(ph.pf_tcol), pf_src, ph.n_pfs,
                                    pf_dst, ph.n_pft, c->d_pspec, ph.fl_ncomp, ph.pf_src_stride,
                                    ph.pf_tgt_stride, s));
-    KRUN(ph.n_work, launch_hadamard<R>(N, ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
+    if constexpr (sizeof(R) == 4)
+      KRUN(ph.n_work, launch_hadamard<R>(N, ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
                                        ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
                                        ar.at<uint16_t>(ph.par_tab), bs->spec, bs->acc, ph.nblocks, c->d_kspec,
                                        c->kstride, s));
@@ -1645,7 +1716,8 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
     KRUN(ph.n_fll, launch_hadamard_fll(N, ar.at<FllGroup>(ph.fll_groups), ph.n_fll, ar.at<int>(ph.fll_tgt),
                                        ar.at<int>(ph.fll_beg), ar.at<int>(ph.fll_len), ar.at<uint32_t>(ph.fll_ent),
                                        bs->spec, bs->acc, ph.nblocks, c->d_kspec, c->kstride, s));
-    KRUN(ph.n_groups, launch_hadamard_list<R>(N, ar.at<ListGroup>(ph.groups), ph.n_groups, ph.max_group_src,
+    const int n_lists = ph.n_groups + ph.n_groups_out;
+    KRUN(n_lists, launch_hadamard_list<R>(N, ar.at<ListGroup>(ph.groups), n_lists, ph.max_group_src,
                                               ar.at<int>(ph.l_tgt), ar.at<int>(ph.l_len), ar.at<int>(ph.l_ent),
                                               ar.at<int>(ph.l_src), bs->spec, bs->acc, ph.nblocks, c->d_kspec,
                                               c->kstride, s));
@@ -1654,11 +1726,11 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
     StageScope sc(bs, 4);
     KRUN(ph.n_pft, launch_pf_inverse<R>(N, pf_dst, ar.at<int>(ph.pf_tch), ar.at<double>(ph.pf_scale), ph.n_pft, unodes, s));
     KRUN(ph.n_inv0, launch_fft_inverse<R>(N, bs->acc, ph.nblocks, ar.at<int>(ph.inv_sid), ar.at<int>(ph.inv_gid),
-                                          ar.at<double>(ph.inv_scale), ph.n_inv0, unodes, s, false));
+                                          ar.at<double>(ph.inv_scale), ph.n_inv0, 0, unodes, s, false));
     const int nc = ph.n_inv - ph.n_inv0;
     KRUN(nc, launch_fft_inverse<R>(N, bs->acc, ph.nblocks, ar.at<int>(ph.inv_sid) + ph.n_inv0,
                                    ar.at<int>(ph.inv_gid) + ph.n_inv0, ar.at<double>(ph.inv_scale) + ph.n_inv0, nc,
-                                   unodes, s, comp));
+                                   ph.n_inv_add, unodes, s, comp));
   }
   {
     StageScope sc(bs, 5);

@@ -36,6 +36,10 @@
 // the remaining near offsets |d|_inf <= 1 have zero spectra in the table
 // (set up that way for octree levels >= 1).
 // Complex multiply-adds are written as four fused multiply-adds.
+// FP32 contexts with FLGF_CTX_MAC = 0 only: FP64 runs every level between
+// parents (parent.cu), coarser ones included, which replaced a three-product
+// form of this kernel (11 x 9 x 13 blocks of 16^3: 6.77 -> 2.1 ms with the near
+// pairs' lists and transforms).
 #include <algorithm>
 #include <unordered_map>
 #include <vector>
@@ -66,27 +70,12 @@ __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup
   const int S = 8 * NC;  // slots per (chunk, group): child b of cell c at b * NC + c
 
   int4* Ks = Fs + (size_t)gp.cpc * NG * S;
-  // FP64 uses the three-product form (see below): per (offset, group) 32 bytes
-  // holding kr, kr + ki, ki - kr and padding; FP32 keeps the complex values
-  constexpr bool G3 = sizeof(R) == 8;
-  constexpr int KV = (G3 ? 2 * kNOff * NG : kNOff * T * (int)sizeof(cplx<R>) / 16);  // 16-byte vectors per chunk
+  constexpr int KV = kNOff * T * (int)sizeof(cplx<R>) / 16;  // 16-byte vectors per chunk
   uint16_t* NB = reinterpret_cast<uint16_t*>(Ks + (size_t)gp.cpc * KV);
   for (int i = tid; i < 27 * gp.nact; i += kHadThreads) NB[i] = par_tab[gp.par_off + i];
-  if constexpr (G3) {
-    for (int i = tid; i < wk.nch * kNOff * T; i += kHadThreads) {
-      const int cs = i / (kNOff * T), d = (i / T) % kNOff, f = i % T;
-      const cplx<R> k = kspec[(size_t)gp.level * kstride + ((size_t)(wk.chunk0 + cs) * kNOff + d) * T + f];
-      R* dst = reinterpret_cast<R*>(Ks + (size_t)cs * KV + (size_t)(d * NG + f) * 2);
-      dst[0] = k.re;
-      dst[1] = k.re + k.im;
-      dst[2] = k.im - k.re;
-      dst[3] = R(0);
-    }
-  } else {
-    for (int i = tid; i < wk.nch * KV; i += kHadThreads) {
-      const int cs = i / KV, v = i % KV;
-      Ks[i] = __ldg(reinterpret_cast<const int4*>(kspec + (size_t)gp.level * kstride + (size_t)(wk.chunk0 + cs) * kNOff * T) + v);
-    }
+  for (int i = tid; i < wk.nch * KV; i += kHadThreads) {
+    const int cs = i / KV, v = i % KV;
+    Ks[i] = __ldg(reinterpret_cast<const int4*>(kspec + (size_t)gp.level * kstride + (size_t)(wk.chunk0 + cs) * kNOff * T) + v);
   }
   for (int cs = 0; cs < wk.nch; ++cs) {
     int4* fdst = Fs + (size_t)cs * NG * S;
@@ -107,22 +96,13 @@ __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup
   const int chunk = wk.chunk0 + cs;
   const int f0 = g * TT;
   const cplx<R>* Fg = reinterpret_cast<const cplx<R>*>(Fs + (size_t)(cs * NG + g) * S);
-  const cplx<R>* Kc = reinterpret_cast<const cplx<R>*>(Ks + (size_t)cs * KV) + f0;  // complex form
-  const int4* Kg = Ks + (size_t)cs * KV + g * 2;                                      // three-product form
+  const cplx<R>* Kc = reinterpret_cast<const cplx<R>*>(Ks + (size_t)cs * KV) + f0;
 
-  // FP32: ar, ai accumulate re and im with four FMAs per pair.  FP64 (bound by
-  // the FP64 FMA rate) takes the three-product form: with s = fr + fi,
-  // re(k f) = kr s - (kr + ki) fi and im(k f) = kr s + (ki - kr) fr, so the
-  // accumulators ar = sum kr s, ai = sum (kr + ki) fi, a3 = sum (ki - kr) fr
-  // take three FMAs per pair, and re = ar - ai, im = ar + a3.
-  R ar[8][TT], ai[8][TT], a3[8][G3 ? TT : 1];
+  R ar[8][TT], ai[8][TT];
 #pragma unroll
   for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int t = 0; t < TT; ++t) {
-      ar[a][t] = R(0); ai[a][t] = R(0);
-      if constexpr (G3) a3[a][t] = R(0);
-    }
+    for (int t = 0; t < TT; ++t) { ar[a][t] = R(0); ai[a][t] = R(0); }
 
   // e stays the (warp-uniform) loop index, so the kernel-spectrum addresses
   // below are uniform across the warp; the next neighbour's cell is read one
@@ -136,14 +116,13 @@ __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup
     const int e0 = e / 9 - 1, e1 = (e / 3) % 3 - 1, e2 = e % 3 - 1;
     // the 8 children b of neighbour parent p + e, TT frequencies each (zero where absent)
     const cplx<R>* fb = Fg + (size_t)c * TT;
-    R fr[8][TT], fi[8][TT], fs[8][G3 ? TT : 1];
+    R fr[8][TT], fi[8][TT];
 #pragma unroll
     for (int b = 0; b < 8; ++b)
 #pragma unroll
       for (int t = 0; t < TT; ++t) {
         const cplx<R> v = fb[(size_t)b * NC * TT + t];
         fr[b][t] = v.re; fi[b][t] = v.im;
-        if constexpr (G3) fs[b][t] = v.re + v.im;
       }
     // d = a - b - 2e takes 27 values delta - 2e (delta = a - b in {-1,0,1}^3):
     // one kernel-spectrum load per delta, applied to every (a, b) pair with a - b = delta
@@ -152,36 +131,20 @@ __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup
     for (int dl = 0; dl < 27; ++dl) {
       const int l0 = dl / 9 - 1, l1 = (dl / 3) % 3 - 1, l2 = dl % 3 - 1;
       const int d = eoff + l0 * 49 + l1 * 7 + l2;
-      if constexpr (G3) {
-        const int4* kp = Kg + (size_t)d * NG * 2;
-        const int4 kv0 = kp[0], kv1 = kp[1];
-        const R k0 = reinterpret_cast<const R*>(&kv0)[0], k1 = reinterpret_cast<const R*>(&kv0)[1];
-        const R k2 = reinterpret_cast<const R*>(&kv1)[0];
+      const int4 kv = *reinterpret_cast<const int4*>(Kc + (size_t)d * T);
+      const cplx<R>* kk = reinterpret_cast<const cplx<R>*>(&kv);
 #pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          const int b0 = (a >> 2) - l0, b1 = ((a >> 1) & 1) - l1, b2 = (a & 1) - l2;
-          if (b0 < 0 || b0 > 1 || b1 < 0 || b1 > 1 || b2 < 0 || b2 > 1) continue;  // resolved at compile time
-          const int b = (b0 << 2) | (b1 << 1) | b2;
-          ar[a][0] = fma(k0, fs[b][0], ar[a][0]);
-          ai[a][0] = fma(k1, fi[b][0], ai[a][0]);
-          a3[a][0] = fma(k2, fr[b][0], a3[a][0]);
-        }
-      } else {
-        const int4 kv = *reinterpret_cast<const int4*>(Kc + (size_t)d * T);
-        const cplx<R>* kk = reinterpret_cast<const cplx<R>*>(&kv);
+      for (int a = 0; a < 8; ++a) {
+        const int b0 = (a >> 2) - l0, b1 = ((a >> 1) & 1) - l1, b2 = (a & 1) - l2;
+        if (b0 < 0 || b0 > 1 || b1 < 0 || b1 > 1 || b2 < 0 || b2 > 1) continue;  // resolved at compile time
+        const int b = (b0 << 2) | (b1 << 1) | b2;
 #pragma unroll
-        for (int a = 0; a < 8; ++a) {
-          const int b0 = (a >> 2) - l0, b1 = ((a >> 1) & 1) - l1, b2 = (a & 1) - l2;
-          if (b0 < 0 || b0 > 1 || b1 < 0 || b1 > 1 || b2 < 0 || b2 > 1) continue;  // resolved at compile time
-          const int b = (b0 << 2) | (b1 << 1) | b2;
-#pragma unroll
-          for (int t = 0; t < TT; ++t) {
-            const cplx<R> k = kk[t];
-            ar[a][t] = fma(k.re, fr[b][t], ar[a][t]);
-            ar[a][t] = fma(-k.im, fi[b][t], ar[a][t]);
-            ai[a][t] = fma(k.re, fi[b][t], ai[a][t]);
-            ai[a][t] = fma(k.im, fr[b][t], ai[a][t]);
-          }
+        for (int t = 0; t < TT; ++t) {
+          const cplx<R> k = kk[t];
+          ar[a][t] = fma(k.re, fr[b][t], ar[a][t]);
+          ar[a][t] = fma(-k.im, fi[b][t], ar[a][t]);
+          ai[a][t] = fma(k.re, fi[b][t], ai[a][t]);
+          ai[a][t] = fma(k.im, fr[b][t], ai[a][t]);
         }
       }
     }
@@ -194,10 +157,7 @@ __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup
     if (sid < 0) continue;
     cplx<R>* o = acc + chunk_offset<R>(chunk, sid, spec_blocks) + f0;
 #pragma unroll
-    for (int t = 0; t < TT; ++t) {
-      if constexpr (G3) o[t] = cplx<R>{ar[a][t] - ai[a][t], ar[a][t] + a3[a][t]};
-      else o[t] = cplx<R>{ar[a][t], ai[a][t]};
-    }
+    for (int t = 0; t < TT; ++t) o[t] = cplx<R>{ar[a][t], ai[a][t]};
   }
 }
 
@@ -325,8 +285,6 @@ template cudaError_t launch_hadamard_list<double>(int, const ListGroup*, int, in
 
 template cudaError_t launch_hadamard<float>(int, const HadGroup*, const HadWork*, int, int, const int*, const int*,
                                             const uint16_t*, const void*, void*, int, const void*, size_t, cudaStream_t);
-template cudaError_t launch_hadamard<double>(int, const HadGroup*, const HadWork*, int, int, const int*, const int*,
-                                             const uint16_t*, const void*, void*, int, const void*, size_t, cudaStream_t);
 
 // Shared memory of a group in 32-byte units: per chunk 8 slots per cell and
 // the 343 kernel spectra, plus the [27][nact] int16 neighbour table.

@@ -418,7 +418,8 @@ static int fl_cell_key(const int* ch) {
   return -1;
 }
 
-void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L, int max_parents, int max_cells) {
+void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L, int max_parents, int max_cells,
+                    bool near_rows) {
   size_t pos = 0;
   while (pos < recs.size()) {
     // consecutive parents (tile order, so they share cells) while the group's cells fit
@@ -459,7 +460,7 @@ void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L, i
         const int key = fl_cell_key(r.cell[e]);
         if (key < 0) continue;
         const uint32_t mask = fl_delta_mask(level, e, r.tgt, r.cell[e]);
-        if (!mask) continue;  // only near pairs of a coarse octree level: nothing to add
+        if (!mask && !near_rows) continue;  // only near pairs of a coarse octree level: nothing to add
         dm[n] = mask;
         row[1 + n++] = (uint16_t)((e << 11) | cell_of.at(key));
       }

@@ -36,7 +36,9 @@ cudaError_t launch_lgf_eval(const double* table, int R, double rt, double ra, co
                             int n, double* out, cudaStream_t s);
 // (2N)^3 circular kernel arrays for octree level k, every offset d in [-3,3]^3:
 // out[d][i0][i1][i2] = G(2^k (N d + Delta)), Delta = i (i < N) or i - 2N (i > N), 0 at i == N.
-cudaError_t launch_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k,
+// near_out: the near offsets (|d|_inf <= 1) hold what takes a near pair out of
+// the parents' products instead: -G where |N d + Delta|_inf > N, 0 elsewhere.
+cudaError_t launch_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k, bool near_out,
                                  double* out, cudaStream_t s);
 
 // ---- a2/a4 FFTs (fft.cu) ---------------------------------------------------
@@ -45,11 +47,11 @@ cudaError_t fft_init_constants();
 template <typename R>
 cudaError_t launch_fft_forward(int N, const R* nodes, const int* gids, const int* sids, int count,
                                void* spec, int spec_blocks, cudaStream_t s);
-// Inverse C2R, keep the first N^3 outputs, scale by scale[i]/(2N)^3, write (or add) to out[gids[i]].
+// Inverse C2R, keep the first N^3 outputs, scale by scale[i]/(2N)^3, write to out[gids[i]]; the last n_add add to it (FP64).
 // compensated: FP32 spectra transformed in float-float arithmetic (ffloat.cuh).
 template <typename R>
 cudaError_t launch_fft_inverse(int N, const void* acc, int spec_blocks, const int* sids, const int* gids,
-                               const double* scales, int count, R* out, cudaStream_t s, bool compensated);
+                               const double* scales, int count, int n_add, R* out, cudaStream_t s, bool compensated);
 // Kernel spectra of one octree level from the (2N)^3 kernel arrays (FP64 FFT),
 // stored as [chunk][343][T] in precision R; zero_near stores the 27 near
 // offsets as zero (octree levels >= 1 never use them).
@@ -102,8 +104,8 @@ struct HadLists {
 // first, equal sets together) instead of keeping the record order.
 void pack_parent_groups(int level, const std::vector<ParentRec>& recs, int nchunk, int kunits, HadLists& L,
                         bool order_by_list = false);
-// Kernel-spectrum shared memory per chunk of the dense MAC, in 32-byte units:
-// the complex values (FP32) or the three-product form (FP64, twice as large).
+// Kernel-spectrum shared memory per chunk of the dense MAC, in 32-byte units
+// (the kernel runs on FP32 data).
 constexpr int had_kernel_units(bool fp64) { return fp64 ? 2 * kNOff : kNOff; }
 template <typename R>
 cudaError_t launch_hadamard(int N, const HadGroup* groups, const HadWork* work, int nwork, int max_units,
@@ -165,9 +167,10 @@ struct FlLists {
   int max_cells = 0, max_parents = 0;
 };
 // Packs parent records, in order, into frequency-lane groups of one octree
-// level, of at most max_parents parents and max_cells neighbour cells.
+// level, of at most max_parents parents and max_cells neighbour cells.  Cells
+// that only near pairs of a coarser level reach have no row, unless near_rows.
 void pack_fl_groups(int level, const std::vector<ParentRec>& recs, FlLists& L, int max_parents = kFlMaxParents,
-                    int max_cells = kFlMaxCells);
+                    int max_cells = kFlMaxCells, bool near_rows = false);
 uint32_t fl_delta_mask(int level, int e, const int* tgt, const int* src);
 size_t fl_smem_bytes(int max_cells, int max_parents);
 // ncomp > 1: a vector block set's components, whose spectrum columns are
@@ -203,8 +206,9 @@ cudaError_t launch_hadamard_fll(int N, const FllGroup* groups, int ngroups, cons
                                 const int* len, const uint32_t* ent, const void* spec, void* acc, int spec_blocks,
                                 const void* kspec, size_t kspec_level_stride, cudaStream_t s);
 
-// ---- the finest octree level between parents (parent.cu) ---------------------
-// The groups are the frequency-lane groups of octree level 0.  Their parents
+// ---- octree levels between parents (parent.cu) --------------------------------
+// The groups are the frequency-lane groups of octree level 0 (FP64: of all
+// levels).  Their parents
 // are taken in items of two neighbours along axis 2 (consecutive in the group)
 // or one.  Item: uint16 entries; 9 q + c (q < 4, c = 3 (e0 + 1) + e1 + 1) = 33 x
 // (index in the group) of the neighbour cell (e0, e1) one down of the first
@@ -216,6 +220,7 @@ cudaError_t launch_hadamard_fll(int N, const FllGroup* groups, int ngroups, cons
 struct PfGroup {
   int ncell, nact, nitem;
   int cell_off, row_off, item_off;
+  int level;  // octree level (kernel spectra)
 };
 constexpr int kPfItem = 40;  // uint16 per item: five 16-byte vectors
 constexpr int kPfMacThreads = 256;
@@ -247,8 +252,11 @@ constexpr size_t pf_smem_bytes(const PfLimits& l, int upc) {
 size_t pf_parent_values(int N);  // complex values of one parent's half-transformed spectrum
 size_t pf_kernel_values(int N);  // complex values of the 27 parent kernel spectra
 size_t pf_setup_bytes(int N);    // scratch of launch_pf_setup
-// Parent kernel arrays (FP64, lgf.cu): out[e][i0][i1][i2] = G(Delta - 2N e), Delta = i (i < 2N) or i - 4N (i > 2N), 0 at 2N.
-cudaError_t launch_parent_kernel_arrays(const double* table, int R, double rt, double ra, int N, double* out,
+// Parent kernel arrays of octree level k (FP64, lgf.cu) for the 8 offsets
+// e_a in {0, 1}: out[4 e0 + 2 e1 + e2][i0][i1][i2] = G(2^k (Delta - 2N e)), Delta = i
+// (i < 2N) or i - 4N (i > 2N), 0 at 2N; above the finest level 0 where
+// |Delta - 2N e|_inf <= N (near blocks only) and at e = 0 (siblings are near).
+cudaError_t launch_parent_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k, double* out,
                                         cudaStream_t s);
 template <typename R>
 cudaError_t launch_pf_setup(int N, const double* karr, void* tmp, void* kspec, cudaStream_t s);

@@ -69,6 +69,10 @@ __device__ double lgf_at(const double* __restrict__ table, int R, double rt2, do
   return lgf_asym2((double)a, (double)b, (double)c);
 }
 
+__device__ __forceinline__ long long max_abs(long long a, long long b, long long c) {
+  return max(max(a < 0 ? -a : a, b < 0 ? -b : b), c < 0 ? -c : c);
+}
+
 __global__ void lgf_eval_kernel(const double* __restrict__ table, int R, double rt2, double ra2,
                                 const int32_t* __restrict__ pts, int n, double* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -84,7 +88,7 @@ cudaError_t launch_lgf_eval(const double* table, int R, double rt, double ra, co
 }
 
 __global__ void kernel_arrays_kernel(const double* __restrict__ table, int R, double rt2, double ra2, int N,
-                                     int k, double* __restrict__ out) {
+                                     int k, bool near_out, double* __restrict__ out) {
   const int P = 2 * N;
   const size_t per = (size_t)P * P * P;
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -98,35 +102,38 @@ __global__ void kernel_arrays_kernel(const double* __restrict__ table, int R, do
   const long long x0 = s * ((long long)N * d0 + (i0 < N ? i0 : i0 - P));
   const long long x1 = s * ((long long)N * d1 + (i1 < N ? i1 : i1 - P));
   const long long x2 = s * ((long long)N * d2 + (i2 < N ? i2 : i2 - P));
-  out[idx] = lgf_at(table, R, rt2, ra2, x0, x1, x2);
+  const double g = lgf_at(table, R, rt2, ra2, x0, x1, x2);
+  const bool near = near_out && abs(d0) <= 1 && abs(d1) <= 1 && abs(d2) <= 1;
+  out[idx] = !near ? g : max_abs(x0, x1, x2) > s * N ? -g : 0.0;
 }
 
 __global__ void parent_kernel_arrays_kernel(const double* __restrict__ table, int R, double rt2, double ra2, int H,
-                                            double* __restrict__ out) {
+                                            int k, double* __restrict__ out) {
   const int P = 2 * H;
   const size_t per = (size_t)P * P * P;
   const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= per * 27) return;
+  if (idx >= per * 8) return;
   const int e = (int)(idx / per), rem = (int)(idx % per);
   const int i0 = rem / (P * P), i1 = (rem / P) % P, i2 = rem % P;
   if (i0 == H || i1 == H || i2 == H) { out[idx] = 0.0; return; }
-  const long long x0 = (i0 < H ? i0 : i0 - P) - (long long)H * (e / 9 - 1);
-  const long long x1 = (i1 < H ? i1 : i1 - P) - (long long)H * ((e / 3) % 3 - 1);
-  const long long x2 = (i2 < H ? i2 : i2 - P) - (long long)H * (e % 3 - 1);
-  out[idx] = lgf_at(table, R, rt2, ra2, x0, x1, x2);
+  const long long x0 = (i0 < H ? i0 : i0 - P) - (long long)H * (e >> 2);
+  const long long x1 = (i1 < H ? i1 : i1 - P) - (long long)H * ((e >> 1) & 1);
+  const long long x2 = (i2 < H ? i2 : i2 - P) - (long long)H * (e & 1);
+  const bool cut = k > 0 && (e == 0 || max_abs(x0, x1, x2) <= H / 2);
+  out[idx] = cut ? 0.0 : lgf_at(table, R, rt2, ra2, x0 * (1LL << k), x1 * (1LL << k), x2 * (1LL << k));
 }
 
-cudaError_t launch_parent_kernel_arrays(const double* table, int R, double rt, double ra, int N, double* out,
+cudaError_t launch_parent_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k, double* out,
                                         cudaStream_t s) {
-  const size_t P = 4 * (size_t)N, total = 27 * P * P * P;
-  parent_kernel_arrays_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(table, R, rt * rt, ra * ra, 2 * N, out);
+  const size_t P = 4 * (size_t)N, total = 8 * P * P * P;
+  parent_kernel_arrays_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(table, R, rt * rt, ra * ra, 2 * N, k, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k, double* out,
+cudaError_t launch_kernel_arrays(const double* table, int R, double rt, double ra, int N, int k, bool near_out, double* out,
                                  cudaStream_t s) {
   const size_t total = (size_t)kNOff * (2 * N) * (2 * N) * (2 * N);
-  kernel_arrays_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(table, R, rt * rt, ra * ra, N, k, out);
+  kernel_arrays_kernel<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(table, R, rt * rt, ra * ra, N, k, near_out, out);
   return cudaGetLastError();
 }
 

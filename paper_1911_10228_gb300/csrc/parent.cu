@@ -1,12 +1,23 @@
-// a2-a4 of the finest octree level between parents: the near field and the
+// a2-a4 between parents, for the finest octree level: the near field and the
 // influence lists of a finest-level target (Sec. 2.1) are together all the
 // children of its parent's 27 neighbours, so the level's interaction is a
 // convolution between PARENT blocks of H = 2N cells a side.  One zero-padded
 // FFT of P = 4N points an axis per parent replaces eight of 2N: a neighbour
 // pair then costs 8 NW complex products (NW frequencies of a child's padded
-// spectrum) where the child pairs cost 64 NW.  (Coarser octree levels exclude
-// the near field, which depends on the child, and keep the child-pair
-// kernels.)
+// spectrum) where the child pairs cost 64 NW.
+//
+// Coarser octree levels exclude the near field, which depends on the child.  In
+// FP64 they run between parents all the same: the parent kernels are zero for
+// |displacement|_inf <= N (reached by near pairs only; a block's siblings, e = 0,
+// need no product at all), and what the near pairs of neighbour parents still
+// get is taken out block by block: at most 19 pair-list entries a target with
+// the kernel -G where |displacement|_inf > N, added by the inverse transform.
+// The parts that cancel are no larger than those that stay, so the error is
+// the same (11 x 9 x 13 blocks of 16^3: 2.4e-14 from 64-bit values both ways).
+// FP64's FMA rate bounds it: 27 x 8 + 152 products instead of 1512 a parent.
+// Coarser levels, products and transforms: 11 x 9 x 13 blocks of 16^3 6.9 -> 2.0
+// ms, three-level torus of 8^3 blocks 4.0 -> 1.0 ms.  FP32 keeps the child-pair
+// kernels there: their spectra go through float-float inverse transforms.
 //
 // The transform along axis 0 is fused with the products, so HBM only holds
 // spectra of the two transformed axes, half as long as padded ones:
@@ -359,7 +370,7 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
     }
     R k0[27], k1[27], k2[G3 ? 27 : 1];
     {
-      const C2* kp = kspec + ((size_t)(unit * 2 + par) * 27) * 32 + lane;
+      const C2* kp = kspec + (((size_t)gp.level * D::U + unit) * 2 + par) * 27 * 32 + lane;
 #pragma unroll
       for (int e = 0; e < 27; ++e) {
         const C2 k = __ldg(kp + e * 32);
@@ -453,8 +464,11 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
   }
 }
 // ---------------------------------------------------------------------------
-// Setup (FP64): the 27 parent kernel arrays [27][P][P][P] to spectra, one axis
-// per pass by plain discrete Fourier sums (a few ms once per context).
+// Setup (FP64): parent kernel arrays to spectra, one axis per pass by plain
+// discrete Fourier sums.  G is even in every component, so the array of a
+// negative e_a is the mirror image along that axis of the positive one's: only
+// the 8 arrays with e_a >= 0 are transformed, and the packing reads the others
+// at negated frequencies (their negative k2 by Hermitian symmetry).
 // ---------------------------------------------------------------------------
 // axis 2: real rows [rows][P] -> [rows][NX]
 __global__ void pf_setup_axis2(const double* __restrict__ in, double2* __restrict__ out, int P, int NX, int rows) {
@@ -502,16 +516,23 @@ __global__ void pf_setup_axis(const double2* __restrict__ in, double2* __restric
     out[(a * P + k) * nb + b] = make_double2(re, im);
   }
 }
-// [27][k0][l] -> [unit][parity][27][32] in precision R
+// [8][k0][l] -> [unit][parity][27][32] in precision R
 template <typename R, int N>
 __global__ void pf_setup_pack(const double2* __restrict__ in, typename Vec2<R>::type* __restrict__ out) {
   using D = PfDims<N>;
+  constexpr int P = D::P, NX = D::NX;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (size_t)D::U * 2 * 27 * 32) return;
   const int lane = i % 32, e = (i / 32) % 27, par = (i / (32 * 27)) % 2, u = (int)(i / (32 * 27 * 2));
-  const int l = u * D::S + lane / D::H, k0 = 2 * (lane % D::H) + par;
-  const double2 v = in[((size_t)e * D::P + k0) * D::L + l];
-  out[i] = typename Vec2<R>::type{(R)v.x, (R)v.y};
+  const int l = u * D::S + lane / D::H, k2 = l % NX;
+  int k0 = 2 * (lane % D::H) + par, k1 = l / NX;
+  const int e0 = e / 9 - 1, e1 = (e / 3) % 3 - 1, e2 = e % 3 - 1;
+  const bool conj = e2 < 0;  // K(k0, k1, -k2) = conj K(-k0, -k1, k2)
+  if ((e0 < 0) != conj) k0 = (P - k0) % P;
+  if ((e1 < 0) != conj) k1 = (P - k1) % P;
+  const int base = (e0 != 0) * 4 + (e1 != 0) * 2 + (e2 != 0);
+  const double2 v = in[((size_t)base * P + k0) * D::L + k1 * NX + k2];
+  out[i] = typename Vec2<R>::type{(R)v.x, (R)(conj ? -v.y : v.y)};
 }
 
 template <typename R, int N>
@@ -519,17 +540,17 @@ static cudaError_t setup_spectra(const double* karr, void* tmp, void* kspec, cud
   using D = PfDims<N>;
   constexpr int P = D::P, NX = D::NX;
   double2* t0 = reinterpret_cast<double2*>(tmp);
-  double2* t1 = t0 + (size_t)27 * P * P * NX;
-  pf_setup_axis2<<<27 * P * P, 64, P * 24, s>>>(karr, t0, P, NX, 27 * P * P);
-  pf_setup_axis<<<27 * P * NX, 64, P * 32, s>>>(t0, t1, P, NX);       // axis 1: a = (e, i0), b = k2
-  pf_setup_axis<<<27 * P * NX, 64, P * 32, s>>>(t1, t0, P, P * NX);   // axis 0: a = e, b = (k1, k2)
+  double2* t1 = t0 + (size_t)8 * P * P * NX;
+  pf_setup_axis2<<<8 * P * P, 64, P * 24, s>>>(karr, t0, P, NX, 8 * P * P);
+  pf_setup_axis<<<8 * P * NX, 64, P * 32, s>>>(t0, t1, P, NX);       // axis 1: a = (e, i0), b = k2
+  pf_setup_axis<<<8 * P * NX, 64, P * 32, s>>>(t1, t0, P, P * NX);   // axis 0: a = e, b = (k1, k2)
   const size_t total = (size_t)D::U * 2 * 27 * 32;
   pf_setup_pack<R, N><<<(unsigned)((total + 255) / 256), 256, 0, s>>>(t0, reinterpret_cast<typename Vec2<R>::type*>(kspec));
   return cudaGetLastError();
 }
 
 size_t pf_kernel_values(int N) { return (size_t)4 * N * (2 * N + 1) * 2 * N * 2 * 27; }
-size_t pf_setup_bytes(int N) { return (size_t)2 * 16 * 27 * 4 * N * 4 * N * (2 * N + 1); }
+size_t pf_setup_bytes(int N) { return (size_t)2 * 16 * 8 * 4 * N * 4 * N * (2 * N + 1); }
 size_t pf_parent_values(int N) { return (size_t)4 * N * (2 * N + 1) * 2 * N; }
 
 template <typename R>
