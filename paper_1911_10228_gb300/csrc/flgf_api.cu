@@ -881,8 +881,8 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
         }
         pscale.push_back(sc);
       }
-      PfGroup pg{g.ncell, g.nact, 0, g.cell_off, g.row_off, (int)(items.size() / kPfItem), g.level};
-      // pairs first, then single parents, so the warps' round-robin ends together
+      PfGroup pg{g.ncell, g.nact, 0, g.cell_off, g.row_off, (int)(items.size() / kPfItem), g.level, 0};
+      // quads first, then pairs and single parents, so the warps' round-robin ends together
       auto add_item = [&](int m, int n) {
         uint16_t it[kPfItem] = {0};
         for (int i = 0; i < 36; ++i) it[i] = (uint16_t)(33 * g.ncell);
@@ -899,13 +899,46 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
         items.insert(items.end(), it, it + kPfItem);
         ++pg.nitem;
       };
-      std::vector<int> single;
+      std::vector<int> single, first(g.nact, 0);  // parents taken alone; 1 at the first of a pair
+      std::vector<int> own(g.ncell, -1);          // cell -> the parent that it is
+      auto cell_at = [&](int m, int e) {
+        const uint16_t* row = &fll.rows[(size_t)(g.row_off + m) * kFlRowStride];
+        for (int j = 0; j < row[0]; ++j)
+          if (row[1 + j] >> 11 == e) return row[1 + j] & 0x7FF;
+        return -1;
+      };
+      for (int m = 0; m < g.nact; ++m)
+        if (const int c = cell_at(m, 13); c >= 0) own[c] = m;
       for (int m = 0; m < g.nact;) {
         const bool pair = m + 1 < g.nact && follows[g.row_off + m + 1];
-        if (pair) add_item(m, 2);
+        if (pair) first[m] = 1;
         else single.push_back(m);
         m += pair ? 2 : 1;
       }
+      // quads: a pair and the one above it along axis 1 (FP32: shared memory bounds the products)
+      if (ctx->prec == FLGF_FP32)
+        for (int m = 0; m < g.nact; ++m) {
+          const int c = first[m] ? cell_at(m, 16) : -1, up = c < 0 ? -1 : own[c];
+          if (up < 0 || !first[up]) continue;
+          first[m] = first[up] = 0;
+          uint16_t it[2 * kPfItem] = {0};
+          for (int i = 0; i < 48; ++i) it[i] = (uint16_t)(33 * g.ncell);
+          for (int a = 0; a < 4; ++a) {
+            const uint16_t* row = &fll.rows[(size_t)(g.row_off + (a < 2 ? m : up) + (a & 1)) * kFlRowStride];
+            for (int j = 0; j < row[0]; ++j) {
+              const int e = row[1 + j] >> 11;
+              it[16 * (e / 9) + 4 * ((e / 3) % 3 + (a >> 1)) + e % 3 + (a & 1)] = (uint16_t)(33 * (row[1 + j] & 0x7FF));
+              it[50] |= (uint16_t)(1 << (e / 9));
+            }
+          }
+          it[48] = (uint16_t)m;
+          it[49] = (uint16_t)up;
+          items.insert(items.end(), it, it + 2 * kPfItem);
+          pg.nitem += 2;
+          ++pg.nquad;
+        }
+      for (int m = 0; m < g.nact; ++m)
+        if (first[m]) add_item(m, 2);
       for (int m : single) add_item(m, 1);
       ph.pf_lim.cells = std::max(ph.pf_lim.cells, pg.ncell);
       ph.pf_lim.parents = std::max(ph.pf_lim.parents, pg.nact);

@@ -144,7 +144,7 @@ extern "C" int flgf_convolve_static(flgf_ctx* ctx, int nblk, const int32_t* coor
     L.col[m] = m;
     L.scale[m] = h * h;
   }
-  L.group = PfGroup{np, np, np, 0, 0, 0, 0};
+  L.group = PfGroup{np, np, np, 0, 0, 0, 0, 0};
   const PfLimits lim{np, np, np};
 
   void* base = nullptr;

@@ -215,12 +215,17 @@ cudaError_t launch_hadamard_fll(int N, const FllGroup* groups, int ngroups, cons
 // parent (q = 0), at it (1), one up (2) and two up (3, pairs only), or 33 x ncell
 // (a zero line) where it has no sources; entry 36 the first parent (index in
 // the group), 37 the parents, 38 bit e0 + 1 set when cells of that e0 exist.
+// FP32 takes two such pairs that are neighbours along axis 1 as a quad, in the
+// room of two items: entry 16 (e0 + 1) + 4 p + q is the cell at (e0, p - 1, q - 1)
+// from the first parent, 48 the first parent, 49 the first one of the upper
+// pair, 50 the bits of e0.
 // Per cell the column of its parent in the source spectra, per target parent
 // its column in the result.  Spectra: [unit][column][32] complex (parent.cu).
 struct PfGroup {
   int ncell, nact, nitem;
   int cell_off, row_off, item_off;
   int level;  // octree level (kernel spectra)
+  int nquad;  // quads, in the first 2 nquad items
 };
 constexpr int kPfItem = 40;  // uint16 per item: five 16-byte vectors
 constexpr int kPfMacThreads = 256;

@@ -275,7 +275,12 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 // kernel values in registers: the pair's 36 distinct source values feed 54
 // products (shared-memory bandwidth bounds the kernel with 27 reads each, and
 // longer runs lost more to their short parts than they saved: 20 sparse
-// problems 7.6 ms with single parents, 8.2 ms with runs).  The sums are
+// problems 7.6 ms with single parents, 8.2 ms with runs).  FP32 joins two pairs
+// that are neighbours along axis 1 where both exist: 48 reads for 108 products
+// and a third fewer table entries to unpack (ncu on pairs: L1 72 %, issue slots
+// 64 %, the ALU pipe 31 %, all of it unpacking); whole solves, 16^3 blocks of
+// 16^3 1.487 -> 1.438 ms, three-level torus 4.33 -> 4.27 ms, two-level vector
+// torus 2.13 -> 2.09 ms.  The sums are
 // transformed back (a thread per line) and the two parities added.
 // FP64 products take the three-multiplication form (kr (fr + fi), (kr + ki)
 // fi, (ki - kr) fr) with fr + fi kept beside the sources, and skip absent cells
@@ -399,7 +404,40 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
     };
     const C2* Xl = X + lane;
     const R* Sl = Sm + lane;
-    for (int it = warp; it < gp.nitem; it += NW) {
+    int it0 = warp;
+    if constexpr (!G3) {
+      for (int iq = warp; iq < gp.nquad; iq += NW) {
+        const uint4* I = IT + 2 * iq * (kPfItem / 8);
+        const uint4 meta = I[6];
+        R a[4][NA];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int t = 0; t < NA; ++t) a[i][t] = R(0);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          if (!(meta.y >> r & 1)) continue;  // no sources at this e0 (uniform)
+          const uint4 v0 = I[2 * r], v1 = I[2 * r + 1];
+          const uint32_t w[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const C2 f = Xl[(i & 1) ? w[i / 2] >> 16 : w[i / 2] & 0xFFFFu];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const int e1 = i / 4 - m / 2, e2 = i % 4 - m % 2;
+              if (e1 >= 0 && e1 < 3 && e2 >= 0 && e2 < 3) product(a[m], 9 * r + 3 * e1 + e2, f, R(0));
+            }
+          }
+        }
+        const int m0 = meta.x & 0xFFFF, m1 = meta.x >> 16;
+        Tp[m0 * kPfStride] = result(a[0]);
+        Tp[(m0 + 1) * kPfStride] = result(a[1]);
+        Tp[m1 * kPfStride] = result(a[2]);
+        Tp[(m1 + 1) * kPfStride] = result(a[3]);
+      }
+      it0 = 2 * gp.nquad + (warp + NW - gp.nquad % NW) % NW;  // the warps go on in turn
+    }
+    for (int it = it0; it < gp.nitem; it += NW) {
       uint32_t w[kPfItem / 2];
 #pragma unroll
       for (int q = 0; q < kPfItem / 8; ++q) {
@@ -411,7 +449,7 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
       R a[2][NA];
 #pragma unroll
       for (int t = 0; t < NA; ++t) a[0][t] = a[1][t] = R(0);
-      // both forms take a parent's 27 products in the same order
+      // all forms take a parent's 27 products in the same order
       if (entry(37) == 2) {
 #pragma unroll
         for (int r = 0; r < 3; ++r) {

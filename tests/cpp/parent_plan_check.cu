@@ -104,7 +104,24 @@ int main(int argc, char** argv) {
              pg.level != g.level ||
              g.nact > ph.pf_lim.parents || g.ncell > ph.pf_lim.cells || pg.nitem > ph.pf_lim.items;
       std::vector<int> seen(g.nact, 0);
-      for (int i = 0; i < pg.nitem; ++i) {
+      bad += pg.nquad < 0 || 2 * pg.nquad > pg.nitem;
+      for (int i = 0; i < pg.nquad; ++i) {  // quads: two pairs, the second one up along axis 1
+        const uint16_t* it = items + (size_t)(pg.item_off + 2 * i) * kPfItem;
+        for (int a = 0; a < 4; ++a) {
+          const int m = it[48 + a / 2] + a % 2;
+          if (m >= g.nact) { ++bad; continue; }
+          seen[m]++;
+          const uint16_t* row = rows + (size_t)(g.row_off + m) * kFlRowStride;
+          int want_cell[27];
+          std::fill(want_cell, want_cell + 27, g.ncell);
+          for (int j = 0; j < row[0]; ++j) want_cell[row[1 + j] >> 11] = row[1 + j] & 0x7FF;
+          for (int e = 0; e < 27; ++e) {
+            bad += it[16 * (e / 9) + 4 * ((e / 3) % 3 + a / 2) + e % 3 + a % 2] != 33 * want_cell[e];
+            bad += want_cell[e] != g.ncell && !((it[50] >> (e / 9)) & 1);
+          }
+        }
+      }
+      for (int i = 2 * pg.nquad; i < pg.nitem; ++i) {
         const uint16_t* it = items + (size_t)(pg.item_off + i) * kPfItem;
         if (it[37] < 1 || it[37] > 2 || it[36] + it[37] > g.nact) { ++bad; continue; }
         for (int p = 0; p < it[37]; ++p) {
