@@ -1417,7 +1417,7 @@ static int blockset_create(flgf_ctx* ctx, int n_problems, const int* n_levels, c
   if (e == cudaSuccess) e = alloc(&bs->spec, 2 * rs * NW * bs->max_phase_blocks);
   if (e == cudaSuccess) e = alloc(&bs->acc, 2 * rs * NW * bs->max_phase_blocks);
   const auto pf = pf_need(bs->ph);
-  if (e == cudaSuccess) e = alloc(&bs->pf_src, 2 * rs * pf_parent_values(N) * pf.first);
+  if (e == cudaSuccess) e = alloc(&bs->pf_src, 2 * rs * pf_source_values(N, rs == 8) * pf.first);
   if (e == cudaSuccess) e = alloc(&bs->pf_dst, 2 * rs * pf_parent_values(N) * pf.second);
   if (e == cudaSuccess) e = alloc(&bs->lap_in, rs * N3 * bs->max_level_blocks);
   if (e == cudaSuccess) e = alloc(&bs->lap_out, rs * N3 * bs->max_level_blocks);
@@ -1597,7 +1597,7 @@ static int build_adjoint(flgf_blockset* bs) {
   if (e == cudaSuccess) e = alloc(&bs->aunodes, rs * N3 * bs->G);
   const auto have = pf_need(bs->ph), need = pf_need(bs->aph);
   const size_t pv = 2 * rs * pf_parent_values(ctx->N);
-  if (e == cudaSuccess && need.first > have.first) e = alloc(&bs->apf_src, pv * need.first);
+  if (e == cudaSuccess && need.first > have.first) e = alloc(&bs->apf_src, 2 * rs * pf_source_values(ctx->N, rs == 8) * need.first);
   if (e == cudaSuccess && need.second > have.second) e = alloc(&bs->apf_dst, pv * need.second);
   if (e == cudaSuccess) e = cudaMemset(bs->gseed, 0, rs * N3 * bs->B);
   if (e != cudaSuccess) {
@@ -1728,6 +1728,7 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
     StageScope sc(bs, 2);
     KRUN(ph.n_fwd, launch_fft_forward<R>(N, nodes, ar.at<int>(ph.fwd_gid), ar.at<int>(ph.fwd_sid), ph.n_fwd, bs->spec,
                                          ph.nblocks, s));
+    if (sizeof(R) == 8 && ph.n_pfs > 0) bs->launches++;  // two kernels
     KRUN(ph.n_pfs, launch_pf_forward<R>(N, nodes, ar.at<int>(ph.pf_sch), ph.n_pfs, pf_src, s));
   }
   {

@@ -33,7 +33,7 @@ using namespace flgf;
 constexpr int kStaticMaxBlocks = 32;
 constexpr size_t kSpecBytes = (size_t)kStaticMaxBlocks * nfreq(16) * 16;  // half-transformed spectra of 8 parents (complex double, N = 16: 8.65 MB)
 constexpr size_t kListBytes = 512 * 1024;
-constexpr size_t kScratchBytes = 2 * kSpecBytes + kListBytes;             // ~18.3 MB
+constexpr size_t kScratchBytes = 3 * kSpecBytes + kListBytes;             // sources (FP64: two halves) and targets, ~27.3 MB
 
 // Shared by every call on a device; see the header for the concurrency rule.
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -152,8 +152,8 @@ extern "C" int flgf_convolve_static(flgf_ctx* ctx, int nblk, const int32_t* coor
   if (e != cudaSuccess) return bad(FLGF_ECUDA, cudaGetErrorString(e));
   unsigned char* sp = static_cast<unsigned char*>(base);
   void* spec = sp;
-  void* acc = sp + kSpecBytes;
-  unsigned char* dl = sp + 2 * kSpecBytes;
+  void* acc = sp + 2 * kSpecBytes;
+  unsigned char* dl = sp + 3 * kSpecBytes;
   cudaStream_t s = cv.stream;
   // the lists travel as kernel parameters, written into the scratch on the stream
   static_lists_kernel<<<1, 256, 0, s>>>(L, reinterpret_cast<int*>(dl));

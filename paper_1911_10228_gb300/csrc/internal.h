@@ -254,7 +254,8 @@ template <typename R>
 constexpr size_t pf_smem_bytes(const PfLimits& l, int upc) {
   return pf_table_offset<R>(l, upc) + (size_t)l.items * kPfItem * 2 + (size_t)(l.cells + l.parents) * 4;
 }
-size_t pf_parent_values(int N);  // complex values of one parent's half-transformed spectrum
+size_t pf_parent_values(int N);  // complex values of one target parent's half-transformed spectrum
+size_t pf_source_values(int N, bool fp64);  // complex values of one source parent's spectrum in memory
 size_t pf_kernel_values(int N);  // complex values of the 27 parent kernel spectra
 size_t pf_setup_bytes(int N);    // scratch of launch_pf_setup
 // Parent kernel arrays of octree level k (FP64, lgf.cu) for the 8 offsets

@@ -22,7 +22,8 @@
 // The transform along axis 0 is fused with the products, so HBM only holds
 // spectra of the two transformed axes, half as long as padded ones:
 //   pf_forward_kernel   planes z of a source parent: axis 2, axis 1
-//   pf_mac_kernel       axis 0 forward, products, axis 0 inverse
+//   pf_axis0_kernel     FP64: axis 0 forward, into fully padded spectra
+//   pf_mac_kernel       axis 0 forward (FP32), products, axis 0 inverse
 //   pf_inverse_kernel   planes z of a target parent: axis 1, axis 2
 // Layout between them: lines l = k1 (H + 1) + k2 (P (H + 1) of them); a unit
 // is the 32 / H lines that fill a warp, stored [unit][parent][32] with lane
@@ -98,6 +99,9 @@ constexpr int pf_plane_stride() {
 }
 
 constexpr int kPfPlaneThreads = 288;
+// Halves of a source parent's spectrum in memory: FP64 both parities of the
+// transformed axis 0, FP32 the planes.
+template <typename R> constexpr int pf_halves() { return sizeof(R) == 8 ? 2 : 1; }
 
 // ---------------------------------------------------------------------------
 // Axes 2 and 1 of ZP planes of a source parent.  Axis 2 transforms the real
@@ -157,12 +161,58 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll
     for (int m = 0; m < H; ++m) {
       const int l = (2 * m + par) * NX + kx;
-      out[((size_t)(l / D::S) * ncol + col) * 32 + (l % D::S) * H + z0 + zl] = C2{xr[m], xi[m]};
+      out[((size_t)(l / D::S) * pf_halves<R>() * ncol + col) * 32 + (l % D::S) * H + z0 + zl] = C2{xr[m], xi[m]};
     }
   };
   for (int i = threadIdx.x; i < 2 * ZP * NX; i += kPfPlaneThreads) {
     if (i < ZP * NX) columns(std::integral_constant<int, 0>{}, i);
     else columns(std::integral_constant<int, 1>{}, i - ZP * NX);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// FP64: axis 0 of every source parent, once, into the two parities' halves of
+// its fully padded spectrum ([unit][parity][parent][32], the planes in parity
+// 0's place).  Fused with the products, as in FP32, a parent's lines would be
+// transformed by every group that reads them (up to three times), and the FP64
+// pipe bounds it; the doubled spectra cost less.  A thread per line, rows
+// staged through shared memory; 64 threads leave three CTAs an SM.
+// Whole solves: 11 x 9 x 13 blocks of 16^3 12.7 -> 11.1 ms, three-level torus
+// of 8^3 blocks 7.44 -> 7.02 ms.
+// ---------------------------------------------------------------------------
+constexpr int kPfAxisThreads = 64;
+template <typename R, int N>
+__global__ void __launch_bounds__(kPfAxisThreads) pf_axis0_kernel(typename Vec2<R>::type* __restrict__ spec, int ncol) {
+  using D = PfDims<N>;
+  using C2 = typename Vec2<R>::type;
+  constexpr int H = D::H, RC = kPfAxisThreads / D::S;  // parents per CTA
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C2* A = reinterpret_cast<C2*>(smem_raw);  // [RC][33] planes, then the odd half
+  C2* B = A + RC * kPfStride;               // [RC][33] the even half
+  const int nch = (ncol + RC - 1) / RC, unit = blockIdx.x / nch, c0 = blockIdx.x % nch * RC, n = min(RC, ncol - c0);
+  C2* even = spec + ((size_t)unit * 2 * ncol + c0) * 32;
+  C2* odd = even + (size_t)ncol * 32;
+  for (int i = threadIdx.x; i < n * 32; i += kPfAxisThreads) A[(i / 32) * kPfStride + i % 32] = even[i];
+  __syncthreads();
+  if (threadIdx.x < n * D::S) {
+    const int off = (threadIdx.x / D::S) * kPfStride + (threadIdx.x % D::S) * H;
+    auto half = [&](auto parity, C2* out) {
+      constexpr int par = decltype(parity)::value;
+      R xr[H], xi[H];
+#pragma unroll
+      for (int z = 0; z < H; ++z) { const C2 v = A[off + z]; xr[z] = v.x; xi[z] = v.y; }
+      LineFFT<H, -1, R, par == 1>::run(xr, xi);
+#pragma unroll
+      for (int k = 0; k < H; ++k) out[off + k] = C2{xr[k], xi[k]};
+    };
+    half(std::integral_constant<int, 0>{}, B);
+    half_barrier();
+    half(std::integral_constant<int, 1>{}, A);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n * 32; i += kPfAxisThreads) {
+    even[i] = B[(i / 32) * kPfStride + i % 32];
+    odd[i] = A[(i / 32) * kPfStride + i % 32];
   }
 }
 
@@ -269,8 +319,9 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 // ---------------------------------------------------------------------------
 // Axis 0 and the products.  A CTA takes a group of target parents (consecutive
 // in tile order, so they share neighbour cells) and upc units of lines (one,
-// unless the groups are small: mac_units); lane = (line, k0).  Per parity of k0 the group's source lines are copied to shared
-// memory and transformed in place (a thread per line); a warp then takes two
+// unless the groups are small: mac_units); lane = (line, k0).  Per parity of k0
+// the group's source lines are copied to shared memory and, in FP32,
+// transformed in place (a thread per line); a warp then takes two
 // parents that are neighbours along axis 2 (or one) at a time, its lane's 27
 // kernel values in registers: the pair's 36 distinct source values feed 54
 // products (shared-memory bandwidth bounds the kernel with 27 reads each, and
@@ -323,11 +374,12 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
     if constexpr (G3) Sm[(size_t)nc * kPfStride + lane] = R(0);
   }
   __syncthreads();
-  const C2* sbase = src + (size_t)unit * nsrc * 32 + lane;
-  auto fill = [&]() {
-    for (int c = warp; c < nc; c += NW) cp_async_complex<R>(X + c * kPfStride + lane, sbase + (size_t)CC[c] * 32);
+  const C2* sbase = src + (size_t)unit * pf_halves<R>() * nsrc * 32 + lane;
+  auto fill = [&](int par) {
+    const C2* sp = sbase + (G3 ? (size_t)par * nsrc * 32 : 0);
+    for (int c = warp; c < nc; c += NW) cp_async_complex<R>(X + c * kPfStride + lane, sp + (size_t)CC[c] * 32);
   };
-  fill();
+  fill(0);
   for (int i = tid; i < nt; i += kPfMacThreads) TC[i] = __ldg(tgt_col + gp.row_off + i) + (int)blockIdx.y * dst_stride;
   for (int i = tid; i < gp.nitem * (kPfItem / 8); i += kPfMacThreads)
     IT[i] = __ldg(reinterpret_cast<const uint4*>(items) + (size_t)gp.item_off * (kPfItem / 8) + i);
@@ -354,23 +406,26 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
 #pragma unroll 1
   for (int par = 0; par < 2; ++par) {
     cp_async_wait();
-    __syncthreads();
-    for (int i = tid; i < upc * nc * D::S; i += kPfMacThreads) {
-      const int j = kOne && D::S == 1 ? 0 : i / nc, c = i - j * nc;
-      C2* line = X0 + (j / D::S) * xs + c * kPfStride + (j % D::S) * H;
-      R xr[H], xi[H];
+    if constexpr (G3) {
+      // the values that this thread copied
+      for (int c = warp; c < nc; c += NW) {
+        const C2 v = X[c * kPfStride + lane];
+        Sm[c * kPfStride + lane] = v.x + v.y;
+      }
+    } else {
+      __syncthreads();
+      for (int i = tid; i < upc * nc * D::S; i += kPfMacThreads) {
+        const int j = kOne && D::S == 1 ? 0 : i / nc, c = i - j * nc;
+        C2* line = X0 + (j / D::S) * xs + c * kPfStride + (j % D::S) * H;
+        R xr[H], xi[H];
 #pragma unroll
-      for (int z = 0; z < H; ++z) { const C2 v = line[z]; xr[z] = v.x; xi[z] = v.y; }
-      if (par)
-        LineFFT<H, -1, R, true>::run(xr, xi);
-      else
-        LineFFT<H, -1, R>::run(xr, xi);
+        for (int z = 0; z < H; ++z) { const C2 v = line[z]; xr[z] = v.x; xi[z] = v.y; }
+        if (par)
+          LineFFT<H, -1, R, true>::run(xr, xi);
+        else
+          LineFFT<H, -1, R>::run(xr, xi);
 #pragma unroll
-      for (int k = 0; k < H; ++k) line[k] = C2{xr[k], xi[k]};
-      if constexpr (G3) {
-        R* sl = S0 + (line - X0);
-#pragma unroll
-        for (int k = 0; k < H; ++k) sl[k] = xr[k] + xi[k];
+        for (int k = 0; k < H; ++k) line[k] = C2{xr[k], xi[k]};
       }
     }
     R k0[27], k1[27], k2[G3 ? 27 : 1];
@@ -484,7 +539,7 @@ __global__ void __launch_bounds__(kPfMacThreads, sizeof(R) == 4 ? 2 : 1)
       Tp[m0 * kPfStride] = result(a[0]);
     }
     __syncthreads();
-    if (par == 0) fill();  // the second parity's copy of the sources
+    if (par == 0) fill(1);  // the second parity's copy of the sources
     if (!kBoth || par == 1) {
       inverse(par);
       __syncthreads();
@@ -590,6 +645,7 @@ static cudaError_t setup_spectra(const double* karr, void* tmp, void* kspec, cud
 size_t pf_kernel_values(int N) { return (size_t)4 * N * (2 * N + 1) * 2 * N * 2 * 27; }
 size_t pf_setup_bytes(int N) { return (size_t)2 * 16 * 8 * 4 * N * 4 * N * (2 * N + 1); }
 size_t pf_parent_values(int N) { return (size_t)4 * N * (2 * N + 1) * 2 * N; }
+size_t pf_source_values(int N, bool fp64) { return pf_parent_values(N) * (fp64 ? pf_halves<double>() : pf_halves<float>()); }
 
 template <typename R>
 cudaError_t launch_pf_setup(int N, const double* karr, void* tmp, void* kspec, cudaStream_t s) {
@@ -609,7 +665,16 @@ static cudaError_t forward_n(const R* nodes, const int* cell_ch, int n, void* ou
   auto k = pf_forward_kernel<R, N, ZP>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
   if (e != cudaSuccess) return e;
-  k<<<n * (PfDims<N>::H / ZP), kPfPlaneThreads, sm, s>>>(nodes, cell_ch, reinterpret_cast<typename Vec2<R>::type*>(out), ncol);
+  using C2 = typename Vec2<R>::type;
+  k<<<n * (PfDims<N>::H / ZP), kPfPlaneThreads, sm, s>>>(nodes, cell_ch, reinterpret_cast<C2*>(out), ncol);
+  if constexpr (pf_halves<R>() == 2) {
+    constexpr int RC = kPfAxisThreads / PfDims<N>::S, sa = 2 * RC * kPfStride * (int)sizeof(C2);
+    const long long ctas = (long long)PfDims<N>::U * ((ncol + RC - 1) / RC);
+    if (ctas >= (1ll << 31)) return cudaErrorInvalidConfiguration;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(pf_axis0_kernel<R, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sa)) != cudaSuccess) return e;
+    pf_axis0_kernel<R, N><<<(unsigned)ctas, kPfAxisThreads, sa, s>>>(reinterpret_cast<C2*>(out), ncol);
+  }
   return cudaGetLastError();
 }
 template <typename R, int N>
