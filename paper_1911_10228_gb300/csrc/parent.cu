@@ -19,15 +19,17 @@
 // ms, three-level torus of 8^3 blocks 4.0 -> 1.0 ms.  FP32 keeps the child-pair
 // kernels there: their spectra go through float-float inverse transforms.
 //
-// The transform along axis 0 is fused with the products, so HBM only holds
-// spectra of the two transformed axes, half as long as padded ones:
+// The transform along axis 0 is fused with the products (FP64: only the
+// inverse), so HBM only holds spectra of the two transformed axes, half as long
+// as padded ones:
 //   pf_forward_kernel   planes z of a source parent: axis 2, axis 1
 //   pf_axis0_kernel     FP64: axis 0 forward, into fully padded spectra
 //   pf_mac_kernel       axis 0 forward (FP32), products, axis 0 inverse
 //   pf_inverse_kernel   planes z of a target parent: axis 1, axis 2
 // Layout between them: lines l = k1 (H + 1) + k2 (P (H + 1) of them); a unit
-// is the 32 / H lines that fill a warp, stored [unit][parent][32] with lane
-// (l % (32 / H)) H + z, so the product kernel reads 256-byte (FP32) rows.
+// is the 32 / H lines that fill a warp, stored [unit][parent][32] (FP64
+// sources: [unit][parity][parent][32]) with lane (l % (32 / H)) H + z, so the
+// product kernel reads 256-byte (FP32) or 512-byte rows.
 //
 // The axis-0 transform is pruned by parity: the even (odd) outputs are the
 // H-point transform of the H inputs (times w^z), and the kept inverse outputs
