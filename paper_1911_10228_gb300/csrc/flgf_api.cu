@@ -45,6 +45,8 @@ struct flgf_ctx {
   // block: FP64 (the FP32 child-pair kernels stay: their spectra go through the
   // float-float inverse transforms of FLGF_OPT_COMPENSATED)
   bool parent_form_coarse() const { return prec == FLGF_FP64; }
+  // bytes of the parents' spectra that a phase may always take at once (build_fmm)
+  size_t pf_bytes = (size_t)256 << 20;
 };
 
 namespace {
@@ -158,8 +160,15 @@ struct Problem {
   std::vector<LevelInfo> lev;
 };
 
+// Groups between parents that run together: their source and target parents
+// (all components' of a vector block set) share the spectrum buffers at once.
+struct PfPass {
+  int g0 = 0, ng = 0, s0 = 0, ns = 0, t0 = 0, nt = 0;
+};
+
 struct PhaseOff {  // arena offsets and counts of one phase's launch lists
   int gid_begin = 0, nblocks = 0;
+  int ncol = 0;  // spectrum columns: blocks that the block-wise transforms read or write (number_columns)
   int n_prep = 0; size_t prep_src = 0, prep_dst = 0, prep_zero = 0;
   std::vector<int> n_ant; std::vector<size_t> ant_par, ant_ch;
   int n_fwd = 0; size_t fwd_gid = 0, fwd_sid = 0;
@@ -175,6 +184,7 @@ struct PhaseOff {  // arena offsets and counts of one phase's launch lists
   // the source and target parents (one component's; the others follow in order)
   int n_pf = 0, n_pfs = 0, n_pft = 0, pf_src_stride = 0, pf_tgt_stride = 0;
   PfLimits pf_lim;
+  std::vector<PfPass> pf_pass;
   size_t pf_groups = 0, pf_items = 0, pf_ccol = 0, pf_tcol = 0, pf_sch = 0, pf_tch = 0, pf_scale = 0;
   int n_fll = 0; size_t fll_groups = 0, fll_tgt = 0, fll_beg = 0, fll_len = 0, fll_ent = 0;
   // finest octree level first (n_inv0); the last n_inv_add add to what the parents' inverse wrote
@@ -222,12 +232,12 @@ struct flgf_blockset {
   void* gtmp = nullptr;    // [B][N^3]
   void* aunodes = nullptr; // FMM outputs of the adjoint, [G][N^3] (the potentials stay in unodes)
   bool adj_solved = false;
+  // source spectra and sums of a phase: of its parents (parent.cu), then, once
+  // their potentials are written, of the blocks with spectra of their own
   void* spec = nullptr;
   void* acc = nullptr;
-  void* pf_src = nullptr;  // half-transformed spectra of the source and target parents of a phase
-  void* pf_dst = nullptr;
-  void* apf_src = nullptr;  // the adjoint's, where its phases need more room than pf_src / pf_dst have
-  void* apf_dst = nullptr;
+  void* aspec = nullptr;  // the adjoint's, where its phases need more room than spec / acc have
+  void* aacc = nullptr;
   void* lap_in = nullptr;
   void* lap_out = nullptr;
   int* d_err = nullptr;
@@ -469,10 +479,8 @@ extern "C" void flgf_blockset_destroy(flgf_blockset* bs) {
   cudaFree(bs->aunodes);
   cudaFree(bs->spec);
   cudaFree(bs->acc);
-  cudaFree(bs->pf_src);
-  cudaFree(bs->pf_dst);
-  cudaFree(bs->apf_src);
-  cudaFree(bs->apf_dst);
+  cudaFree(bs->aspec);
+  cudaFree(bs->aacc);
   cudaFree(bs->lap_in);
   cudaFree(bs->lap_out);
   cudaFree(bs->d_err);
@@ -855,17 +863,44 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   if (ph.n_pf > 0) {
     std::vector<double> scale_of(ph.nblocks, 0.0);
     for (const Tgt& t : tgt0) scale_of[t.gid - ph.gid_begin] = t.scale;
-    std::unordered_map<int, int> col_of;  // first source child of a parent -> its column
+    std::unordered_map<int, int> col_of;  // first source child of a parent -> its column in the pass
     std::vector<int> ccol, tcol, sch, tch;
     std::vector<double> pscale;
     std::vector<PfGroup> pgroups;
     std::vector<uint16_t> items;  // [items][kPfItem]
+    // The groups run in passes whose parents' spectra and sums take no more
+    // than a spectrum and a sum for every block would (or pf_bytes).  Parents
+    // with few blocks need several: their spectra are as large as full ones.
+    // A parent whose neighbours are in two passes is transformed in both.
+    // (A vector block set takes one pass.)
+    const bool f64 = ctx->prec == FLGF_FP64;
+    const size_t csz = f64 ? 16 : 8, src_bytes = csz * pf_source_values(N, f64), dst_bytes = csz * pf_parent_values(N);
+    const size_t most = vcomp > 1 ? SIZE_MAX : std::max(ctx->pf_bytes, 2 * csz * nfreq(N) * bs->max_phase_blocks);
+    auto cell_key = [&](const int* ch) {
+      int key = -1;
+      for (int b = 0; b < 8 && key < 0; ++b) key = ch[b];
+      return key;
+    };
+    ph.pf_pass.push_back(PfPass());
     for (int gi = 0; gi < ph.n_pf; ++gi) {
       const FlGroup& g = fll.groups[gi];
+      {
+        const PfPass& q = ph.pf_pass.back();
+        size_t ns = q.ns;
+        for (int c = 0; c < g.ncell; ++c) ns += !col_of.count(cell_key(&fll.cells[(size_t)(g.cell_off + c) * 8]));
+        if (q.ng > 0 && ns * src_bytes + (size_t)(q.nt + g.nact) * dst_bytes > most) {
+          PfPass n;
+          n.g0 = gi;
+          n.s0 = q.s0 + q.ns;
+          n.t0 = q.t0 + q.nt;
+          ph.pf_pass.push_back(n);
+          col_of.clear();
+        }
+      }
+      PfPass& ps = ph.pf_pass.back();
       for (int c = 0; c < g.ncell; ++c) {
         const int* ch = &fll.cells[(size_t)(g.cell_off + c) * 8];
-        int key = -1;
-        for (int b = 0; b < 8 && key < 0; ++b) key = ch[b];
+        const int key = cell_key(ch);
         const auto it = col_of.emplace(key, (int)col_of.size());
         if (it.second)
           for (int b = 0; b < 8; ++b) sch.push_back(ch[b] < 0 ? -1 : ch[b] + ph.gid_begin);
@@ -874,13 +909,16 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
       for (int m = 0; m < g.nact; ++m) {
         const int* t = &fll.tgt_ids[(size_t)(g.row_off + m) * 8];
         double sc = 0.0;
-        tcol.push_back((int)pscale.size());
+        tcol.push_back((int)pscale.size() - ps.t0);
         for (int b = 0; b < 8; ++b) {
           tch.push_back(t[b] < 0 ? -1 : t[b] + ph.gid_begin);
           if (t[b] >= 0) sc = scale_of[t[b]];
         }
         pscale.push_back(sc);
       }
+      ++ps.ng;
+      ps.ns = (int)col_of.size();
+      ps.nt += g.nact;
       PfGroup pg{g.ncell, g.nact, 0, g.cell_off, g.row_off, (int)(items.size() / kPfItem), g.level, 0};
       // quads first, then pairs and single parents, so the warps' round-robin ends together
       auto add_item = [&](int m, int n) {
@@ -957,6 +995,10 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     }
     ph.n_pfs = (int)sch.size() / 8;
     ph.n_pft = (int)tch.size() / 8;
+    if (vcomp > 1) {  // one pass, of every component's parents
+      ph.pf_pass[0].ns = ph.n_pfs;
+      ph.pf_pass[0].nt = ph.n_pft;
+    }
     ph.pf_groups = ar.add(pgroups);
     ph.pf_items = ar.add(items);
     ph.pf_ccol = ar.add(ccol);
@@ -1101,6 +1143,12 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   ph.l_len = ar.add(l_len);
   ph.l_ent = ar.add(l_ent);
   ph.l_src = ar.add(l_src);
+  {
+    std::vector<uint8_t> used(ph.nblocks, 0);
+    for (int i : fwd_sid) used[i] = 1;
+    for (int i : inv_sid) used[i] = 1;
+    ph.ncol = (int)std::count(used.begin(), used.end(), 1);
+  }
   ph.n_inv = (int)inv_gid.size();
   ph.inv_sid = ar.add(inv_sid);
   ph.inv_gid = ar.add(inv_gid);
@@ -1366,14 +1414,77 @@ static int plan_blockset(flgf_ctx* ctx, flgf_blockset* bs, int n_problems, const
   return FLGF_OK;
 }
 
-// Most source and target parents of a phase (parent.cu).
-static std::pair<size_t, size_t> pf_need(const std::vector<PhaseOff>& phases) {
+// Bytes of the largest source spectra and of the largest sums that are held at
+// once: of the parents of a pass or the blocks with spectra of their own, one
+// after the other in the same buffers.
+static std::pair<size_t, size_t> spectra_need(const flgf_ctx* ctx, const std::vector<PhaseOff>& phases) {
+  const bool f64 = ctx->prec == FLGF_FP64;
+  const size_t csz = f64 ? 16 : 8;
   std::pair<size_t, size_t> n{0, 0};
   for (const PhaseOff& ph : phases) {
-    n.first = std::max(n.first, (size_t)ph.n_pfs);
-    n.second = std::max(n.second, (size_t)ph.n_pft);
+    const size_t blocks = csz * nfreq(ctx->N) * ph.ncol;
+    n.first = std::max(n.first, blocks);
+    n.second = std::max(n.second, blocks);
+    for (const PfPass& q : ph.pf_pass) {
+      n.first = std::max(n.first, csz * pf_source_values(ctx->N, f64) * q.ns);
+      n.second = std::max(n.second, csz * pf_parent_values(ctx->N) * q.nt);
+    }
   }
   return n;
+}
+
+// The launch lists of a phase name blocks by their phase-local ids; most blocks
+// have no spectrum of their own (dense tiles between parents), so on the device
+// the lists name spectrum columns instead: the blocks that are transformed, in
+// the order of their ids.  Replaces the ids in img, a copy of the arena.  (The
+// components of a vector block set hold the same blocks, so their columns keep
+// a fixed distance, ncol / components.)
+static void number_columns(const PhaseOff& ph, char* img) {
+  auto ints = [&](size_t off) { return reinterpret_cast<int*>(img + off); };
+  std::vector<int> col(ph.nblocks, -1);
+  for (int i = 0; i < ph.n_fwd; ++i) col[ints(ph.fwd_sid)[i]] = 0;
+  for (int i = 0; i < ph.n_inv; ++i) col[ints(ph.inv_sid)[i]] = 0;
+  int n = 0;
+  for (int& c : col)
+    if (c >= 0) c = n++;
+  auto number = [&](int* p, size_t count) {
+    for (size_t i = 0; i < count; ++i)
+      if (p[i] >= 0) p[i] = col[p[i]];
+  };
+  number(ints(ph.fwd_sid), ph.n_fwd);
+  number(ints(ph.inv_sid), ph.n_inv);
+  const HadGroup* hg = reinterpret_cast<const HadGroup*>(img + ph.hgroups);
+  for (int g = 0; g < ph.n_groups_dense; ++g) {
+    number(ints(ph.src_ids) + hg[g].src_off, (size_t)8 * hg[g].ncell);
+    number(ints(ph.tgt_ids) + hg[g].tgt_off, (size_t)8 * hg[g].nact);
+  }
+  const FlGroup* fg = reinterpret_cast<const FlGroup*>(img + ph.fl_groups);
+  for (int g = ph.n_pf; g < ph.n_fl; ++g) {
+    number(ints(ph.fl_cells) + (size_t)8 * fg[g].cell_off, (size_t)8 * fg[g].ncell);
+    number(ints(ph.fl_tgt) + (size_t)8 * fg[g].row_off, (size_t)8 * fg[g].nact);
+  }
+  const FllGroup* qg = reinterpret_cast<const FllGroup*>(img + ph.fll_groups);
+  uint32_t* ent = reinterpret_cast<uint32_t*>(img + ph.fll_ent);
+  for (int g = 0; g < ph.n_fll; ++g)
+    for (int t = qg[g].tgt_off; t < qg[g].tgt_off + qg[g].ntgt; ++t) {
+      number(ints(ph.fll_tgt) + t, 1);
+      for (int j = ints(ph.fll_beg)[t], e = j + ints(ph.fll_len)[t]; j < e; ++j)
+        ent[j] = (uint32_t)col[ent[j] >> 9] << 9 | (ent[j] & 511u);
+    }
+  const ListGroup* lg = reinterpret_cast<const ListGroup*>(img + ph.groups);
+  for (int g = 0; g < ph.n_groups + ph.n_groups_out; ++g) {
+    number(ints(ph.l_tgt) + lg[g].tgt_off, lg[g].ntgt);
+    number(ints(ph.l_src) + lg[g].src_off, lg[g].nsrc);
+  }
+}
+
+// An arena to the device, its lists with spectrum columns.
+static cudaError_t upload(flgf_ctx* ctx, Arena& ar, const std::vector<PhaseOff>& phases) {
+  cudaError_t e = dev_alloc(ctx, (void**)&ar.dev, ar.host.size());
+  if (e != cudaSuccess) return e;
+  std::vector<char> img = ar.host;
+  for (const PhaseOff& ph : phases) number_columns(ph, img.data());
+  return cudaMemcpy(ar.dev, img.data(), img.size(), cudaMemcpyHostToDevice);
 }
 
 static int blockset_create(flgf_ctx* ctx, int n_problems, const int* n_levels, const int* nblk,
@@ -1401,24 +1512,18 @@ static int blockset_create(flgf_ctx* ctx, int n_problems, const int* n_levels, c
       bs->masked |= std::any_of(L.want.begin(), L.want.end(), [](uint8_t v) { return v == 0; });
   const int N = ctx->N;
   const size_t N3 = (size_t)N * N * N;
-  Arena& ar = bs->ar;
   // ---- device memory ---------------------------------------------------------
   const size_t rs = ctx->prec == FLGF_FP64 ? 8 : 4;
-  const size_t NW = (size_t)nfreq(N);
   auto alloc = [&](void** p, size_t bytes) { return dev_alloc(ctx, p, bytes); };
-  cudaError_t e = cudaSuccess;
-  if (e == cudaSuccess) e = alloc((void**)&ar.dev, ar.host.size());
-  if (e == cudaSuccess) e = cudaMemcpy(ar.dev, ar.host.data(), ar.host.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = upload(ctx, bs->ar, bs->ph);
   if (e == cudaSuccess) e = alloc(&bs->nodes, rs * N3 * bs->G);
   if (e == cudaSuccess) e = alloc(&bs->unodes, rs * N3 * bs->G);
   if (e == cudaSuccess) e = alloc(&bs->fuser, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->fwork, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->wfield, rs * N3 * bs->B);
-  if (e == cudaSuccess) e = alloc(&bs->spec, 2 * rs * NW * bs->max_phase_blocks);
-  if (e == cudaSuccess) e = alloc(&bs->acc, 2 * rs * NW * bs->max_phase_blocks);
-  const auto pf = pf_need(bs->ph);
-  if (e == cudaSuccess) e = alloc(&bs->pf_src, 2 * rs * pf_source_values(N, rs == 8) * pf.first);
-  if (e == cudaSuccess) e = alloc(&bs->pf_dst, 2 * rs * pf_parent_values(N) * pf.second);
+  const auto need = spectra_need(ctx, bs->ph);
+  if (e == cudaSuccess) e = alloc(&bs->spec, need.first);
+  if (e == cudaSuccess) e = alloc(&bs->acc, need.second);
   if (e == cudaSuccess) e = alloc(&bs->lap_in, rs * N3 * bs->max_level_blocks);
   if (e == cudaSuccess) e = alloc(&bs->lap_out, rs * N3 * bs->max_level_blocks);
   if (e == cudaSuccess) e = alloc((void**)&bs->d_err, sizeof(int));
@@ -1486,7 +1591,7 @@ static int build_adjoint(flgf_blockset* bs) {
   if (bs->masked) return fail(ctx, FLGF_ESTATE, "the adjoint needs a block set without a target mask");
   const size_t N3 = (size_t)ctx->N * ctx->N * ctx->N;
   // start from nothing, so a call after a failed one (out of memory) rebuilds cleanly
-  for (void** p : {&bs->gseed, &bs->gW, &bs->gf, &bs->gtmp, &bs->aunodes, &bs->apf_src, &bs->apf_dst}) {
+  for (void** p : {&bs->gseed, &bs->gW, &bs->gf, &bs->gtmp, &bs->aunodes, &bs->aspec, &bs->aacc}) {
     cudaFree(*p);
     *p = nullptr;
   }
@@ -1588,17 +1693,15 @@ static int build_adjoint(flgf_blockset* bs) {
   }
   const size_t rs = ctx->prec == FLGF_FP64 ? 8 : 4;
   auto alloc = [&](void** p, size_t bytes) { return dev_alloc(ctx, p, bytes); };
-  cudaError_t e = alloc((void**)&aar.dev, aar.host.size());
-  if (e == cudaSuccess) e = cudaMemcpy(aar.dev, aar.host.data(), aar.host.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = upload(ctx, aar, bs->aph);
   if (e == cudaSuccess) e = alloc(&bs->gseed, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->gW, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->gf, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->gtmp, rs * N3 * bs->B);
   if (e == cudaSuccess) e = alloc(&bs->aunodes, rs * N3 * bs->G);
-  const auto have = pf_need(bs->ph), need = pf_need(bs->aph);
-  const size_t pv = 2 * rs * pf_parent_values(ctx->N);
-  if (e == cudaSuccess && need.first > have.first) e = alloc(&bs->apf_src, 2 * rs * pf_source_values(ctx->N, rs == 8) * need.first);
-  if (e == cudaSuccess && need.second > have.second) e = alloc(&bs->apf_dst, pv * need.second);
+  const auto have = spectra_need(ctx, bs->ph), need = spectra_need(ctx, bs->aph);
+  if (e == cudaSuccess && need.first > have.first) e = alloc(&bs->aspec, need.first);
+  if (e == cudaSuccess && need.second > have.second) e = alloc(&bs->aacc, need.second);
   if (e == cudaSuccess) e = cudaMemset(bs->gseed, 0, rs * N3 * bs->B);
   if (e != cudaSuccess) {
     const int code = (e == cudaErrorMemoryAllocation) ? FLGF_ENOMEM : FLGF_ECUDA;
@@ -1696,10 +1799,11 @@ struct StageScope {
   }
 };
 
-// FMM of one phase: upward pass over `nodes`, forward FFTs, spectrum MAC,
-// inverse FFTs and downward pass into `unodes`.
+// FMM of one phase: upward pass over `nodes`, forward FFTs, spectrum MAC and
+// inverse FFTs between parents, then those between blocks, and the downward pass
+// into `unodes`; spec and acc hold first the parents' spectra, then the blocks'.
 template <typename R>
-cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, R* unodes, void* pf_src, void* pf_dst) {
+cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, R* unodes, void* spec, void* acc) {
   flgf_ctx* c = bs->ctx;
   const int N = c->N;
   cudaStream_t s = c->stream;
@@ -1724,45 +1828,54 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
   // back (inverse FFT) and interpolates in float-float arithmetic; the finest
   // level's inverse FFTs, which nothing amplifies, stay plain FP32.
   const bool comp = bs->compensated;
+  for (const PfPass& q : ph.pf_pass) {
+    {
+      StageScope sc(bs, 2);
+      if (sizeof(R) == 8 && q.ns > 0) bs->launches++;  // two kernels
+      KRUN(q.ns, launch_pf_forward<R>(N, nodes, ar.at<int>(ph.pf_sch) + 8 * (size_t)q.s0, q.ns, spec, s));
+    }
+    {
+      StageScope sc(bs, 3);
+      KRUN(q.ng, launch_pf_mac<R>(N, ar.at<PfGroup>(ph.pf_groups) + q.g0, q.ng, ph.pf_lim, ar.at<uint16_t>(ph.pf_items),
+                                  ar.at<int>(ph.pf_ccol), ar.at<int>(ph.pf_tcol), spec, q.ns, acc, q.nt, c->d_pspec,
+                                  ph.fl_ncomp, ph.pf_src_stride, ph.pf_tgt_stride, s));
+    }
+    {
+      StageScope sc(bs, 4);
+      KRUN(q.nt, launch_pf_inverse<R>(N, acc, ar.at<int>(ph.pf_tch) + 8 * (size_t)q.t0, ar.at<double>(ph.pf_scale) + q.t0,
+                                      q.nt, unodes, s));
+    }
+  }
   {
     StageScope sc(bs, 2);
-    KRUN(ph.n_fwd, launch_fft_forward<R>(N, nodes, ar.at<int>(ph.fwd_gid), ar.at<int>(ph.fwd_sid), ph.n_fwd, bs->spec,
-                                         ph.nblocks, s));
-    if (sizeof(R) == 8 && ph.n_pfs > 0) bs->launches++;  // two kernels
-    KRUN(ph.n_pfs, launch_pf_forward<R>(N, nodes, ar.at<int>(ph.pf_sch), ph.n_pfs, pf_src, s));
+    KRUN(ph.n_fwd, launch_fft_forward<R>(N, nodes, ar.at<int>(ph.fwd_gid), ar.at<int>(ph.fwd_sid), ph.n_fwd, spec,
+                                         ph.ncol, s));
   }
   {
     StageScope sc(bs, 3);
-    KRUN(ph.n_pf, launch_pf_mac<R>(N, ar.at<PfGroup>(ph.pf_groups), ph.n_pf, ph.pf_lim, ar.at<uint16_t>(ph.pf_items),
-                                   ar.at<int>(ph.pf_ccol), ar.at<int>(ph.pf_tcol), pf_src, ph.n_pfs,
-                                   pf_dst, ph.n_pft, c->d_pspec, ph.fl_ncomp, ph.pf_src_stride,
-                                   ph.pf_tgt_stride, s));
     if constexpr (sizeof(R) == 4)
       KRUN(ph.n_work, launch_hadamard<R>(N, ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
-                                       ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
-                                       ar.at<uint16_t>(ph.par_tab), bs->spec, bs->acc, ph.nblocks, c->d_kspec,
-                                       c->kstride, s));
+                                         ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
+                                         ar.at<uint16_t>(ph.par_tab), spec, acc, ph.ncol, c->d_kspec, c->kstride, s));
     const int n_fl = ph.n_fl - ph.n_pf;
     KRUN(n_fl, launch_hadamard_fl(N, ar.at<FlGroup>(ph.fl_groups) + ph.n_pf, n_fl, ph.fl_max_cells, ph.fl_max_parents,
-                                     ar.at<uint16_t>(ph.fl_rows), ar.at<uint32_t>(ph.fl_dlms), ar.at<int>(ph.fl_tgt),
-                                     ar.at<int>(ph.fl_cells), bs->spec, bs->acc, ph.nblocks, c->d_kspec, c->kstride,
-                                     ph.fl_ncomp, ph.fl_cstride, ph.fl_split, s));
+                                  ar.at<uint16_t>(ph.fl_rows), ar.at<uint32_t>(ph.fl_dlms), ar.at<int>(ph.fl_tgt),
+                                  ar.at<int>(ph.fl_cells), spec, acc, ph.ncol, c->d_kspec, c->kstride, ph.fl_ncomp,
+                                  ph.ncol / ph.fl_ncomp, ph.fl_split, s));
     KRUN(ph.n_fll, launch_hadamard_fll(N, ar.at<FllGroup>(ph.fll_groups), ph.n_fll, ar.at<int>(ph.fll_tgt),
                                        ar.at<int>(ph.fll_beg), ar.at<int>(ph.fll_len), ar.at<uint32_t>(ph.fll_ent),
-                                       bs->spec, bs->acc, ph.nblocks, c->d_kspec, c->kstride, s));
+                                       spec, acc, ph.ncol, c->d_kspec, c->kstride, s));
     const int n_lists = ph.n_groups + ph.n_groups_out;
     KRUN(n_lists, launch_hadamard_list<R>(N, ar.at<ListGroup>(ph.groups), n_lists, ph.max_group_src,
-                                              ar.at<int>(ph.l_tgt), ar.at<int>(ph.l_len), ar.at<int>(ph.l_ent),
-                                              ar.at<int>(ph.l_src), bs->spec, bs->acc, ph.nblocks, c->d_kspec,
-                                              c->kstride, s));
+                                          ar.at<int>(ph.l_tgt), ar.at<int>(ph.l_len), ar.at<int>(ph.l_ent),
+                                          ar.at<int>(ph.l_src), spec, acc, ph.ncol, c->d_kspec, c->kstride, s));
   }
   {
     StageScope sc(bs, 4);
-    KRUN(ph.n_pft, launch_pf_inverse<R>(N, pf_dst, ar.at<int>(ph.pf_tch), ar.at<double>(ph.pf_scale), ph.n_pft, unodes, s));
-    KRUN(ph.n_inv0, launch_fft_inverse<R>(N, bs->acc, ph.nblocks, ar.at<int>(ph.inv_sid), ar.at<int>(ph.inv_gid),
+    KRUN(ph.n_inv0, launch_fft_inverse<R>(N, acc, ph.ncol, ar.at<int>(ph.inv_sid), ar.at<int>(ph.inv_gid),
                                           ar.at<double>(ph.inv_scale), ph.n_inv0, 0, unodes, s, false));
     const int nc = ph.n_inv - ph.n_inv0;
-    KRUN(nc, launch_fft_inverse<R>(N, bs->acc, ph.nblocks, ar.at<int>(ph.inv_sid) + ph.n_inv0,
+    KRUN(nc, launch_fft_inverse<R>(N, acc, ph.ncol, ar.at<int>(ph.inv_sid) + ph.n_inv0,
                                    ar.at<int>(ph.inv_gid) + ph.n_inv0, ar.at<double>(ph.inv_scale) + ph.n_inv0, nc,
                                    ph.n_inv_add, unodes, s, comp));
   }
@@ -1816,8 +1929,8 @@ cudaError_t enqueue_adjoint(flgf_blockset* bs) {
       KRUN(ao.n_prep, launch_combine_blocks<R>(N, nodes, aa.at<int>(ao.prep_dst), gseed, aa.at<int>(ao.prep_s1), gW,
                                                aa.at<int>(ao.prep_s2), 0, ao.n_prep, s));
     }
-    if ((e = enqueue_fmm<R>(bs, aa, bs->aph[l], unodes, bs->apf_src ? bs->apf_src : bs->pf_src,
-                            bs->apf_dst ? bs->apf_dst : bs->pf_dst)) != cudaSuccess) return e;
+    if ((e = enqueue_fmm<R>(bs, aa, bs->aph[l], unodes, bs->aspec ? bs->aspec : bs->spec,
+                            bs->aacc ? bs->aacc : bs->acc)) != cudaSuccess) return e;
     {
       StageScope sc(bs, 6);
       KRUN(ao.n_gacc, launch_combine_blocks<R>(N, gf, aa.at<int>(ao.gacc_dst), unodes, aa.at<int>(ao.gacc_s1), unodes,
@@ -1877,7 +1990,7 @@ cudaError_t enqueue_solve(flgf_blockset* bs) {
       KRUN(ph.n_prep, launch_copy_blocks<R>(N, fwork, ar.at<int>(ph.prep_src), nodes, ar.at<int>(ph.prep_dst),
                                             ar.at<uint8_t>(ph.prep_zero), ph.n_prep, s));
     }
-    if ((e = enqueue_fmm<R>(bs, bs->ar, ph, unodes, bs->pf_src, bs->pf_dst)) != cudaSuccess) return e;
+    if ((e = enqueue_fmm<R>(bs, bs->ar, ph, unodes, bs->spec, bs->acc)) != cudaSuccess) return e;
     {
       StageScope sc(bs, 6);
       R* wf = (R*)bs->wfield;
