@@ -99,9 +99,11 @@ void flgf_destroy(flgf_ctx* ctx);
  *                      neighbour parents is 8 x 8 child pairs (absent blocks
  *                      included); where the dense form multiplies whole parents
  *                      (FP64, and the finest octree level in FP32 with
- *                      FLGF_CTX_MAC >= 1), it counts as 32 (FP64) or 16 (FP32),
- *                      and the near pairs that the coarser levels take out of
- *                      it count in full.
+ *                      FLGF_CTX_MAC >= 1), it counts as 32 (FP64) or 16 (FP32)
+ *                      up to the default percentage, growing linearly to 64 at
+ *                      100, and the near pairs that the coarser levels take out
+ *                      of it count in full.  100 lists every tile that is not
+ *                      completely full.
  *   FLGF_CTX_TILE      tile in parents, t0 | t1 << 8 | t2 << 16 with
  *                      1 <= t_a <= 8, t0 t1 t2 <= 128 and
  *                      (t0 + 2)(t1 + 2)(t2 + 2) <= 397; default 4 x 4 x 8.

@@ -21,7 +21,7 @@ using namespace flgf;
 struct flgf_ctx {
   int N = 16, nI = 6, prec = FLGF_FP64, max_oct = 6, R = 100, RA = 600;
   // plan options for block sets created afterwards (flgf_ctx_set_option)
-  int list_pct = 30;             // pair-list MAC below this useful fraction of the dense kernel's work
+  int list_pct = kListPct;       // pair-list MAC below this useful fraction of the dense kernel's work
   int tile[3] = {4, 4, 8};       // dense MAC tile in parents
   bool order_by_list = false;    // dense MAC groups: parents ordered by neighbour set (FLGF_CTX_ORDER)
   int mac = 1;                   // FP32 MAC form (FLGF_CTX_MAC): 1 frequency-lane (dense and lists), 2 frequency-lane
@@ -596,9 +596,9 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     };
     const bool excl = k > 0;
     // products of a neighbour cell in the dense kernel, in units of a child
-    // pair's: 64 of the child-pair kernels; the parent form's cost (8 products
-    // and its share of the parents' transforms) is that of kPfPairs pairs
-    const int per_cell = by_parents(k) ? pf_pairs(ctx->prec == FLGF_FP64) : 64;
+    // pair's: 64 of the child-pair kernels; of the parent form (8 products and its
+    // share of the parents' transforms) pf_pairs
+    const int per_cell = by_parents(k) ? pf_pairs(ctx->prec == FLGF_FP64, list_pct) : 64;
     for (int t0 = lo[0]; t0 <= hi[0]; t0 += TP[0])
       for (int t1 = lo[1]; t1 <= hi[1]; t1 += TP[1])
         for (int t2 = lo[2]; t2 <= hi[2]; t2 += TP[2]) {

@@ -231,7 +231,13 @@ constexpr int kPfItem = 40;  // uint16 per item: five 16-byte vectors
 constexpr int kPfMacThreads = 256;
 // Cost of a neighbour pair of parents, its share of the parents' transforms
 // included, in child pairs of the pair lists (the rule of FLGF_CTX_LIST_PCT).
-constexpr int pf_pairs(bool fp64) { return fp64 ? 32 : 16; }
+// Above the default percentage it grows to a pair's 64 child pairs, so that 100
+// lists every tile that is not completely full, as for the child-pair kernels.
+constexpr int kListPct = 30;
+constexpr int pf_pairs(bool fp64, int list_pct) {
+  const int cost = fp64 ? 32 : 16;
+  return list_pct <= kListPct ? cost : cost + (64 - cost) * (list_pct - kListPct) / (100 - kListPct);
+}
 // Group limits: FP32 two CTAs of at most 113 KB per SM, FP64 one of 227 KB.
 constexpr int pf_max_cells(bool fp64) { return fp64 ? 192 : 256; }
 constexpr int pf_max_parents(bool fp64) { return fp64 ? 64 : 128; }
