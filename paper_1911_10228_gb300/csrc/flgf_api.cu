@@ -243,6 +243,7 @@ struct flgf_blockset {
   int* d_err = nullptr;
   int* h_err = nullptr;       // pinned: where the device flag is read to
   bool err_known = false;     // *h_err is the flag of the last solve (forward or adjoint)
+  bool replayed = false;      // a solve was captured by the caller: replays change the flag unseen
   // host source loads run on their own stream: they wait only until the
   // solve in flight has copied the source buffer (ev_fuser_free), so they
   // overlap the rest of that solve; the next solve waits for ev_loaded
@@ -2115,12 +2116,21 @@ extern "C" int flgf_set_option(flgf_blockset* bs, int key, int value) {
   return FLGF_OK;
 }
 
+// Before a solve (forward or adjoint): the flag read after the last one is stale.
+static cudaError_t forget_flag(flgf_blockset* bs) {
+  bs->err_known = false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(bs->ctx->stream, &st);
+  bs->replayed |= st == cudaStreamCaptureStatusActive;
+  return e;
+}
+
 extern "C" int flgf_solve(flgf_blockset* bs) {
   if (!bs) return FLGF_EINVAL;
   flgf_ctx* ctx = bs->ctx;
   collect_times(bs);
   cudaError_t e;
-  bs->err_known = false;
+  CK(forget_flag(bs));
   if (bs->load_pending) {  // a host load on the copy stream feeds this solve
     CK(cudaStreamWaitEvent(ctx->stream, bs->ev_loaded, 0));
     bs->load_pending = false;
@@ -2171,7 +2181,8 @@ namespace {
 int check_device_flag(flgf_blockset* bs, const char* what) {
   flgf_ctx* ctx = bs->ctx;
   // one round trip: the flag is read behind the caller's copy, once per solve
-  if (!bs->err_known) CK(cudaMemcpyAsync(bs->h_err, bs->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  // (at every read once the caller has captured a solve)
+  if (!bs->err_known || bs->replayed) CK(cudaMemcpyAsync(bs->h_err, bs->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
   CK(cudaStreamSynchronize(ctx->stream));
   bs->err_known = true;
   if (*bs->h_err) return fail(ctx, FLGF_EDEVICE, std::string(what) + ": a coarse-fine interpolation met a missing halo block");
@@ -2203,7 +2214,7 @@ extern "C" int flgf_solve_adjoint(flgf_blockset* bs) {
   }
   collect_times(bs);
   bs->ev_used = 0;
-  bs->err_known = false;
+  CK(forget_flag(bs));
   cudaError_t e = ctx->prec == FLGF_FP64 ? enqueue_adjoint<double>(bs) : enqueue_adjoint<float>(bs);
   if (e != cudaSuccess) return fail(ctx, FLGF_ECUDA, std::string("solve_adjoint: ") + cudaGetErrorString(e));
   bs->ev_pending = bs->timing && bs->ev_used > 0;
