@@ -175,10 +175,13 @@ struct PhaseOff {  // arena offsets and counts of one phase's launch lists
   int n_groups_dense = 0, n_work = 0, max_units = 0;
   size_t hgroups = 0, work = 0, src_ids = 0, tgt_ids = 0, par_tab = 0;
   int n_groups = 0, n_groups_out = 0, max_group_src = 0; size_t groups = 0, l_tgt = 0, l_len = 0, l_ent = 0, l_src = 0;
-  int n_fl = 0, fl_max_cells = 0, fl_max_parents = 0;
+  int n_fl = 0, fl_max_cells = 0, fl_max_parents = 0;  // of all groups, with those between parents
   size_t fl_groups = 0, fl_rows = 0, fl_dlms = 0, fl_tgt = 0, fl_cells = 0;
   int fl_ncomp = 1, fl_cstride = 0;  // components sharing the frequency-lane groups, their column stride
-  bool fl_split = false;              // rows nearly all full: the two-path product form
+  bool fl_split = false;              // rows of all groups nearly all full
+  // the same of the groups that the frequency-lane kernel runs (from n_pf on): its two-path form and shared memory
+  bool fl_run_split = false;
+  int fl_run_cells = 0, fl_run_parents = 0;
   // the octree levels between parents (parent.cu): the first n_pf
   // frequency-lane groups, their items and column tables, and the children of
   // the source and target parents (one component's; the others follow in order)
@@ -1008,15 +1011,23 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     ph.pf_tch = ar.add(tch);
     ph.pf_scale = ar.add(pscale);
   }
-  {
+  auto nearly_full = [&](int g0) {
     size_t rows = 0, full = 0;
-    for (const FlGroup& g : fll.groups)
+    for (size_t i = g0; i < fll.groups.size(); ++i) {
+      const FlGroup& g = fll.groups[i];
       for (int m = 0; m < g.nact; ++m) {
         const int n = fll.rows[(size_t)(g.row_off + m) * kFlRowStride];
         rows += n;
         for (int j = 0; j < n; ++j) full += fll.dlms[(size_t)(g.row_off + m) * kFlDelta + j] >> 31;
       }
-    ph.fl_split = rows > 0 && (double)full >= kFlSplitFullFraction * (double)rows;
+    }
+    return rows > 0 && (double)full >= kFlSplitFullFraction * (double)rows;
+  };
+  ph.fl_split = nearly_full(0);
+  ph.fl_run_split = nearly_full(ph.n_pf);
+  for (size_t i = ph.n_pf; i < fll.groups.size(); ++i) {
+    ph.fl_run_cells = std::max(ph.fl_run_cells, fll.groups[i].ncell);
+    ph.fl_run_parents = std::max(ph.fl_run_parents, fll.groups[i].nact);
   }
   ph.fl_ncomp = vcomp;
   ph.fl_cstride = ph.nblocks / vcomp;
@@ -1859,10 +1870,10 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
                                          ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
                                          ar.at<uint16_t>(ph.par_tab), spec, acc, ph.ncol, c->d_kspec, c->kstride, s));
     const int n_fl = ph.n_fl - ph.n_pf;
-    KRUN(n_fl, launch_hadamard_fl(N, ar.at<FlGroup>(ph.fl_groups) + ph.n_pf, n_fl, ph.fl_max_cells, ph.fl_max_parents,
+    KRUN(n_fl, launch_hadamard_fl(N, ar.at<FlGroup>(ph.fl_groups) + ph.n_pf, n_fl, ph.fl_run_cells, ph.fl_run_parents,
                                   ar.at<uint16_t>(ph.fl_rows), ar.at<uint32_t>(ph.fl_dlms), ar.at<int>(ph.fl_tgt),
                                   ar.at<int>(ph.fl_cells), spec, acc, ph.ncol, c->d_kspec, c->kstride, ph.fl_ncomp,
-                                  ph.ncol / ph.fl_ncomp, ph.fl_split, s));
+                                  ph.ncol / ph.fl_ncomp, ph.fl_run_split, s));
     KRUN(ph.n_fll, launch_hadamard_fll(N, ar.at<FllGroup>(ph.fll_groups), ph.n_fll, ar.at<int>(ph.fll_tgt),
                                        ar.at<int>(ph.fll_beg), ar.at<int>(ph.fll_len), ar.at<uint32_t>(ph.fll_ent),
                                        spec, acc, ph.ncol, c->d_kspec, c->kstride, s));

@@ -3,7 +3,8 @@
 // block-wise list names has a column, the same one in every list, below the
 // phase's count; the components of a vector block set keep one distance; the
 // passes between parents cover the groups in turn, each with its own parents'
-// columns; and the spectra and the sums together take no more room than those of
+// columns; the frequency-lane kernel's form and shared memory follow the groups
+// that it runs; and the spectra and the sums together take no more room than those of
 // every block of the largest phase would, but for a pass of a single group.
 //
 // usage: spectrum_columns_check <mesh file> <list_pct> <fp64 0|1> <mac> <ncomp> <pass bytes>
@@ -78,6 +79,20 @@ int main(int argc, char** argv) {
           bad += t >= 0 && col[t + c * ph.fl_cstride] != col[t] + c * (ph.ncol / ph.fl_ncomp);
         }
     }
+    long rows = 0, full = 0;
+    int cells = 0, parents = 0;
+    for (int g = ph.n_pf; g < ph.n_fl; ++g) {
+      cells = std::max(cells, fg[g].ncell);
+      parents = std::max(parents, fg[g].nact);
+      for (int m = fg[g].row_off; m < fg[g].row_off + fg[g].nact; ++m) {
+        const int k = reinterpret_cast<const uint16_t*>(host.data() + ph.fl_rows)[(size_t)m * kFlRowStride];
+        rows += k;
+        for (int j = 0; j < k; ++j)
+          full += reinterpret_cast<const uint32_t*>(host.data() + ph.fl_dlms)[(size_t)m * kFlDelta + j] >> 31;
+      }
+    }
+    bad += cells != ph.fl_run_cells || parents != ph.fl_run_parents ||
+           ph.fl_run_split != (rows > 0 && (double)full >= kFlSplitFullFraction * (double)rows);
     const FllGroup* qg = reinterpret_cast<const FllGroup*>(host.data() + ph.fll_groups);
     for (int g = 0; g < ph.n_fll; ++g)
       for (int t = qg[g].tgt_off; t < qg[g].tgt_off + qg[g].ntgt; ++t) {
