@@ -165,6 +165,34 @@ def ncu_traffic(kernel_src: str, kernel: str, workload: str):
     return None
 
 
+def executed_work(w: dict, N: int, rs: int) -> dict:
+    """Operations of the spectrum products and bytes of the FFT stages of one
+    solve, from BlockSet.work_detail(): what the kernels execute.  rs: bytes of a
+    real value.  A product of two complex values is 8 flops, or 6 (three FMAs)
+    in the FP64 form between parents; the axis-0 transforms that share the
+    parents' kernel are left out.  A parent counts with 8 blocks; in FP64 its
+    axis 0 is a pass of its own over half a padded spectrum, into a whole one."""
+    H, block = 2 * N, (2 * N) * (2 * N) * (N + 1)        # complex values of a block's spectrum
+    half = 2 * H * (H + 1) * H                           # and of half a parent's (axes 1 and 2 transformed)
+    fields, csz = 8 * N ** 3 * rs, 2 * rs
+    return {
+        "mac_flops": w["parent_pairs"] * 2 * half * (6.0 if rs == 8 else 8.0) + w["block_pairs"] * block * 8.0,
+        "fwd_bytes": w["parent_fwd"] * (fields + half * csz * (4 if rs == 8 else 1))
+                     + w["block_fwd"] * (fields / 8 + block * csz),
+        "inv_bytes": w["parent_inv"] * (half * csz + fields) + w["block_inv"] * (block * csz + fields / 8),
+    }
+
+
+def fraction(rate, peak, what: str, errors: list):
+    """rate / peak; a value above 1 means that the work is not what ran: it is
+    listed as an error and reported as None."""
+    f = rate / peak
+    if f <= 1.0:
+        return f
+    errors.append(f"{what}: {f:.3f} of its peak")
+    return None
+
+
 def leaf_linf(outs_a, outs_b, probs):
     """max over problems and leaf cells of |a - b|, over max |b| (per problem)."""
     import torch
@@ -320,7 +348,7 @@ def run_ours(a, rank, world):
                      "blockset_create_s": t_create,
                      "launches_per_step": bbs.launch_count(),
                      "stages_ms": {k: v / max(n_timed, 1) for k, v in stage.items()},
-                     "work": bbs.work_counts()}
+                     "work": {**bbs.work_counts(), **bbs.work_detail()}}
         outs[prec] = [[bbs.potential(i, l) for l in range(p.n_levels)] for i, p in enumerate(probs)]
         if prec == "fp32":
             keep_ctx, keep_bs = bctx, bbs
@@ -330,13 +358,13 @@ def run_ours(a, rank, world):
     if "fp64" in outs:
         batched["fp32_vs_fp64_linf"] = leaf_linf(outs["fp32"], outs["fp64"], probs)
     N = 16
-    NW = 2 * N * 2 * N * (N + 1)
     r32 = res["fp32"]
     mac_ms = r32["stages_ms"]["spectrum_mac"]
-    mac_flops = r32["work"]["pairs"] * NW * 8.0
+    mac_flops = executed_work(r32["work"], N, 4)["mac_flops"]
+    errors = []   # fractions above 1
     mac_tflops = mac_flops / (mac_ms / 1e3) / 1e12 if mac_ms > 0 else None
     batched["fp32"] = {k: v for k, v in r32.items() if k != "work"}
-    batched["fp32"]["pairs"] = r32["work"]["pairs"]
+    batched["fp32"]["work"] = r32["work"]
     if "fp64" in res:
         r64 = res["fp64"]
         batched["fp64"] = {k: v for k, v in r64.items() if k != "work"}
@@ -365,20 +393,21 @@ def run_ours(a, rank, world):
             ms = timed(ctx.stream, bs.solve, n)
             stage, nt = bs.stage_times(reset=True)
             st = {k: v / max(nt, 1) for k, v in stage.items()}
-            w = bs.work_counts()
             rs = 4 if prec == "fp32" else 8
-            flops = w["pairs"] * NW * 8.0
+            ex = executed_work(bs.work_detail(), N, rs)
             row = {"value": udof * world / (ms / 1e3), "unit": "DoF/s", "ms_per_step": ms, "steps": n,
                    "stages_ms": st, "launches_per_step": bs.launch_count(),
-                   "spectrum_mac_tflops": flops / (st["spectrum_mac"] / 1e3) / 1e12,
-                   "fft_forward_gbs": w["fwd_ffts"] * (N ** 3 * rs + NW * 2 * rs) / (st["fft_forward"] / 1e3) / 1e9,
-                   "fft_inverse_gbs": w["inv_ffts"] * (N ** 3 * rs + NW * 2 * rs) / (st["fft_inverse"] / 1e3) / 1e9}
+                   "spectrum_mac_tflops": ex["mac_flops"] / (st["spectrum_mac"] / 1e3) / 1e12,
+                   "fft_forward_gbs": ex["fwd_bytes"] / (st["fft_forward"] / 1e3) / 1e9,
+                   "fft_inverse_gbs": ex["inv_bytes"] / (st["fft_inverse"] / 1e3) / 1e9}
             if prec == "fp32":
-                row["spectrum_mac_frac_of_fp32_fma"] = row["spectrum_mac_tflops"] / fp32_alu_peak()
-                row["fft_forward_frac_of_hbm"] = row["fft_forward_gbs"] / hbm
-                row["fft_inverse_frac_of_hbm"] = row["fft_inverse_gbs"] / hbm
+                row["spectrum_mac_frac_of_fp32_fma"] = fraction(row["spectrum_mac_tflops"], fp32_alu_peak(),
+                                                                "uniform FP32 MAC", errors)
+                row["fft_forward_frac_of_hbm"] = fraction(row["fft_forward_gbs"], hbm, "uniform FP32 forward FFT", errors)
+                row["fft_inverse_frac_of_hbm"] = fraction(row["fft_inverse_gbs"], hbm, "uniform FP32 inverse FFT", errors)
             else:
-                row["spectrum_mac_frac_of_fp64_nominal"] = row["spectrum_mac_tflops"] / FP64_NOMINAL_TFLOPS
+                row["spectrum_mac_frac_of_fp64_nominal"] = fraction(row["spectrum_mac_tflops"], FP64_NOMINAL_TFLOPS,
+                                                                    "uniform FP64 MAC", errors)
             uniform[prec] = row
             uniform.setdefault("_u", {})[prec] = bs.potential(0, 0).double().cpu().numpy()
             bs.close()
@@ -589,6 +618,9 @@ def run_ours(a, rank, world):
         uniform.pop("_u", None)
 
     peak = fp32_alu_peak()
+    # DRAM bytes of the MAC's kernels, while both captures are of the current sources
+    traffic = [ncu_traffic("hadamard_fl.cu", "spectrum_mac", f"batched{a.problems}"),
+               ncu_traffic("parent.cu", "parent_mac", f"batched{a.problems}")]
     line = {
         "metric": METRIC,
         "value": r32["value"],
@@ -607,14 +639,17 @@ def run_ours(a, rank, world):
                    "compensated_coarse_levels": True, "cuda_graph": not a.no_graph,
                    "parallelism": "independent problems per rank" if world > 1 else "single GPU"},
         "rel_err": {"fp32_vs_fp64_linf": batched.get("fp32_vs_fp64_linf"), **(err or {})},
-        "roofline": {"bound": "alu", "kernel": "spectrum MAC (hadamard_fl_kernel + hadamard_fll_kernel), "
-                                               "all launches of one batched solve",
+        "roofline": {"bound": "alu", "kernel": "spectrum MAC (pf_mac_kernel + hadamard_fl_kernel + "
+                                               "hadamard_fll_kernel), all launches of one batched solve",
                      "achieved": mac_tflops, "peak": peak, "unit": "TFLOP/s",
-                     "frac": (mac_tflops / peak) if mac_tflops else None,
-                     "traffic": ncu_traffic("hadamard_fl.cu", "spectrum_mac", f"batched{a.problems}"),
+                     "frac": fraction(mac_tflops, peak, "batched MAC", errors) if mac_tflops else None,
+                     "traffic": sum(traffic) if None not in traffic else None,
                      "peak_note": f"FP32 FMA: {n_sm} SMs x {FP32_LANES} lanes x 2 flop x {sm_mhz_peak:.0f} MHz",
                      "flops_per_step": mac_flops,
-                     "flops_note": "useful (target, source) block pairs x 2N*2N*(N+1) frequencies x 8 flop"},
+                     "flops_note": "products of parents that exist x 4N*4N*(2N+1) frequencies x 8 flop + products of "
+                                   "blocks x 2N*2N*(N+1) x 8 flop; the axis-0 transforms in pf_mac_kernel are "
+                                   "not counted",
+                     "errors": errors},
         "hbm": {"peak_gbs": hbm, "peak_source": hbm_src},
         "batched": batched,
         "uniform256": uniform,

@@ -306,10 +306,23 @@ int flgf_set_option(flgf_blockset* bs, int key, int value);
 int flgf_stage_times(flgf_blockset* bs, double* ms, int n_stages, int* n_solves, int reset);
 
 /* Work of one solve for roofline accounting: the number of (target, source)
- * block pairs of the spectrum MAC, of forward and inverse FFTs and of cached
- * kernel-spectrum offsets it touches. */
+ * block pairs that interact, of source and target blocks, and of kernel-spectrum
+ * offsets of the octree levels.  They describe the method (one product and one
+ * transform per pair and block); flgf_work_detail counts what is executed. */
 int flgf_work_counts(const flgf_blockset* bs, int64_t* pairs, int64_t* fwd_ffts, int64_t* inv_ffts,
                      int64_t* kernel_offsets);
+
+/* What one solve executes, for roofline accounting (v[FLGF_WORK_*], n of them):
+ * products of neighbour parents (spectra of 2N blocks a side, padded to 4N
+ * points; absent neighbours, which FP32 multiplies as zeros, not counted),
+ * products of blocks (padded to 2N points; with the near pairs that the coarser
+ * FP64 levels take out), and parents and blocks transformed forwards and back
+ * (a parent in two passes counts twice). */
+enum {
+  FLGF_WORK_PARENT_PAIRS = 0, FLGF_WORK_BLOCK_PAIRS = 1, FLGF_WORK_PARENT_FWD = 2, FLGF_WORK_PARENT_INV = 3,
+  FLGF_WORK_BLOCK_FWD = 4, FLGF_WORK_BLOCK_INV = 5, FLGF_WORK_COUNT = 6
+};
+int flgf_work_detail(const flgf_blockset* bs, int64_t* v, int n);
 
 /* Exact block convolution without device allocation: u = h^2 (G * f) over
  * nblk <= 32 blocks of N^3 cells whose parents (c >> 1) lie within one block

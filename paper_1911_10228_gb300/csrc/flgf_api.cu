@@ -223,6 +223,7 @@ struct flgf_blockset {
   std::vector<AdjOff> adj;
   int Lmax = 0, G = 0, B = 0, max_phase_blocks = 0, max_level_blocks = 0;
   int64_t dof = 0, pairs = 0, n_fwd = 0, n_inv = 0, n_koff = 0;
+  int64_t work[FLGF_WORK_COUNT] = {0};  // flgf_work_detail
   Arena ar;
   void* nodes = nullptr;
   void* unodes = nullptr;
@@ -562,7 +563,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     int k;
     std::vector<ParentRec> drecs;                           // parents of dense tiles, in tile order
     std::vector<std::pair<int, std::vector<int>>> lrecs;   // targets of sparse tiles with their pair lists
-    int64_t pairs = 0;
+    int64_t pairs = 0, listed = 0;  // interacting pairs, those of them in lrecs
   };
   std::vector<TileJob> jobs;
   auto run_tiles = [&](TileJob& job) {
@@ -706,6 +707,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
           // (the near pairs to take out run on the list kernel at its own cost)
           if (list_pct > 0 && useful * 100 < (int64_t)list_pct * dense + 100 * out) {
             // sparse tile: its targets join the pair-list pool of octree level k
+            job.listed += useful;
             for (int ti = 0; ti < (int)tg.size(); ++ti)
               if (tg[ti] >= 0) job.lrecs.push_back({tg[ti], std::move(plist[ti])});
             continue;
@@ -777,7 +779,10 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     for (auto& th : pool) th.join();
   }
   for (TileJob& job : jobs) {
-    if (count) bs->pairs += job.pairs;
+    if (count) {
+      bs->pairs += job.pairs;
+      bs->work[FLGF_WORK_BLOCK_PAIRS] += by_parents(job.k) ? job.listed : job.pairs;
+    }
     if (vcomp > 1 && job.inp->p > 0) job.drecs.clear();  // component 0's groups serve it
     if (!job.drecs.empty()) {
       if ((int)dpool.size() <= job.k) dpool.resize(job.k + 1);
@@ -999,6 +1004,14 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     }
     ph.n_pfs = (int)sch.size() / 8;
     ph.n_pft = (int)tch.size() / 8;
+    if (count) {
+      for (size_t r = 0; r < np; ++r)
+        bs->work[FLGF_WORK_PARENT_PAIRS] += (int64_t)vcomp * fll.rows[r * kFlRowStride];
+      bs->work[FLGF_WORK_PARENT_FWD] += ph.n_pfs;
+      bs->work[FLGF_WORK_PARENT_INV] += ph.n_pft;
+      for (const auto& pool : opool)
+        for (const auto& r : pool) bs->work[FLGF_WORK_BLOCK_PAIRS] += (int64_t)r.second.size();
+    }
     if (vcomp > 1) {  // one pass, of every component's parents
       ph.pf_pass[0].ns = ph.n_pfs;
       ph.pf_pass[0].nt = ph.n_pft;
@@ -1160,6 +1173,10 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     for (int i : fwd_sid) used[i] = 1;
     for (int i : inv_sid) used[i] = 1;
     ph.ncol = (int)std::count(used.begin(), used.end(), 1);
+  }
+  if (count) {
+    bs->work[FLGF_WORK_BLOCK_FWD] += (int64_t)fwd_gid.size();
+    bs->work[FLGF_WORK_BLOCK_INV] += (int64_t)inv_gid.size();
   }
   ph.n_inv = (int)inv_gid.size();
   ph.inv_sid = ar.add(inv_sid);
@@ -1733,6 +1750,12 @@ extern "C" int flgf_work_counts(const flgf_blockset* bs, int64_t* pairs, int64_t
   if (fwd) *fwd = bs->n_fwd;
   if (inv) *inv = bs->n_inv;
   if (koff) *koff = bs->n_koff;
+  return FLGF_OK;
+}
+
+extern "C" int flgf_work_detail(const flgf_blockset* bs, int64_t* v, int n) {
+  if (!bs || !v || n < 0 || n > FLGF_WORK_COUNT) return FLGF_EINVAL;
+  std::copy(bs->work, bs->work + n, v);
   return FLGF_OK;
 }
 

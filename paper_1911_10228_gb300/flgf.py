@@ -75,6 +75,7 @@ PROTOTYPES = {
     "flgf_ctx_set_option": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int]),
     "flgf_stage_times": (ctypes.c_int, [ctypes.c_void_p, _c_dbl_p, ctypes.c_int, _c_int_p, ctypes.c_int]),
     "flgf_work_counts": (ctypes.c_int, [ctypes.c_void_p, _c_i64_p, _c_i64_p, _c_i64_p, _c_i64_p]),
+    "flgf_work_detail": (ctypes.c_int, [ctypes.c_void_p, _c_i64_p, ctypes.c_int]),
     "flgf_launch_count": (ctypes.c_int64, [ctypes.c_void_p]),
     "flgf_load_adjoint": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_int]),
     "flgf_solve_adjoint": (ctypes.c_int, [ctypes.c_void_p]),
@@ -292,6 +293,13 @@ class BlockSet:
         v = [ctypes.c_int64() for _ in range(4)]
         self.ctx.check(self.lib.flgf_work_counts(self.handle, *[ctypes.byref(x) for x in v]), "flgf_work_counts")
         return dict(zip(("pairs", "fwd_ffts", "inv_ffts", "kernel_offsets"), (x.value for x in v)))
+
+    def work_detail(self):
+        """What one solve executes: products and transforms of parents and of blocks."""
+        names = ("parent_pairs", "block_pairs", "parent_fwd", "parent_inv", "block_fwd", "block_inv")
+        v = np.zeros(len(names), dtype=np.int64)
+        self.ctx.check(self.lib.flgf_work_detail(self.handle, _ptr(v, ctypes.c_int64), len(names)), "flgf_work_detail")
+        return dict(zip(names, v.tolist()))
 
     def launch_count(self) -> int:
         """Kernels enqueued by the last solve."""

@@ -6,6 +6,7 @@
 // columns; the frequency-lane kernel's form and shared memory follow the groups
 // that it runs; and the spectra and the sums together take no more room than those of
 // every block of the largest phase would, but for a pass of a single group.
+// The counts of flgf_work_detail are those of the forward tables.
 //
 // usage: spectrum_columns_check <mesh file> <list_pct> <fp64 0|1> <mac> <ncomp> <pass bytes>
 #include "../../paper_1911_10228_gb300/csrc/flgf_api.cu"
@@ -44,7 +45,8 @@ int main(int argc, char** argv) {
   long bad = 0, named = 0, cols = 0, passes = 0;
   bool single = false;  // a pass of one group exceeds the bound
   const size_t csz = ctx.prec == FLGF_FP64 ? 16 : 8, all = csz * (size_t)nfreq(N) * bs->max_phase_blocks;
-  auto check = [&](const PhaseOff& ph, const std::vector<char>& host) {
+  int64_t work[FLGF_WORK_COUNT] = {0};
+  auto check = [&](const PhaseOff& ph, const std::vector<char>& host, bool forward) {
     std::vector<char> img = host;
     number_columns(ph, img.data());
     auto at = [](const std::vector<char>& v, size_t off) { return reinterpret_cast<const int*>(v.data() + off); };
@@ -142,11 +144,50 @@ int main(int argc, char** argv) {
       ++passes;
     }
     bad += g0 != ph.n_pf || s0 != ph.n_pfs || t0 != ph.n_pft;
+    if (!forward) return;
+    for (int g = 0; g < ph.n_pf; ++g)
+      for (int m = 0; m < fg[g].nact; ++m)
+        work[FLGF_WORK_PARENT_PAIRS] +=
+            ph.fl_ncomp * reinterpret_cast<const uint16_t*>(host.data() + ph.fl_rows)[(size_t)(fg[g].row_off + m) * kFlRowStride];
+    work[FLGF_WORK_PARENT_FWD] += s0;
+    work[FLGF_WORK_PARENT_INV] += t0;
+    work[FLGF_WORK_BLOCK_FWD] += ph.n_fwd;
+    work[FLGF_WORK_BLOCK_INV] += ph.n_inv;
+    for (int g = 0; g < ph.n_fll; ++g)
+      for (int t = qg[g].tgt_off; t < qg[g].tgt_off + qg[g].ntgt; ++t) work[FLGF_WORK_BLOCK_PAIRS] += at(host, ph.fll_len)[t];
+    for (int g = 0; g < ph.n_groups + ph.n_groups_out; ++g)
+      for (int m = 0; m < lg[g].ntgt; ++m) work[FLGF_WORK_BLOCK_PAIRS] += at(host, ph.l_len)[lg[g].len_off + m];
+    auto pairs = [&](int level, const int* tgt, const int* src, int e) {
+      for (int a = 0; a < 8; ++a)
+        for (int b = 0; b < 8; ++b) {
+          const int d0 = (a >> 2) - (b >> 2) - 2 * (e / 9 - 1), d1 = (a >> 1 & 1) - (b >> 1 & 1) - 2 * (e / 3 % 3 - 1),
+                    d2 = (a & 1) - (b & 1) - 2 * (e % 3 - 1);
+          const bool near = std::abs(d0) <= 1 && std::abs(d1) <= 1 && std::abs(d2) <= 1;
+          work[FLGF_WORK_BLOCK_PAIRS] += tgt[a] >= 0 && src[b] >= 0 && !(level > 0 && near) ? ph.fl_ncomp : 0;
+        }
+    };
+    for (int g = ph.n_pf; g < ph.n_fl; ++g)
+      for (int m = 0; m < fg[g].nact; ++m) {
+        const uint16_t* row = reinterpret_cast<const uint16_t*>(host.data() + ph.fl_rows) + (size_t)(fg[g].row_off + m) * kFlRowStride;
+        for (int j = 1; j <= row[0]; ++j)
+          pairs(fg[g].level, at(host, ph.fl_tgt) + 8 * (fg[g].row_off + m),
+                at(host, ph.fl_cells) + 8 * (fg[g].cell_off + (row[j] & 0x7FF)), row[j] >> 11);
+      }
+    for (int g = 0; g < ph.n_groups_dense; ++g)
+      for (int m = 0; m < hg[g].nact; ++m)
+        for (int e = 0; e < 27; ++e) {
+          const uint16_t c = reinterpret_cast<const uint16_t*>(host.data() + ph.par_tab)[hg[g].par_off + e * hg[g].nact + m];
+          if (c == kNbEnd) continue;
+          int src[8];
+          for (int b = 0; b < 8; ++b) src[b] = at(host, ph.src_ids)[hg[g].src_off + b * hg[g].ncell + c];
+          pairs(hg[g].level, at(host, ph.tgt_ids) + hg[g].tgt_off + 8 * m, src, e);
+        }
   };
   for (int l = 0; l < bs->Lmax; ++l) {
-    check(bs->ph[l], bs->ar.host);
-    check(bs->aph[l], bs->aar.host);
+    check(bs->ph[l], bs->ar.host, true);
+    check(bs->aph[l], bs->aar.host, false);
   }
+  for (int i = 0; i < FLGF_WORK_COUNT; ++i) bad += work[i] != bs->work[i];
   const auto f = spectra_need(&ctx, bs->ph), a = spectra_need(&ctx, bs->aph);
   const size_t most = std::max(ctx.pf_bytes, 2 * all);
   bad += !single && bs->ncomp == 1 && (f.first + f.second > most || a.first + a.second > most);
