@@ -544,7 +544,6 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
   int max_group_src = 0;
   // targets of sparse tiles per octree level, in tile order: (target id, pair list)
   std::vector<std::vector<std::pair<int, std::vector<int>>>> lpool;
-  const int nchunk = ctx->prec == FLGF_FP64 ? nchunks<double>(N) : nchunks<float>(N);
   // FP32 frequency-lane MAC: the dense tiles' parents go to its groups (sparse
   // tiles still to the pair lists)
   const bool fl = ctx->prec == FLGF_FP32 && ctx->mac >= 1;
@@ -807,7 +806,7 @@ static void build_fmm(flgf_blockset* bs, Arena& ar, int l, const std::vector<con
     } else if (fl)
       pack_fl_groups(k, dpool[k], fll);
     else
-      pack_parent_groups(k, dpool[k], nchunk, had_kernel_units(ctx->prec == FLGF_FP64), hl, ctx->order_by_list);
+      pack_parent_groups(k, dpool[k], nchunks<float>(N), had_kernel_units(false), hl, ctx->order_by_list);  // FP32
   }
   ph.n_fl = (int)fll.groups.size();
   // the near pairs of the coarser levels that the parents' products contain:
@@ -1889,9 +1888,9 @@ cudaError_t enqueue_fmm(flgf_blockset* bs, const Arena& ar, const PhaseOff& ph, 
   {
     StageScope sc(bs, 3);
     if constexpr (sizeof(R) == 4)
-      KRUN(ph.n_work, launch_hadamard<R>(N, ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
-                                         ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
-                                         ar.at<uint16_t>(ph.par_tab), spec, acc, ph.ncol, c->d_kspec, c->kstride, s));
+      KRUN(ph.n_work, launch_hadamard(ar.at<HadGroup>(ph.hgroups), ar.at<HadWork>(ph.work), ph.n_work,
+                                   ph.max_units, ar.at<int>(ph.src_ids), ar.at<int>(ph.tgt_ids),
+                                   ar.at<uint16_t>(ph.par_tab), spec, acc, ph.ncol, c->d_kspec, c->kstride, s));
     const int n_fl = ph.n_fl - ph.n_pf;
     KRUN(n_fl, launch_hadamard_fl(N, ar.at<FlGroup>(ph.fl_groups) + ph.n_pf, n_fl, ph.fl_run_cells, ph.fl_run_parents,
                                   ar.at<uint16_t>(ph.fl_rows), ar.at<uint32_t>(ph.fl_dlms), ar.at<int>(ph.fl_tgt),

@@ -49,15 +49,16 @@
 
 namespace flgf {
 
-template <typename R, int TT>
 __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup* __restrict__ groups,
                                                                   const HadWork* __restrict__ work,
                                                                   const int* __restrict__ src_ids,
                                                                   const int* __restrict__ tgt_ids,
                                                                   const uint16_t* __restrict__ par_tab,
-                                                                  const cplx<R>* __restrict__ spec,
-                                                                  cplx<R>* __restrict__ acc, int spec_blocks,
-                                                                  const cplx<R>* __restrict__ kspec, size_t kstride) {
+                                                                  const cplx<float>* __restrict__ spec,
+                                                                  cplx<float>* __restrict__ acc, int spec_blocks,
+                                                                  const cplx<float>* __restrict__ kspec, size_t kstride) {
+  using R = float;
+  constexpr int TT = 2;  // frequencies per thread
   constexpr int T = ChunkT<R>::value;
   constexpr int NG = T / TT;  // frequency groups per chunk
   static_assert(TT * sizeof(cplx<R>) == 16, "one 16-byte vector per (group, slot)");
@@ -161,24 +162,21 @@ __global__ void __launch_bounds__(kHadThreads, 2) hadamard_kernel(const HadGroup
   }
 }
 
-template <typename R>
-cudaError_t launch_hadamard(int N, const HadGroup* groups, const HadWork* work, int nwork, int max_units,
-                            const int* src_ids, const int* tgt_ids, const uint16_t* par_tab, const void* spec, void* acc,
-                            int spec_blocks, const void* kspec, size_t kspec_level_stride, cudaStream_t s) {
+cudaError_t launch_hadamard(const HadGroup* groups, const HadWork* work, int nwork, int max_units, const int* src_ids,
+                            const int* tgt_ids, const uint16_t* par_tab, const void* spec, void* acc, int spec_blocks,
+                            const void* kspec, size_t kspec_level_stride, cudaStream_t s) {
   if (nwork <= 0) return cudaSuccess;
-  constexpr int TT = (sizeof(R) == 4) ? 2 : 1;
+  using C = cplx<float>;
   // per chunk the group's source spectra and the 343 kernel spectra, and the
   // neighbour table: max_units 32-byte units
   const size_t sm = 32 * (size_t)max_units;
   if (sm > kHadSmemBytes) return cudaErrorInvalidConfiguration;
   // per device and cheap, so set on every launch (two CTAs per SM)
-  cudaError_t e = cudaFuncSetAttribute(hadamard_kernel<R, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)kHadSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(hadamard_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHadSmemBytes);
   if (e != cudaSuccess) return e;
-  hadamard_kernel<R, TT><<<nwork, kHadThreads, sm, s>>>(groups, work, src_ids, tgt_ids, par_tab,
-                                                       reinterpret_cast<const cplx<R>*>(spec),
-                                                       reinterpret_cast<cplx<R>*>(acc), spec_blocks,
-                                                       reinterpret_cast<const cplx<R>*>(kspec), kspec_level_stride);
+  hadamard_kernel<<<nwork, kHadThreads, sm, s>>>(groups, work, src_ids, tgt_ids, par_tab,
+                                                 reinterpret_cast<const C*>(spec), reinterpret_cast<C*>(acc), spec_blocks,
+                                                 reinterpret_cast<const C*>(kspec), kspec_level_stride);
   return cudaGetLastError();
 }
 
@@ -282,9 +280,6 @@ template cudaError_t launch_hadamard_list<float>(int, const ListGroup*, int, int
 template cudaError_t launch_hadamard_list<double>(int, const ListGroup*, int, int, const int*, const int*,
                                                   const int*, const int*, const void*, void*, int, const void*,
                                                   size_t, cudaStream_t);
-
-template cudaError_t launch_hadamard<float>(int, const HadGroup*, const HadWork*, int, int, const int*, const int*,
-                                            const uint16_t*, const void*, void*, int, const void*, size_t, cudaStream_t);
 
 // Shared memory of a group in 32-byte units: per chunk 8 slots per cell and
 // the 343 kernel spectra, plus the [27][nact] int16 neighbour table.

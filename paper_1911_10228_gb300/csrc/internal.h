@@ -60,7 +60,7 @@ cudaError_t launch_kernel_spectra(int N, const double* karr, void* kspec_level, 
                                   cudaStream_t s);
 
 // ---- a3 spectrum multiply-accumulate (hadamard.cu) ------------------------
-// Dense MAC: groups of parents (see hadamard.cu).
+// Dense MAC of FP32 contexts with FLGF_CTX_MAC = 0: groups of parents (see hadamard.cu).
 struct HadGroup {
   int level;     // octree level k (selects the kernel spectra)
   int nact;      // parents (<= kHadMaxParents)
@@ -105,12 +105,11 @@ struct HadLists {
 void pack_parent_groups(int level, const std::vector<ParentRec>& recs, int nchunk, int kunits, HadLists& L,
                         bool order_by_list = false);
 // Kernel-spectrum shared memory per chunk of the dense MAC, in 32-byte units
-// (the kernel runs on FP32 data).
+// (fp64: of the packer alone; the kernel runs on FP32 data).
 constexpr int had_kernel_units(bool fp64) { return fp64 ? 2 * kNOff : kNOff; }
-template <typename R>
-cudaError_t launch_hadamard(int N, const HadGroup* groups, const HadWork* work, int nwork, int max_units,
-                            const int* src_ids, const int* tgt_ids, const uint16_t* par_tab, const void* spec, void* acc,
-                            int spec_blocks, const void* kspec, size_t kspec_level_stride, cudaStream_t s);
+cudaError_t launch_hadamard(const HadGroup* groups, const HadWork* work, int nwork, int max_units, const int* src_ids,
+                            const int* tgt_ids, const uint16_t* par_tab, const void* spec, void* acc, int spec_blocks,
+                            const void* kspec, size_t kspec_level_stride, cudaStream_t s);
 // Sparse tiles: explicit (target, source) pair lists.  The targets of the
 // sparse tiles of one octree level are pooled in tile order and cut into
 // groups of up to kListTargets targets (sorted by list length within a group)
