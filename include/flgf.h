@@ -32,7 +32,8 @@
  * Values are double for FLGF_FP64 contexts and float for FLGF_FP32.
  *
  * Ownership: the library allocates and owns all device memory of a context
- * and a block set (allocation happens only in the *_create calls).  Pointers
+ * and a block set (allocation happens in the *_create calls, at the first
+ * adjoint call of a block set, and for flgf_refine_level's scratch).  Pointers
  * passed in are borrowed for the duration of the call.  All GPU work is
  * enqueued on the context's stream; calls that read results into host memory
  * synchronise that stream.  A handle must not be used from two threads at
@@ -121,10 +122,10 @@ void flgf_destroy(flgf_ctx* ctx);
  *                      dense kernels, sparse tiles in the shared-memory
  *                      pair-list kernel (one target per thread); 0: the
  *                      parent-group kernel (one parent per thread) and the
- *                      shared-memory pair-list kernel.  FP64 contexts always
- *                      use form 0, but for the finest octree level, where
- *                      their dense tiles are convolutions between parents;
- *                      FLGF_CTX_ORDER applies to form 0 only.
+ *                      shared-memory pair-list kernel.  No effect in FP64
+ *                      contexts: the dense tiles of all their octree levels are
+ *                      convolutions between parents, the others shared-memory
+ *                      pair lists.  FLGF_CTX_ORDER applies to form 0 only.
  *   FLGF_CTX_ORDER     0 (default): the parents of each dense-kernel group keep
  *                      the tile order; 1: they are ordered by their set of
  *                      neighbours with sources (most first, equal sets
@@ -337,7 +338,7 @@ int flgf_work_detail(const flgf_blockset* bs, int64_t* v, int n);
  *   f, u    DEVICE arrays [nblk][N][N][N] in the context precision (borrowed),
  *           16-byte aligned
  *   h       lattice spacing (> 0)
- * Scratch: the spectra and launch lists live in a fixed ~18 MB array in
+ * Scratch: the spectra and launch lists live in a fixed 27.3 MB array in
  * device memory that the library declares statically; every GPU that loads
  * the library holds it until the process exits.  The first call on a device
  * looks up that array's device address (cudaGetSymbolAddress); make that

@@ -3,12 +3,13 @@
 The launch lists of a block set fix two choices that decide how fast the
 level interactions (Sec. 2.1) run on a given mesh:
 
-* the dense tile, in parents, of the parent-group kernel (each thread owns the
-  8 children of one parent; the tile's source region is staged in shared
-  memory), and
-* the useful-pair percentage below which a tile runs on the pair-list kernel
-  instead (explicit (target, source) lists: no work on absent blocks, but two
-  shared-memory reads per pair).
+* the dense tile, in parents: tiles are the unit of the pair-list decision, and
+  their order is the order in which parents are packed into the dense kernels'
+  groups, and
+* the percentage of a tile's dense work (products between parents or between
+  their children, see FLGF_CTX_LIST_PCT in include/flgf.h) below which its
+  useful pairs run on the pair-list kernel instead (explicit (target, source)
+  lists: no work on absent blocks, but two reads per pair).
 
 ``autotune`` builds the block set under each candidate plan, times its solve
 with CUDA events on the context's stream, and leaves the context on the

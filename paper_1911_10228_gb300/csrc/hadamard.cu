@@ -38,8 +38,7 @@
 // Complex multiply-adds are written as four fused multiply-adds.
 // FP32 contexts with FLGF_CTX_MAC = 0 only: FP64 runs every level between
 // parents (parent.cu), coarser ones included, which replaced a three-product
-// form of this kernel (11 x 9 x 13 blocks of 16^3: 6.77 -> 2.1 ms with the near
-// pairs' lists and transforms).
+// form of this kernel.
 #include <algorithm>
 #include <unordered_map>
 #include <vector>

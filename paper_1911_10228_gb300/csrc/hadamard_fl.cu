@@ -19,7 +19,7 @@
 // parents): a cell child's 64 frequencies are four 128-byte lines of the
 // chunked spectrum layout, one 16-byte load per lane, and the next cell's
 // sources are in flight while the current one is multiplied.  One CTA of
-// kFlWarps = 12 warps per SM.
+// kFlWarps = 16 warps per SM.
 //
 // Per (parent, cell) the structure of the block-pair offsets is used as in
 // the parent-group kernel: the 8 x 8 (target a, source b) pairs of the parent

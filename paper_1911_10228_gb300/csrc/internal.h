@@ -178,7 +178,10 @@ cudaError_t launch_hadamard_fl(int N, const FlGroup* groups, int ngroups, int ma
                                const uint16_t* rows, const uint32_t* dlms, const int* tgt_ids, const int* cells,
                                const void* spec, void* acc, int spec_blocks, const void* kspec,
                                size_t kspec_level_stride, int ncomp, int cstride, bool split, cudaStream_t s);
-// Full rows at or above this fraction of a phase's rows: the two-path product form.
+// Full rows at or above this fraction of the rows that a phase runs here: the
+// two-path product form.  16^3 blocks (all full): 1.417 ms, 1.460 without it;
+// three-level torus (21 to 72 % full) 4.23 ms, 4.25 with it; 20 sparse problems
+// (13 to 44 %) 25.5 and 26.5 ms.
 constexpr double kFlSplitFullFraction = 0.9;
 // FP32 frequency-lane pair lists (hadamard_fl.cu), for the targets of sparse
 // tiles: a CTA takes a group of at most kFllTargets targets and a block of
@@ -230,6 +233,12 @@ constexpr int kPfItem = 40;  // uint16 per item: five 16-byte vectors
 constexpr int kPfMacThreads = 256;
 // Cost of a neighbour pair of parents, its share of the parents' transforms
 // included, in child pairs of the pair lists (the rule of FLGF_CTX_LIST_PCT).
+// Measured on random boxes (16^3 of 16^3, 24^3 of 8^3 cells), all tiles between
+// parents against all in lists, transforms included: equal cost at 9 to 13 (FP32)
+// and 12 to 15 (FP64) child pairs a neighbour cell where most parents exist, at
+// 14 to 30 where few do (too few groups to fill the chip).  The default's line,
+// 30 % of the cost = 4.8 and 9.6, lies below: tiles are mixed, and on 64 sparse
+// problems it is the best (percentage 15, 30, 40, 50: 62.4, 58.9, 59.8, 60.8 ms).
 // Above the default percentage it grows to a pair's 64 child pairs, so that 100
 // lists every tile that is not completely full, as for the child-pair kernels.
 constexpr int kListPct = 30;

@@ -16,9 +16,10 @@
 // the children of the sorted flagged blocks are then in order as they are
 // (halving the coordinates keeps the order of the keys); of the neighbours only
 // those missing from the level are listed and sorted.  4096 blocks with 459
-// flagged, a call: 1.6 ms with a stable split of five launches per varying bit of
-// three sorts, 459 x 26 candidates sorted and an allocation per scratch array;
-// 0.18 ms (84 us of kernels, three round trips).
+// flagged, none of whose neighbours is missing, a call: 1.65 ms with a stable
+// split of five launches per varying bit of three sorts, 459 x 26 candidates
+// sorted and an allocation per scratch array; 0.18 ms (84 us of kernels and two
+// round trips; a third where neighbours are missing).
 #include <algorithm>
 #include <cstdint>
 #include <utility>

@@ -15,9 +15,9 @@
 // The parts that cancel are no larger than those that stay, so the error is
 // the same (11 x 9 x 13 blocks of 16^3: 2.4e-14 from 64-bit values both ways).
 // FP64's FMA rate bounds it: 27 x 8 + 152 products instead of 1512 a parent.
-// Coarser levels, products and transforms: 11 x 9 x 13 blocks of 16^3 6.9 -> 2.0
-// ms, three-level torus of 8^3 blocks 4.0 -> 1.0 ms.  FP32 keeps the child-pair
-// kernels there: their spectra go through float-float inverse transforms.
+// Whole solves: 11 x 9 x 13 blocks of 16^3 17.6 -> 12.7 ms, three-level torus of
+// 8^3 blocks 10.5 -> 7.4 ms.  FP32 keeps the child-pair kernels there: their
+// spectra go through float-float inverse transforms.
 //
 // The transform along axis 0 is fused with the products (FP64: only the
 // inverse), so HBM only holds spectra of the two transformed axes, half as long
@@ -330,10 +330,14 @@ __global__ void __launch_bounds__(kPfPlaneThreads, sizeof(R) == 4 ? 2 : 1)
 // longer runs lost more to their short parts than they saved: 20 sparse
 // problems 7.6 ms with single parents, 8.2 ms with runs).  FP32 joins two pairs
 // that are neighbours along axis 1 where both exist: 48 reads for 108 products
-// and a third fewer table entries to unpack (ncu on pairs: L1 72 %, issue slots
-// 64 %, the ALU pipe 31 %, all of it unpacking); whole solves, 16^3 blocks of
-// 16^3 1.487 -> 1.438 ms, three-level torus 4.33 -> 4.27 ms, two-level vector
-// torus 2.13 -> 2.09 ms.  The sums are
+// and a third fewer table entries to unpack; whole solves, 16^3 blocks of 16^3
+// 1.487 -> 1.438 ms, three-level torus 4.33 -> 4.27 ms, two-level vector torus
+// 2.13 -> 2.09 ms.  FP32 now, 16^3 blocks of 16^3 (0.65 ms): issue slots 62 %, L1
+// 64 %, the FMA pipe 39 %, the ALU pipe (unpacking, addresses) 24 %, 4 warps a
+// scheduler; copies, line transforms and products take turns behind barriers.
+// FP64, 11 x 9 x 13 blocks (6.3 ms): the FP64 pipe 80 %.  FP32 multiplies absent
+// neighbours of an item as zeros: 1.2 (that box) to 1.5 times (torus, sparse
+// problems) the products that exist.  The sums are
 // transformed back (a thread per line) and the two parities added.
 // FP64 products take the three-multiplication form (kr (fr + fi), (kr + ki)
 // fi, (ki - kr) fr) with fr + fi kept beside the sources, and skip absent cells
@@ -657,7 +661,9 @@ cudaError_t launch_pf_setup(int N, const double* karr, void* tmp, void* kspec, c
 }
 
 // Planes per CTA of the plane kernels: FP32 8 of 32 (16 at N = 8, whole
-// parents), FP64 half of that: about 68 KB of shared memory.
+// parents), FP64 half of that: about 68 KB of shared memory.  Two CTAs an SM
+// hold FP32 at N = 16 to 96 registers, of which the forward kernel spills 88
+// bytes a thread and the inverse 60.
 template <typename R, int N> constexpr int pf_planes() { return (N == 16 ? 8 : 16) / (sizeof(R) == 8 ? 2 : 1); }
 
 template <typename R, int N>

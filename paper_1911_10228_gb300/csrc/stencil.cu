@@ -598,7 +598,8 @@ __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(
 // come from the neighbour block.  Bound by HBM (the field read and the result
 // written once; the rows of faces hit L2).  The terms are added in the order
 // +0, -0, +1, -1, +2, -2.  16^3 blocks of 16^3, FP32 (134 MB), a call: 154 us
-// with a thread per cell and scalar loads, 45 us.
+// with a thread per cell and scalar loads, 45 us (3.0 TB/s; long-scoreboard
+// stalls, and L1 at 79 %: a warp's 16-byte vectors lie a row apart).
 template <typename R, int N>
 __global__ void __launch_bounds__(N * N) laplacian_kernel(const R* __restrict__ u, const int* __restrict__ nbr6, R inv_h2,
                                                           R* __restrict__ out) {
